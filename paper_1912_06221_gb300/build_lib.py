@@ -26,6 +26,8 @@ for _n in range(1, 7):
         SOURCES.append(("rhs_order.cu", "rhs_%s%d" % (_tag, _n),
                         ["-DRDG_ORDER=%d" % _n, "-DRDG_REAL=%s" % _t, "-DRDG_TAG=%s" % _tag,
                          "-DRDG_TAG_IS_F=%d" % (_tag == "f")]))
+    # the face form: its order's operators are written into the build folder first (gen_face.cpp)
+    SOURCES.append(("face_order.cu", "face_%d" % _n, ["-DRDG_ORDER=%d" % _n, "-I", os.path.join(OUT, "gen")]))
 
 
 def nvcc_path():
@@ -33,6 +35,23 @@ def nvcc_path():
         if c and os.path.exists(c):
             return c
     raise RuntimeError("nvcc not found")
+
+
+def _generate(nvcc):
+    """Writes every order's face-form operators, face_ops_<N>.h, with the host program gen_face.cpp."""
+    gen = os.path.join(OUT, "gen")
+    os.makedirs(gen, exist_ok=True)
+    exe = os.path.join(gen, "gen_face")
+    r = subprocess.run([nvcc, "-std=c++17", "-O1", "-x", "c++", os.path.join(SRC, "gen_face.cpp"),
+                        os.path.join(SRC, "refops.cpp"), "-o", exe], capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("compile failed: gen_face\n%s\n%s" % (r.stdout, r.stderr))
+    for n in range(1, 7):
+        r = subprocess.run([exe, str(n)], capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError("gen_face %d failed: %s" % (n, r.stderr))
+        with open(os.path.join(gen, "face_ops_%d.h" % n), "w") as f:
+            f.write(r.stdout)
 
 
 def _compile(nvcc, src, obj, extra):
@@ -54,6 +73,7 @@ def build(verbose: bool = False, ptxas_info: bool = False, force: bool = False) 
         if os.path.getmtime(LIB) >= newest:
             return LIB
     extra = ["-Xptxas", "-v"] if ptxas_info else []
+    _generate(nvcc)
     objs = []
     jobs = []
     workers = max(1, min(len(SOURCES), os.cpu_count() or 1))

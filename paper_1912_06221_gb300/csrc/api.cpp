@@ -72,6 +72,12 @@ void free_ops(rdg_ctx* ctx) {
   dfree(ctx->d_fb, s);
   dfree(ctx->d_f12, s);
   dfree(ctx->d_Dn, s);
+  dfree(ctx->d_fpar, s);
+  dfree(ctx->d_gpar, s);
+  dfree(ctx->d_rec[0], s);
+  dfree(ctx->d_rec[1], s);
+  dfree(ctx->d_gpart, s);
+  ctx->face = false;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
   ctx->ops_ok = false;
@@ -453,8 +459,10 @@ int rdg_query_bytes(int N, int64_t nt, int64_t n_edges, int64_t n_boundary, int 
 
 }  // extern "C"
 
+// Per-edge operators in the forms asked for (each may be null), the face form's parameters (faces),
+// and, unless W_dense is wanted alone, the element coefficients.
 static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz, double* W_dense,
-                          float* P_tiled = nullptr) {
+                          float* P_tiled = nullptr, bool faces = false) {
   const int64_t K = ctx->K, E = ctx->E;
   std::vector<int32_t> k1(E), f1(E), k2(E), f2(E);
   std::vector<double> sh(2 * E);
@@ -530,7 +538,8 @@ static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz,
   }
   EdgeSetupIn in{d_xy, d_i, d_i + E, d_i + 2 * E, d_i + 3 * E, d_sh, d_D, d_Dy, d_Dn64, d_nref, d_refs, E, ctx->vx,
                  ctx->vy, ctx->iface, (int64_t)refs.size()};
-  rc = setup_edges(ctx->N, in, W_tiled, esz, W_dense, P_tiled, s);
+  if (W_tiled || W_dense || P_tiled) rc = setup_edges(ctx->N, in, W_tiled, esz, W_dense, P_tiled, s);
+  if (rc == RDG_OK && faces) rc = setup_faces(in, K, ctx->d_fpar, ctx->d_gpar, s);
   if (rc == RDG_OK && ctx->d_geo && !W_dense)
     rc = setup_elements(K, d_xy, nodal ? nullptr : d_D, d_Dy, ctx->vx, ctx->vy, ctx->d_geo, esz, s);
   e = cudaStreamSynchronize(s);
@@ -543,6 +552,57 @@ static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz,
 extern "C" {
 
 }  // extern "C"
+
+namespace rdg {
+
+// The face form serves every FP32 context with an element-wise D, unless a per-edge stage form was
+// set explicitly or the tensor-core kernels' test hook is.
+bool use_face(const rdg_ctx* ctx) {
+  return ctx->face && ctx->stage_form == RDG_STAGE_AUTO && ctx->gemm_hold == 0;
+}
+
+// Buffers and operators of the per-edge forms, built on first need.
+int ensure_edge_form(rdg_ctx* ctx) {
+  if (ctx->d_W) return RDG_OK;
+  const RefOps* o = get_refops(ctx->N, nullptr);
+  const int N = ctx->N;
+  const int64_t K = ctx->K, E = ctx->E, Np = o->Np, Nfp = o->Nfp, esz = ctx->esz;
+  void* W = nullptr;   // kept only when complete
+  CK(dalloc(&W, ctx->gemm ? edge_data_bytes(N, E, ctx->prec) : w_bytes(N, E, (int)esz), ctx->stream));
+  std::vector<int32_t> k1(E), k2(E), f12(E);
+  for (int64_t e = 0; e < E; ++e) {
+    k1[e] = ctx->edges[e].k1;
+    k2[e] = ctx->edges[e].k2;
+    f12[e] = ctx->edges[e].f1 | ((ctx->edges[e].k2 >= 0 ? ctx->edges[e].f2 : 0) << 2);
+  }
+  struct Want { void** p; int64_t bytes; const void* src; };
+  const Want wants[] = {{(void**)&ctx->d_k1, E * 4, k1.data()},
+                        {(void**)&ctx->d_k2, E * 4, k2.data()},
+                        {(void**)&ctx->d_f12, E * 4, f12.data()},
+                        {(void**)&ctx->d_eref, 3 * K * 4, ctx->eref.data()},
+                        {&ctx->d_flux, E * Nfp * esz, nullptr},
+                        {&ctx->d_vol, K * Np * esz, nullptr},
+                        {&ctx->d_fb, K * 3 * Nfp * esz, nullptr}};
+  for (const Want& w : wants) {
+    cudaError_t e = *w.p ? cudaSuccess : dalloc(w.p, w.bytes, ctx->stream);
+    if (e == cudaSuccess && w.src) e = cudaMemcpyAsync(*w.p, w.src, w.bytes, cudaMemcpyHostToDevice, ctx->stream);
+    if (e != cudaSuccess) {
+      dfree(W, ctx->stream);
+      cudaStreamSynchronize(ctx->stream);
+      return cuda_fail(ctx, e, "per-edge buffers");
+    }
+  }
+  int rc = ctx->gemm ? build_edge_ops(ctx, o, nullptr, (int)esz, nullptr, static_cast<float*>(W))
+                     : build_edge_ops(ctx, o, W, (int)esz, nullptr);   // synchronises: the host arrays may go
+  if (rc != RDG_OK) {
+    dfree(W, ctx->stream);
+    return rc;
+  }
+  ctx->d_W = W;
+  return RDG_OK;
+}
+
+}  // namespace rdg
 
 // Operator set-up; Dy (may be null) is the y diffusion of a diagonal tensor (D_elem then
 // holds the x diffusion), which needs the stored operators.
@@ -578,20 +638,18 @@ static int operator_setup_impl(rdg_ctx* ctx, int N, const double* D_elem, const 
   else ctx->Dy.clear();
   if (Dn) ctx->Dn.assign(Dn, Dn + ctx->K * np_of(N));
   else ctx->Dn.clear();
-  const int64_t K = ctx->K, E = ctx->E, Np = o->Np, Nfp = o->Nfp, esz = ctx->esz;
+  const int64_t K = ctx->K, Np = o->Np, esz = ctx->esz;
   const int64_t stb = K * Np * esz;
-  CK(dalloc(&ctx->d_W, ctx->gemm ? edge_data_bytes(N, E, precision) : w_bytes(N, E, (int)esz), ctx->stream));
-  CK(dalloc(&ctx->d_k1, E * 4, ctx->stream));
-  CK(dalloc(&ctx->d_k2, E * 4, ctx->stream));
-  CK(dalloc(&ctx->d_eref, 3 * K * 4, ctx->stream));
+  ctx->face = precision != RDG_FP64 && !ctx->gemm && !Dn;
   CK(dalloc(&ctx->d_geo, 6 * K * esz, ctx->stream));
-  CK(dalloc(&ctx->d_flux, E * Nfp * esz, ctx->stream));
   CK(dalloc(&ctx->d_u, stb, ctx->stream));
   CK(dalloc(&ctx->d_u1, stb, ctx->stream));
   CK(dalloc(&ctx->d_u2, stb, ctx->stream));
-  CK(dalloc(&ctx->d_vol, stb, ctx->stream));
-  CK(dalloc(&ctx->d_fb, K * 3 * Nfp * esz, ctx->stream));
-  CK(dalloc(&ctx->d_f12, E * 4, ctx->stream));
+  if (ctx->face) {
+    CK(dalloc(&ctx->d_fpar, 6 * K * sizeof(float4), ctx->stream));
+    if (ctx->B) CK(dalloc(&ctx->d_gpar, 2 * ctx->B * sizeof(float4), ctx->stream));
+    for (auto& r : ctx->d_rec) CK(dalloc(&r, 3 * face_rec_pairs(N) * K * sizeof(float2), ctx->stream));
+  }
   if (Dn) {   // the volume term's nodal D, in the context's precision
     CK(dalloc(&ctx->d_Dn, K * Np * esz, ctx->stream));
     if (esz == 8) {
@@ -603,19 +661,10 @@ static int operator_setup_impl(rdg_ctx* ctx, int N, const double* D_elem, const 
       CK(cudaStreamSynchronize(ctx->stream));
     }
   }
-  std::vector<int32_t> k1(E), k2(E), f12(E);
-  for (int64_t e = 0; e < E; ++e) {
-    k1[e] = ctx->edges[e].k1;
-    k2[e] = ctx->edges[e].k2;
-    f12[e] = ctx->edges[e].f1 | ((ctx->edges[e].k2 >= 0 ? ctx->edges[e].f2 : 0) << 2);
-  }
-  CK(cudaMemcpyAsync(ctx->d_f12, f12.data(), E * 4, cudaMemcpyHostToDevice, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->d_k1, k1.data(), E * 4, cudaMemcpyHostToDevice, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->d_k2, k2.data(), E * 4, cudaMemcpyHostToDevice, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->d_eref, ctx->eref.data(), 3 * K * 4, cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemsetAsync(ctx->d_u, 0, stb, ctx->stream));
-  int rc = ctx->gemm ? build_edge_ops(ctx, o, nullptr, (int)esz, nullptr, static_cast<float*>(ctx->d_W))
-                     : build_edge_ops(ctx, o, ctx->d_W, (int)esz, nullptr);
+  int rc = RDG_OK;
+  if (ctx->face) rc = build_edge_ops(ctx, o, nullptr, (int)esz, nullptr, nullptr, true);
+  if (rc == RDG_OK && !use_face(ctx)) rc = ensure_edge_form(ctx);
   if (rc != RDG_OK) {
     free_ops(ctx);
     return rc;
@@ -777,6 +826,15 @@ int rdg_set_forcing(rdg_ctx* ctx, int nsrc, const double* S, const int32_t* src_
     f.gomega[m] = ghost_omega[m];
   }
   ctx->frc = f;
+  if (ctx->face) {   // the ghost data's parts of the boundary fluxes
+    dfree(ctx->d_gpart, ctx->stream);
+    if (nghost) {
+      CK(dalloc(&ctx->d_gpart, (int64_t)nghost * ctx->B * 2 * face_rec_pairs(ctx->N) * sizeof(float), ctx->stream));
+      rc = launch_face_ghost(ctx->N, ctx->iface == RDG_IFACE_ALG1, (const float*)ctx->d_G, ctx->d_gpar, ctx->B, nghost,
+                             ctx->d_gpart, ctx->stream);
+      if (rc != RDG_OK) return fail(ctx, rc, "kernel launch failed");
+    }
+  }
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
   return RDG_OK;
@@ -885,12 +943,87 @@ bool splittable_stage(const rdg_ctx* ctx, int mode) {
          !(mode <= 3 && one_kernel_stage(ctx));
 }
 
+FaceArgs face_args(const rdg_ctx* ctx, const float* us, const TimeArg& ta) {
+  FaceArgs a{};
+  a.us = us;
+  a.par = ctx->d_fpar;
+  a.geo = (const float*)ctx->d_geo;
+  a.S = (const float*)ctx->d_S;
+  a.gpart = ctx->d_gpart;
+  a.K = ctx->K;
+  a.B = ctx->B;
+  a.frc = ctx->frc;
+  a.time = ta;
+  a.err = ctx->d_err;
+  return a;
+}
+
+// Face records of elements [k0, k1) of us into the current buffer.
+int enqueue_face_parts(rdg_ctx* ctx, const float* us, int64_t k0, int64_t k1) {
+  FaceArgs a = face_args(ctx, us, TimeArg{nullptr, 0.0, 1.0, 0.0});
+  a.fout = ctx->d_rec[ctx->rec_cur];
+  a.k_begin = k0 & ~(int64_t)3;   // 16-byte rows; the few elements before k0 get the same records again
+  a.k_end = k1;
+  return launch_face_parts(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, ls(ctx));
+}
+
+// A stage in the face form.  fresh: the records of us are formed first (they are current only after
+// a stage that kept them, with nothing else having touched its result); keep: leave the records of
+// the result, in the other buffer.  On a split mesh, part 0: the owned elements' records (they read
+// owned rows only), part 1: the halo elements' records, then the stage.
+int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* out, int mode, float dt, const TimeArg& ta,
+                       float* out2, float rka, float rkb, int part, bool fresh, bool keep) {
+  if (part == 0) return enqueue_face_parts(ctx, us, 0, ctx->n_owned);
+  cudaStream_t st = ls(ctx);
+  const bool prof = ctx->prof && !ctx->capturing;
+  cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+  if (prof) {
+    for (auto& e : ev) e = take_event(ctx);
+    cudaEventRecord(ev[0], st);
+  }
+  int rc = RDG_OK;
+  if (part == 1) rc = enqueue_face_parts(ctx, us, ctx->n_owned, ctx->K);
+  else if (fresh) rc = enqueue_face_parts(ctx, us, 0, ctx->K);
+  if (prof) {
+    cudaEventRecord(ev[1], st);
+    cudaEventRecord(ev[2], st);
+  }
+  FaceArgs a = face_args(ctx, us, ta);
+  a.un = un;
+  a.out = out;
+  a.out2 = out2;
+  a.fin = ctx->d_rec[ctx->rec_cur];
+  a.fout = keep ? ctx->d_rec[ctx->rec_cur ^ 1] : nullptr;
+  a.mode = mode;
+  a.dt = dt;
+  a.rka = rka;
+  a.rkb = rkb;
+  if (rc == RDG_OK) rc = launch_face_stage(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st);
+  if (rc == RDG_OK && keep) ctx->rec_cur ^= 1;
+  if (prof) {
+    cudaEventRecord(ev[3], st);
+    ctx->ev_pending[0].push_back({ev[0], ev[1]});
+    ctx->ev_pending[1].push_back({ev[2], ev[3]});
+  }
+  return rc;
+}
+
 // part -1: the whole stage.  On a split mesh, part 0: the edges with no halo side and the owned
 // elements' volume terms (they read owned rows only); part 1: the remaining edges and the
 // element update.  A stage that cannot be split runs whole in part 1 (part 0 enqueues nothing).
 template <typename T>
 int enqueue_stage(rdg_ctx* ctx, const void* us, const void* un, void* out, int mode, T dt, const TimeArg& ta,
-                  void* out2 = nullptr, T rka = T(0), T rkb = T(0), int part = -1) {
+                  void* out2 = nullptr, T rka = T(0), T rkb = T(0), int part = -1, bool fresh = true, bool keep = false) {
+  if constexpr (sizeof(T) == 4)
+    if (use_face(ctx)) {
+      // a mesh that is not split runs its stage whole in part 1
+      if (part >= 0 && ctx->n_owned == ctx->K) {
+        if (part == 0) return RDG_OK;
+        part = -1;
+      }
+      return enqueue_face_stage(ctx, (const float*)us, (const float*)un, (float*)out, mode, dt, ta, (float*)out2, rka, rkb,
+                                part, fresh, keep);
+    }
   EdgeArgs<T> ea{ctx->d_k1, ctx->d_k2, ctx->d_W, (const T*)us, (T*)ctx->d_flux, (const T*)ctx->d_G,
                  ctx->E, ctx->B, ctx->frc, ta, ctx->d_err, ctx->K, (T*)ctx->d_vol,
                  (const T*)ctx->d_geo, ctx->d_f12, (T*)ctx->d_fb, keep_tiles(ctx), (const T*)ctx->d_Dn};
@@ -983,36 +1116,39 @@ constexpr double kLsrkC[5] = {0.0, 1432997174477.0 / 9575080441755.0, 2526269341
                               2006345519317.0 / 3224310063776.0, 2802321613138.0 / 2924317926251.0};
 
 template <typename T>
-int enqueue_lsrk_step(rdg_ctx* ctx, const TimeArg& base, double dt) {
+int enqueue_lsrk_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, bool keep) {
   // two registers: u (d_u) and the residual du (d_u1), both updated in place per stage
   int rc = RDG_OK;
   for (int i = 0; i < 5 && rc == RDG_OK; ++i) {
     TimeArg ti = base;
     ti.off = base.off + kLsrkC[i];
-    rc = enqueue_stage<T>(ctx, ctx->d_u, ctx->d_u1, ctx->d_u, 4, (T)dt, ti, ctx->d_u1, (T)kLsrkA[i], (T)kLsrkB[i]);
+    rc = enqueue_stage<T>(ctx, ctx->d_u, ctx->d_u1, ctx->d_u, 4, (T)dt, ti, ctx->d_u1, (T)kLsrkA[i], (T)kLsrkB[i],
+                          -1, fresh && i == 0, keep || i < 4);
   }
   return rc;
 }
 
-int enqueue_rk_step(rdg_ctx* ctx, const TimeArg& base, double dt) {
-  if (ctx->integrator == RDG_INTEGRATOR_LSRK54)
-    return ctx->esz == 4 ? enqueue_lsrk_step<float>(ctx, base, dt) : enqueue_lsrk_step<double>(ctx, base, dt);
+// One step.  fresh, keep: see enqueue_face_stage; only a mesh that is not split passes the records on
+// from stage to stage (the halo rows of a split one change between its stages).
+template <typename T>
+int enqueue_ssp_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, bool keep) {
   // stage times t, t + dt, t + dt/2 (as offsets in units of dt)
   TimeArg t1 = base, t2 = base, t3 = base;
   t2.off = base.off + 1.0;
   t3.off = base.off + 0.5;
-  int rc;
-  if (ctx->esz == 4) {
-    float d = (float)dt;
-    rc = enqueue_stage<float>(ctx, ctx->d_u, nullptr, ctx->d_u1, 1, d, t1);
-    if (rc == RDG_OK) rc = enqueue_stage<float>(ctx, ctx->d_u1, ctx->d_u, ctx->d_u2, 2, d, t2);
-    if (rc == RDG_OK) rc = enqueue_stage<float>(ctx, ctx->d_u2, ctx->d_u, ctx->d_u, 3, d, t3);
-  } else {
-    rc = enqueue_stage<double>(ctx, ctx->d_u, nullptr, ctx->d_u1, 1, dt, t1);
-    if (rc == RDG_OK) rc = enqueue_stage<double>(ctx, ctx->d_u1, ctx->d_u, ctx->d_u2, 2, dt, t2);
-    if (rc == RDG_OK) rc = enqueue_stage<double>(ctx, ctx->d_u2, ctx->d_u, ctx->d_u, 3, dt, t3);
-  }
+  const T d = (T)dt;
+  int rc = enqueue_stage<T>(ctx, ctx->d_u, nullptr, ctx->d_u1, 1, d, t1, nullptr, T(0), T(0), -1, fresh, true);
+  if (rc == RDG_OK) rc = enqueue_stage<T>(ctx, ctx->d_u1, ctx->d_u, ctx->d_u2, 2, d, t2, nullptr, T(0), T(0), -1, false, true);
+  if (rc == RDG_OK) rc = enqueue_stage<T>(ctx, ctx->d_u2, ctx->d_u, ctx->d_u, 3, d, t3, nullptr, T(0), T(0), -1, false, keep);
   return rc;
+}
+
+int enqueue_rk_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, bool keep) {
+  if (ctx->integrator == RDG_INTEGRATOR_LSRK54)
+    return ctx->esz == 4 ? enqueue_lsrk_step<float>(ctx, base, dt, fresh, keep)
+                         : enqueue_lsrk_step<double>(ctx, base, dt, fresh, keep);
+  return ctx->esz == 4 ? enqueue_ssp_step<float>(ctx, base, dt, fresh, keep)
+                       : enqueue_ssp_step<double>(ctx, base, dt, fresh, keep);
 }
 
 // Input buffer of stage `stage` of the selected integrator (SSP-RK3: u, u1, u2; the
@@ -1049,15 +1185,19 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 namespace rdg {
 
-int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double dt) {
+int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double dt, bool fresh, bool keep) {
   cudaStream_t saved = ctx->cap_stream;
   const bool was = ctx->capturing;
   ctx->cap_stream = s;
   ctx->capturing = true;
-  int rc = enqueue_rk_step(ctx, base, dt);
+  int rc = enqueue_rk_step(ctx, base, dt, fresh, keep);
   ctx->cap_stream = saved;
   ctx->capturing = was;
   return rc;
+}
+
+int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta) {
+  return enqueue_face_stage(ctx, u, nullptr, rhs, 0, 0.0f, ta, nullptr, 0.0f, 0.0f, -1, true, false);
 }
 
 }  // namespace rdg
@@ -1083,7 +1223,7 @@ int rdg_rk_step(rdg_ctx* ctx, double t, double dt) {
   if (!(dt > 0) || !std::isfinite(t)) return fail(ctx, RDG_EINVAL, "dt must be positive and t finite");
   DeviceGuard g(ctx->device);
   TimeArg ta{nullptr, t, dt, 0.0};
-  int rc = enqueue_rk_step(ctx, ta, dt);
+  int rc = enqueue_rk_step(ctx, ta, dt, true, false);
   return rc == RDG_OK ? RDG_OK : fail(ctx, rc, "kernel launch failed");
 }
 
@@ -1163,10 +1303,13 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
     CK(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
     ctx->capturing = true;
     int rc = RDG_OK;
+    // the face records of the chunk's first stage input are in buffer 0 when it is replayed, and an
+    // even number of stages later those of its result are again
+    ctx->rec_cur = 0;
     for (int i = 0; i < chunk && rc == RDG_OK; ++i) {
       // the captured steps read their time origin and step count from device memory
       TimeArg ta{ctx->d_time, 0.0, dt, (double)i};
-      rc = enqueue_rk_step(ctx, ta, dt);
+      rc = enqueue_rk_step(ctx, ta, dt, false, true);
     }
     if (rc == RDG_OK) rc = advance_time(ctx->d_time, chunk, ctx->cap_stream);
     cudaError_t e = cudaStreamEndCapture(ctx->cap_stream, &graph);
@@ -1182,12 +1325,16 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
   int64_t done = 0;
   if (nsteps >= chunk) {
     int rc = set_time(ctx->d_time, t0, ctx->stream);
+    if (rc == RDG_OK && use_face(ctx)) {
+      ctx->rec_cur = 0;
+      rc = enqueue_face_parts(ctx, (const float*)ctx->d_u, 0, ctx->K);
+    }
     if (rc != RDG_OK) return fail(ctx, rc, "kernel launch failed");
     for (; done + chunk <= nsteps; done += chunk) CK(cudaGraphLaunch(ctx->gexec, ctx->stream));
   }
   for (; done < nsteps; ++done) {
     TimeArg ta{nullptr, t0 + done * dt, dt, 0.0};
-    int rc = enqueue_rk_step(ctx, ta, dt);
+    int rc = enqueue_rk_step(ctx, ta, dt, done == 0, done + 1 < nsteps);
     if (rc != RDG_OK) return fail(ctx, rc, "kernel launch failed");
   }
   return RDG_OK;
@@ -1207,6 +1354,11 @@ int rdg_set_stage_form(rdg_ctx* ctx, int form) {
   if (!ctx) return RDG_EINVAL;
   if (form != RDG_STAGE_AUTO && form != RDG_STAGE_TWO_KERNELS && form != RDG_STAGE_ONE_KERNEL)
     return fail(ctx, RDG_EINVAL, "form must be RDG_STAGE_AUTO, RDG_STAGE_TWO_KERNELS or RDG_STAGE_ONE_KERNEL");
+  if (ctx->ops_ok && ctx->face && form != RDG_STAGE_AUTO) {   // what the per-edge forms stream
+    DeviceGuard g(ctx->device);
+    int rc = ensure_edge_form(ctx);
+    if (rc != RDG_OK) return rc;
+  }
   ctx->stage_form = form;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
@@ -1216,6 +1368,11 @@ int rdg_set_stage_form(rdg_ctx* ctx, int form) {
 int rdg_gemm_hold_tile(rdg_ctx* ctx, int64_t tile) {
   if (!ctx) return RDG_EINVAL;
   if (tile < -1) return fail(ctx, RDG_EINVAL, "tile must be >= -1");
+  if (ctx->ops_ok && ctx->face && tile >= 0) {   // the held kernel belongs to the per-edge form
+    DeviceGuard g(ctx->device);
+    int rc = ensure_edge_form(ctx);
+    if (rc != RDG_OK) return rc;
+  }
   ctx->gemm_hold = tile + 1;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;

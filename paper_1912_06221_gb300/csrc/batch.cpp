@@ -121,7 +121,9 @@ int prepare_persistent(rdg_batch* b) {
   bool orders[7] = {false, false, false, false, false, false, false};
   int64_t off = 0, offb = 0;
   for (int i = 0; i < nm; ++i) {
-    const rdg_ctx* c = b->members[i].ctx;
+    rdg_ctx* c = b->members[i].ctx;
+    int rc = rdg::ensure_edge_form(c);
+    if (rc != RDG_OK) return bfail(b, rc, std::string("member: ") + rdg_last_error(c));
     rdg::BMember& d = hm[i];
     d.W = c->d_W;
     d.k1 = c->d_k1;
@@ -222,7 +224,7 @@ int enqueue_all(rdg_batch* b, cudaStream_t root, int nsteps) {
     if ((e = cudaStreamWaitEvent(m.branch, b->ev_fork, 0)) != cudaSuccess) return bcuda(b, e, "cudaStreamWaitEvent");
     for (int k = 0; k < nsteps; ++k) {
       rdg::TimeArg ta{m.ctx->d_time, 0.0, m.dt, (double)k};
-      int rc = rdg::enqueue_rk_step_on(m.ctx, m.branch, ta, m.dt);
+      int rc = rdg::enqueue_rk_step_on(m.ctx, m.branch, ta, m.dt, k == 0, k + 1 < nsteps);
       if (rc != RDG_OK) return bfail(b, rc, "kernel launch failed");
     }
     int rc = rdg::advance_time(m.ctx->d_time, nsteps, m.branch);
@@ -321,6 +323,11 @@ int rdg_batch_add(rdg_batch* b, rdg_ctx* ctx, double t0, double dt) {
   for (auto& m : b->members)
     if (m.ctx == ctx) return bfail(b, RDG_EINVAL, "context is already in the batch");
   DevGuard g(b->device);
+  // the persistent launch streams per-edge operators: built here, not in the first step
+  if (b->mode != RDG_BATCH_GRAPH && ctx->face && ctx->integrator == RDG_INTEGRATOR_SSP_RK3) {
+    int rc = rdg::ensure_edge_form(ctx);
+    if (rc != RDG_OK) return bfail(b, rc, std::string("member: ") + rdg_last_error(ctx));
+  }
   rdg_batch::Member m{ctx, dt, nullptr, nullptr, nullptr};
   bool ok = cudaEventCreateWithFlags(&m.ev_in, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&m.ev_join, cudaEventDisableTiming) == cudaSuccess &&

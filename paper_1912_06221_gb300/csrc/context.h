@@ -56,6 +56,12 @@ struct rdg_ctx {
   void* d_vol = nullptr;            // volume terms of the current stage [K][Np]
   void* d_fb = nullptr;             // face fluxes of the current stage [K][3][Nfp]
   int32_t* d_f12 = nullptr;         // per edge f1 | f2 << 2
+  // face form (FP32, element-wise D): parameters, two alternating record buffers, ghost data's parts
+  bool face = false;
+  float4 *d_fpar = nullptr, *d_gpar = nullptr;
+  float2* d_rec[2] = {nullptr, nullptr};
+  float* d_gpart = nullptr;
+  int rec_cur = 0;                  // buffer holding the records of the current stage input
   TimeState* d_time = nullptr;
   int* d_err = nullptr;            // device error bits (kernel self-checks)
   int64_t l2_keep_bytes = -1;       // operator bytes kept L2-resident (-1: default)
@@ -73,9 +79,16 @@ struct rdg_ctx {
 };
 
 namespace rdg {
-// One SSP-RK3 step of ctx's resident state with every launch on stream s (which may be
-// capturing); used by the batch, whose member steps run on per-member branch streams.
-int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double dt);
+// Whether stages run in the face form, and building what the per-edge forms need beside it (the
+// persistent batch launch, an explicitly set stage form).
+bool use_face(const rdg_ctx* ctx);
+int ensure_edge_form(rdg_ctx* ctx);
+// One step of ctx's resident state with every launch on stream s (which may be capturing); used by
+// the batch, whose member steps run on per-member branch streams.  fresh: the face records of the
+// state are formed first; keep: the last stage leaves the records of its result.
+int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double dt, bool fresh, bool keep);
+// Right-hand side of u in the face form (two launches, no allocation).
+int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta);
 // Row gather (dst[i] = src[idx[i]]) or scatter (dst[idx[i]] = src[i]) of np-value rows of
 // esz-byte values; indices outside 0..nrows-1 are recorded in err and skipped.
 int launch_rows(int esz, int np, const void* src, const int32_t* idx, int64_t n, void* dst, bool scatter,

@@ -95,6 +95,28 @@ struct ElemArgs {
   T rka, rkb;
 };
 
+// Face form of a stage (face_kernels.cuh): FP32, element-wise D.
+struct FaceArgs {
+  const float* us;        // stage input
+  const float* un;        // step start, or the low-storage residual register
+  float* out;
+  float* out2;            // low-storage stage: the residual register written
+  const float2* fin;      // face records of the stage input, planes [3 RP][K]
+  float2* fout;           // records of the stage's result, or null: not wanted
+  const float4* par;      // face parameters [3][2][K]: {c, h, A, B}, {C, D, s, neighbour}; neighbour =
+                          // 4 element + face, or 4 boundary edge + 3
+  const float* geo;       // [6][K]
+  const float* S;         // [nsrc][K][Np]
+  const float* gpart;     // parts of the ghost data [nghost][B][2 RP]
+  int64_t K, B;
+  int64_t k_begin, k_end; // parts kernel: elements of this launch
+  Forcing frc;
+  TimeArg time;
+  int* err;               // device error word; may be null
+  int mode;               // as below
+  float dt, rka, rkb;
+};
+
 // mode: 0 rhs only; 1..3 the three SSP-RK3 stage combinations; 4 a low-storage RK stage
 int launch_edge32(int N, const EdgeArgs<float>& a, cudaStream_t s);
 int launch_edge64(int N, const EdgeArgs<double>& a, cudaStream_t s);
@@ -122,6 +144,11 @@ int launch_volume32(int N, const EdgeArgs<float>& a, cudaStream_t s);
 // Edge blocks only (fluxes into the face slots), every order and precision.
 int launch_edge_only32(int N, const EdgeArgs<float>& a, cudaStream_t s);
 int launch_edge_only64(int N, const EdgeArgs<double>& a, cudaStream_t s);
+// Face form: parts of elements [k_begin, k_end) from us into fout; a stage; the ghost data's parts.
+int launch_face_parts(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
+int launch_face_stage(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
+int launch_face_ghost(int N, bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out, cudaStream_t s);
+inline int face_rec_pairs(int N) { return (N + 3) / 2; }   // float2 words of a face record
 int gemm_param_words(int N);   // 16-byte words of an edge's parameter record
 
 // ---- setup (FP64) -------------------------------------------------------------------
@@ -147,6 +174,8 @@ struct EdgeSetupIn {
 // (W_dense), and/or the GEMM-form parameter record (P_tiled, FP32); any may be null.
 int setup_edges(int N, const EdgeSetupIn& in, void* W_tiled, int elem_bytes, double* W_dense, float* P_tiled,
                 cudaStream_t s);
+// Face parameters of the face form, FP64 arithmetic: par [3][2][K] and the ghosts' gpar [B][2].
+int setup_faces(const EdgeSetupIn& in, int64_t K, float4* par, float4* gpar, cudaStream_t s);
 int setup_elements(int64_t K, const double* xy, const double* D, const double* Dy, double vx, double vy, void* geo,
                    int elem_bytes,
                    cudaStream_t s);

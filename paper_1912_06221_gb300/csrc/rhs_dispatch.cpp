@@ -75,6 +75,22 @@ int launch_volume32(int N, const EdgeArgs<float>& a, cudaStream_t s) {
   return N == 6 ? launch_volume_f6(a, s) : RDG_EINVAL;
 }
 
+#define RDG_FACE_DECL(n)                                                                               \
+  int launch_face_parts_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                             \
+  int launch_face_stage_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                             \
+  int launch_face_ghost_##n(bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out, cudaStream_t s);
+RDG_FACE_DECL(1) RDG_FACE_DECL(2) RDG_FACE_DECL(3) RDG_FACE_DECL(4) RDG_FACE_DECL(5) RDG_FACE_DECL(6)
+
+#define CALL_FACE_PARTS(tag, n) launch_face_parts_##n(alg1, a, s)
+#define CALL_FACE_STAGE(tag, n) launch_face_stage_##n(alg1, a, s)
+#define CALL_FACE_GHOST(tag, n) launch_face_ghost_##n(alg1, G, gpar, B, nghost, out, s)
+int launch_face_parts(int N, bool alg1, const FaceArgs& a, cudaStream_t s) { RDG_SWITCH(f, CALL_FACE_PARTS) }
+int launch_face_stage(int N, bool alg1, const FaceArgs& a, cudaStream_t s) { RDG_SWITCH(f, CALL_FACE_STAGE) }
+int launch_face_ghost(int N, bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out,
+                      cudaStream_t s) {
+  RDG_SWITCH(f, CALL_FACE_GHOST)
+}
+
 int gemm_param_words(int N) { return (2 * np_of(N) + nfp_of(N) + 3 + 3) / 4; }
 
 int upload_elem_tables(int device) {

@@ -75,7 +75,9 @@ extern "C" int rdg_rhs_eval_static(rdg_ctx* ctx, const void* u_dev, void* rhs_de
     // every edge writes all of its Nfp fluxes before the element kernel reads them, so the
     // array needs no clearing between calls
     TimeArg ta{nullptr, t, 1.0, 0.0};
-    if (ctx->esz == 4) {
+    if (use_face(ctx)) {
+      rc = enqueue_face_rhs(ctx, (const float*)u_dev, (float*)rhs_dev, ta);   // in the context's own records
+    } else if (ctx->esz == 4) {
       EdgeArgs<float> ea{ctx->d_k1, ctx->d_k2, ctx->d_W, (const float*)u_dev, (float*)flux, (const float*)ctx->d_G,
                          ctx->E, ctx->B, ctx->frc, ta, ctx->d_err, ctx->K};
       ElemArgs<float> la{(const float*)u_dev, nullptr, (float*)rhs_dev, (const float*)flux, ctx->d_eref,

@@ -457,6 +457,69 @@ __global__ void __launch_bounds__(32 * setup_warps<N>()) edge_setup_kernel(EdgeS
   }
 }
 
+// Face parameters of the face form, one thread per edge, both sides' records in FP64 and rounded
+// once: the apex (c, h) of each sub-triangle in its face's frame and the weights of the reference
+// matrices.  With w_jR = -J_f n.(D_j grad R) (the neighbour's frame is the point reflection of the
+// own one, so n and grad R both change sign and w_jR is the same number from either side), A =
+// (w_oR + w_oS + w_nR + w_nS)/4, B = (w_oR - w_oS + w_nR - w_nS)/4, C = (w_oR + w_oS - w_nR - w_nS)/4,
+// D = (w_oR - w_oS - w_nR + w_nS)/4 for own side o and neighbour n (Algorithm 1); the one-coefficient
+// rules use A = (w_R + w_S)/2, B = (w_R - w_S)/2.
+__global__ void __launch_bounds__(128) face_setup_kernel(EdgeSetupIn in, int64_t K, float4* par, float4* gpar) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= in.E) return;
+  const int fb[3] = {1, 2, 0}, fc[3] = {2, 0, 1};
+  const int k1 = in.k1[e], f1 = in.f1[e], k2 = in.k2[e], f2 = in.f2[e];
+  const double* x1 = in.xy + (int64_t)k1 * 6;
+  const D2 e1 = mk(x1[2 * f1], x1[2 * f1 + 1]);
+  const D2 e2 = mk(x1[2 * fb[f1]], x1[2 * fb[f1] + 1]);
+  const D2 q1 = mk(x1[2 * fc[f1]], x1[2 * fc[f1] + 1]);
+  D2 q2 = (e1 + e2) - q1;   // ghost: point reflection of element k1 about the edge midpoint
+  if (k2 >= 0) {
+    const double* x2 = in.xy + (int64_t)k2 * 6;
+    q2 = mk(x2[2 * fc[f2]] + in.shift[2 * e], x2[2 * fc[f2] + 1] + in.shift[2 * e + 1]);
+  }
+  const int kd = k2 >= 0 ? k2 : k1;
+  const bool aniso = in.Dy != nullptr;
+  D2 Do = mk(in.D[k1], aniso ? in.Dy[k1] : in.D[k1]), Dn = mk(in.D[kd], aniso ? in.Dy[kd] : in.D[kd]);
+  if (in.iface == RDG_IFACE_ALG2) Do = Dn = 0.5 * (Do + Dn);
+  if (in.iface == RDG_IFACE_HARMONIC) Do = Dn = mk(2.0 * Do.x * Dn.x / (Do.x + Dn.x), 2.0 * Do.y * Dn.y / (Do.y + Dn.y));
+  const D2 p1 = parallelogram_apex(e1, e2, q1, q2);
+  const D2 p2 = (e1 + e2) - p1;
+  double al[2], be[2];
+  frame_coords(e1, e2, q1, p1, al[0], be[0]);
+  frame_coords(e2, e1, q2, p2, al[1], be[1]);
+  const D2 d = e2 - e1;
+  const double len = sqrt(d.x * d.x + d.y * d.y);
+  const D2 n1 = mk(d.y / len, -d.x / len);
+  const double Jf = 0.5 * len;
+  const D2 xR = 0.5 * (e1 - p1), xS = 0.5 * (e2 - p1);
+  const double m = -Jf / cross(xR, xS);
+  const D2 gR = mk(m * n1.x * xS.y, -m * n1.y * xS.x), gS = mk(-m * n1.x * xR.y, m * n1.y * xR.x);
+  const double oR = Do.x * gR.x + Do.y * gR.y, oS = Do.x * gS.x + Do.y * gS.y;
+  const double nR = Dn.x * gR.x + Dn.y * gR.y, nS = Dn.x * gS.x + Dn.y * gS.y;
+  const bool two = in.iface == RDG_IFACE_ALG1;
+  const float A = (float)(two ? 0.25 * ((oR + oS) + (nR + nS)) : 0.5 * (oR + oS));
+  const float B = (float)(two ? 0.25 * ((oR - oS) + (nR - nS)) : 0.5 * (oR - oS));
+  const float C = (float)(two ? 0.25 * ((oR + oS) - (nR + nS)) : 0.0);
+  const float D = (float)(two ? 0.25 * ((oR - oS) - (nR - nS)) : 0.0);
+  const float s = (float)(Jf * (n1.x * in.vx + n1.y * in.vy));
+  const float c[2] = {(float)(0.5 * (be[0] - al[0])), (float)(0.5 * (be[1] - al[1]))};
+  const float h[2] = {(float)(-0.5 * (al[0] + be[0])), (float)(-0.5 * (al[1] + be[1]))};
+  const int64_t bb = -1 - (int64_t)k2;
+  const unsigned r1 = k2 >= 0 ? 4u * (unsigned)k2 + (unsigned)f2 : 4u * (unsigned)bb + 3u;
+  par[(int64_t)(2 * f1) * K + k1] = make_float4(c[0], h[0], A, B);
+  par[(int64_t)(2 * f1 + 1) * K + k1] = make_float4(C, D, s, __uint_as_float(r1));
+  const float4 a2 = make_float4(c[1], h[1], A, B);
+  const float4 b2 = make_float4(-C, -D, -s, __uint_as_float(4u * (unsigned)k1 + (unsigned)f1));
+  if (k2 >= 0) {
+    par[(int64_t)(2 * f2) * K + k2] = a2;
+    par[(int64_t)(2 * f2 + 1) * K + k2] = b2;
+  } else {
+    gpar[2 * bb] = a2;
+    gpar[2 * bb + 1] = b2;
+  }
+}
+
 __global__ void elem_setup_kernel(int64_t K, const double* xy, const double* D, const double* Dy, double vx, double vy,
                                   void* geo, int elem_bytes) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -512,6 +575,12 @@ int setup_edges(int N, const EdgeSetupIn& in, void* W_tiled, int elem_bytes, dou
     case 6: return launch_setup<6>(in, W_tiled, elem_bytes, W_dense, P_tiled, s);
     default: return RDG_EINVAL;
   }
+}
+
+int setup_faces(const EdgeSetupIn& in, int64_t K, float4* par, float4* gpar, cudaStream_t s) {
+  if (in.E == 0) return RDG_OK;
+  face_setup_kernel<<<(unsigned)((in.E + 127) / 128), 128, 0, s>>>(in, K, par, gpar);
+  return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
 }
 
 int setup_elements(int64_t K, const double* xy, const double* D, const double* Dy, double vx, double vy, void* geo,

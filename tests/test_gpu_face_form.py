@@ -1,0 +1,57 @@
+"""The face form (FP32, element-wise D: one kernel per stage, csrc/face_kernels.cuh) against the FP64
+per-edge kernels, which the oracle pins, at the sizes where its tiles can go wrong: less than one
+128-element tile, exactly one, a ragged second one, several; a right-hand side and a solve of 19
+steps (a replayed chunk of 16, then three steps that pass the records on) with both integrators;
+convection, both interface rules, tensor D, Dirichlet data with time-dependent sources.  The
+tolerance is the FP32 parity tolerance, 1e-5 of the largest value."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1912_06221_gb300 as rdg
+from synth import unit_square_mesh, random_nodal
+from tests.test_gpu_parity import parity_err
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _run(N, m, prec, kind, iface, bc, integ):
+    xy, tri = unit_square_mesh(m, 0.1, m)
+    K = tri.shape[0]
+    rng = np.random.default_rng(N)
+    D = {"jump": np.where(rng.uniform(size=K) < 0.4, 1.0, 0.05), "tensor": rng.uniform(0.3, 1.0, (K, 2))}[kind]
+    s = rdg.Solver(xy, tri, N, D, v=(0.6, -0.9), bc=bc, precision=prec, interface=iface)
+    s.set_integrator(integ)
+    if bc == rdg.BC_DIRICHLET:
+        x, g = s.node_coords(), s.ghost_coords()
+        s.set_forcing([(np.sin(3 * x[..., 0]) * x[..., 1], rdg.TAU_COS, 2.0), (x[..., 0], rdg.TAU_CONST, 0.0)],
+                      [(g[..., 0] - g[..., 1], rdg.TAU_SIN, 3.0), (g[..., 1] ** 2, rdg.TAU_COS, 1.0)])
+    u = torch.tensor(random_nodal(K, s.Np, 7).astype(np.float32), dtype=s.dtype, device="cuda")
+    r = torch.empty_like(u)
+    s.rhs_eval(u, r, 0.4)
+    s.set_state(u)
+    s.solve_to_time(0.2, 0.05 / m ** 2 / (N + 1) ** 4, 19)
+    out = [r.double().cpu().numpy(), s.get_state_host().astype(np.float64)]
+    s.synchronize()
+    s.close()
+    return out
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("m,kind,iface,bc,integ", [
+    (3, "jump", rdg.IFACE_ALG1, rdg.BC_PERIODIC, rdg.SSP_RK3),
+    (8, "tensor", rdg.IFACE_ALG1, rdg.BC_DIRICHLET, rdg.LSRK54),
+    (9, "jump", rdg.IFACE_ALG2, rdg.BC_DIRICHLET, rdg.SSP_RK3),
+    (21, "tensor", rdg.IFACE_ALG2, rdg.BC_PERIODIC, rdg.LSRK54),
+    (21, "jump", rdg.IFACE_HARMONIC, rdg.BC_DIRICHLET, rdg.SSP_RK3)])
+def test_face_form_matches_fp64(N, m, kind, iface, bc, integ):
+    got = _run(N, m, rdg.FP32, kind, iface, bc, integ)
+    want = _run(N, m, rdg.FP64, kind, iface, bc, integ)
+    for a, b in zip(got, want):
+        assert parity_err(a, b) < 1e-5
