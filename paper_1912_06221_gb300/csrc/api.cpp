@@ -72,11 +72,13 @@ void free_ops(rdg_ctx* ctx) {
   dfree(ctx->d_fb, s);
   dfree(ctx->d_f12, s);
   dfree(ctx->d_Dn, s);
-  dfree(ctx->d_fpar, s);
-  dfree(ctx->d_gpar, s);
+  dfree(ctx->face_tab.p4, s);
+  dfree(ctx->face_tab.gpar, s);
+  ctx->face_tab = FaceTables{};
   dfree(ctx->d_rec[0], s);
   dfree(ctx->d_rec[1], s);
   dfree(ctx->d_gpart, s);
+  dfree(ctx->d_tau, s);
   ctx->face = false;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
@@ -539,7 +541,7 @@ static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz,
   EdgeSetupIn in{d_xy, d_i, d_i + E, d_i + 2 * E, d_i + 3 * E, d_sh, d_D, d_Dy, d_Dn64, d_nref, d_refs, E, ctx->vx,
                  ctx->vy, ctx->iface, (int64_t)refs.size()};
   if (W_tiled || W_dense || P_tiled) rc = setup_edges(ctx->N, in, W_tiled, esz, W_dense, P_tiled, s);
-  if (rc == RDG_OK && faces) rc = setup_faces(in, K, ctx->d_fpar, ctx->d_gpar, s);
+  if (rc == RDG_OK && faces) rc = setup_faces(in, K, ctx->face_tab, s);
   if (rc == RDG_OK && ctx->d_geo && !W_dense)
     rc = setup_elements(K, d_xy, nodal ? nullptr : d_D, d_Dy, ctx->vx, ctx->vy, ctx->d_geo, esz, s);
   e = cudaStreamSynchronize(s);
@@ -640,15 +642,20 @@ static int operator_setup_impl(rdg_ctx* ctx, int N, const double* D_elem, const 
   else ctx->Dn.clear();
   const int64_t K = ctx->K, Np = o->Np, esz = ctx->esz;
   const int64_t stb = K * Np * esz;
-  ctx->face = precision != RDG_FP64 && !ctx->gemm && !Dn;
+  ctx->face = precision != RDG_FP64 && !ctx->gemm && !Dn && K <= kMaxFaceElements;
   CK(dalloc(&ctx->d_geo, 6 * K * esz, ctx->stream));
   CK(dalloc(&ctx->d_u, stb, ctx->stream));
   CK(dalloc(&ctx->d_u1, stb, ctx->stream));
   CK(dalloc(&ctx->d_u2, stb, ctx->stream));
   if (ctx->face) {
-    CK(dalloc(&ctx->d_fpar, 6 * K * sizeof(float4), ctx->stream));
-    if (ctx->B) CK(dalloc(&ctx->d_gpar, 2 * ctx->B * sizeof(float4), ctx->stream));
-    for (auto& r : ctx->d_rec) CK(dalloc(&r, 3 * face_rec_pairs(N) * K * sizeof(float2), ctx->stream));
+    FaceTables& t = ctx->face_tab;
+    CK(dalloc(&t.p4, 3 * K * (sizeof(float4) + sizeof(float2) + sizeof(float) + sizeof(unsigned)), ctx->stream));
+    t.p2 = reinterpret_cast<float2*>(t.p4 + 3 * K);
+    t.p1 = reinterpret_cast<float*>(t.p2 + 3 * K);
+    t.nbr = reinterpret_cast<unsigned*>(t.p1 + 3 * K);
+    if (ctx->B) CK(dalloc(&t.gpar, 2 * ctx->B * sizeof(float4), ctx->stream));
+    CK(dalloc(&ctx->d_tau, kTauSteps * kTauStages * kTauRow * sizeof(float), ctx->stream));
+    for (auto& r : ctx->d_rec) CK(dalloc(&r, face_rec_floats(N, K) * sizeof(float), ctx->stream));
   }
   if (Dn) {   // the volume term's nodal D, in the context's precision
     CK(dalloc(&ctx->d_Dn, K * Np * esz, ctx->stream));
@@ -829,8 +836,8 @@ int rdg_set_forcing(rdg_ctx* ctx, int nsrc, const double* S, const int32_t* src_
   if (ctx->face) {   // the ghost data's parts of the boundary fluxes
     dfree(ctx->d_gpart, ctx->stream);
     if (nghost) {
-      CK(dalloc(&ctx->d_gpart, (int64_t)nghost * ctx->B * 2 * face_rec_pairs(ctx->N) * sizeof(float), ctx->stream));
-      rc = launch_face_ghost(ctx->N, ctx->iface == RDG_IFACE_ALG1, (const float*)ctx->d_G, ctx->d_gpar, ctx->B, nghost,
+      CK(dalloc(&ctx->d_gpart, (int64_t)nghost * ctx->B * (ctx->N + 2) * sizeof(float), ctx->stream));
+      rc = launch_face_ghost(ctx->N, ctx->iface == RDG_IFACE_ALG1, (const float*)ctx->d_G, ctx->face_tab.gpar, ctx->B, nghost,
                              ctx->d_gpart, ctx->stream);
       if (rc != RDG_OK) return fail(ctx, rc, "kernel launch failed");
     }
@@ -943,24 +950,41 @@ bool splittable_stage(const rdg_ctx* ctx, int mode) {
          !(mode <= 3 && one_kernel_stage(ctx));
 }
 
-FaceArgs face_args(const rdg_ctx* ctx, const float* us, const TimeArg& ta) {
+FaceArgs face_args(const rdg_ctx* ctx, const float* us) {
   FaceArgs a{};
   a.us = us;
-  a.par = ctx->d_fpar;
+  a.p4 = ctx->face_tab.p4;
+  a.p2 = ctx->face_tab.p2;
+  a.p1 = ctx->face_tab.p1;
+  a.nbr = ctx->face_tab.nbr;
   a.geo = (const float*)ctx->d_geo;
   a.S = (const float*)ctx->d_S;
   a.gpart = ctx->d_gpart;
   a.K = ctx->K;
   a.B = ctx->B;
-  a.frc = ctx->frc;
-  a.time = ta;
   a.err = ctx->d_err;
   return a;
 }
 
+// The forcing factors at stage time ta: a row of the replayed chunk's table, or evaluated here.
+void face_forcing(const rdg_ctx* ctx, const TimeArg& ta, int stage, FaceArgs& a) {
+  const Forcing& f = ctx->frc;
+  a.nsrc = f.nsrc;
+  a.nghost = f.nghost;
+  if (f.nsrc + f.nghost == 0) return;
+  if (ta.ts) {
+    // offsets within a replayed chunk count whole steps; the stage's own offset is in its row
+    a.tau_row = ctx->d_tau + (ctx->tau_step % kTauSteps * kTauStages + stage) * kTauRow;
+    return;
+  }
+  const double t = ta.t0 + ta.off * ta.dt;
+  for (int m = 0; m < f.nsrc; ++m) a.tau[m] = (float)host_tau(f.kind[m], f.omega[m], t);
+  for (int m = 0; m < f.nghost; ++m) a.tau[RDG_MAX_FORCING_TERMS + m] = (float)host_tau(f.gkind[m], f.gomega[m], t);
+}
+
 // Face records of elements [k0, k1) of us into the current buffer.
 int enqueue_face_parts(rdg_ctx* ctx, const float* us, int64_t k0, int64_t k1) {
-  FaceArgs a = face_args(ctx, us, TimeArg{nullptr, 0.0, 1.0, 0.0});
+  FaceArgs a = face_args(ctx, us);
   a.fout = ctx->d_rec[ctx->rec_cur];
   a.k_begin = k0 & ~(int64_t)3;   // 16-byte rows; the few elements before k0 get the same records again
   a.k_end = k1;
@@ -972,7 +996,7 @@ int enqueue_face_parts(rdg_ctx* ctx, const float* us, int64_t k0, int64_t k1) {
 // the result, in the other buffer.  On a split mesh, part 0: the owned elements' records (they read
 // owned rows only), part 1: the halo elements' records, then the stage.
 int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* out, int mode, float dt, const TimeArg& ta,
-                       float* out2, float rka, float rkb, int part, bool fresh, bool keep) {
+                       float* out2, float rka, float rkb, int part, bool fresh, bool keep, int stage) {
   if (part == 0) return enqueue_face_parts(ctx, us, 0, ctx->n_owned);
   cudaStream_t st = ls(ctx);
   const bool prof = ctx->prof && !ctx->capturing;
@@ -988,7 +1012,8 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
     cudaEventRecord(ev[1], st);
     cudaEventRecord(ev[2], st);
   }
-  FaceArgs a = face_args(ctx, us, ta);
+  FaceArgs a = face_args(ctx, us);
+  face_forcing(ctx, ta, stage, a);
   a.un = un;
   a.out = out;
   a.out2 = out2;
@@ -1013,7 +1038,7 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
 // element update.  A stage that cannot be split runs whole in part 1 (part 0 enqueues nothing).
 template <typename T>
 int enqueue_stage(rdg_ctx* ctx, const void* us, const void* un, void* out, int mode, T dt, const TimeArg& ta,
-                  void* out2 = nullptr, T rka = T(0), T rkb = T(0), int part = -1, bool fresh = true, bool keep = false) {
+                  void* out2 = nullptr, T rka = T(0), T rkb = T(0), int part = -1, bool fresh = true, bool keep = false, int stage = 0) {
   if constexpr (sizeof(T) == 4)
     if (use_face(ctx)) {
       // a mesh that is not split runs its stage whole in part 1
@@ -1022,7 +1047,7 @@ int enqueue_stage(rdg_ctx* ctx, const void* us, const void* un, void* out, int m
         part = -1;
       }
       return enqueue_face_stage(ctx, (const float*)us, (const float*)un, (float*)out, mode, dt, ta, (float*)out2, rka, rkb,
-                                part, fresh, keep);
+                                part, fresh, keep, stage);
     }
   EdgeArgs<T> ea{ctx->d_k1, ctx->d_k2, ctx->d_W, (const T*)us, (T*)ctx->d_flux, (const T*)ctx->d_G,
                  ctx->E, ctx->B, ctx->frc, ta, ctx->d_err, ctx->K, (T*)ctx->d_vol,
@@ -1123,7 +1148,7 @@ int enqueue_lsrk_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, 
     TimeArg ti = base;
     ti.off = base.off + kLsrkC[i];
     rc = enqueue_stage<T>(ctx, ctx->d_u, ctx->d_u1, ctx->d_u, 4, (T)dt, ti, ctx->d_u1, (T)kLsrkA[i], (T)kLsrkB[i],
-                          -1, fresh && i == 0, keep || i < 4);
+                          -1, fresh && i == 0, keep || i < 4, i);
   }
   return rc;
 }
@@ -1137,13 +1162,23 @@ int enqueue_ssp_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, b
   t2.off = base.off + 1.0;
   t3.off = base.off + 0.5;
   const T d = (T)dt;
-  int rc = enqueue_stage<T>(ctx, ctx->d_u, nullptr, ctx->d_u1, 1, d, t1, nullptr, T(0), T(0), -1, fresh, true);
-  if (rc == RDG_OK) rc = enqueue_stage<T>(ctx, ctx->d_u1, ctx->d_u, ctx->d_u2, 2, d, t2, nullptr, T(0), T(0), -1, false, true);
-  if (rc == RDG_OK) rc = enqueue_stage<T>(ctx, ctx->d_u2, ctx->d_u, ctx->d_u, 3, d, t3, nullptr, T(0), T(0), -1, false, keep);
+  int rc = enqueue_stage<T>(ctx, ctx->d_u, nullptr, ctx->d_u1, 1, d, t1, nullptr, T(0), T(0), -1, fresh, true, 0);
+  if (rc == RDG_OK) rc = enqueue_stage<T>(ctx, ctx->d_u1, ctx->d_u, ctx->d_u2, 2, d, t2, nullptr, T(0), T(0), -1, false, true, 1);
+  if (rc == RDG_OK) rc = enqueue_stage<T>(ctx, ctx->d_u2, ctx->d_u, ctx->d_u, 3, d, t3, nullptr, T(0), T(0), -1, false, keep, 2);
   return rc;
 }
 
 int enqueue_rk_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, bool keep) {
+  if (base.ts && use_face(ctx) && ctx->frc.nsrc + ctx->frc.nghost > 0) {
+    // replayed steps read their forcing factors from a table, refilled every kTauSteps steps
+    ctx->tau_step = (int)base.off;
+    if (ctx->tau_step % kTauSteps == 0) {
+      const bool ls5 = ctx->integrator == RDG_INTEGRATOR_LSRK54;
+      StageOffsets off{{0.0, ls5 ? kLsrkC[1] : 1.0, ls5 ? kLsrkC[2] : 0.5, ls5 ? kLsrkC[3] : 0.0, ls5 ? kLsrkC[4] : 0.0}};
+      int rc = launch_face_tau(ctx->frc, base, off, ctx->d_tau, ls(ctx));
+      if (rc != RDG_OK) return rc;
+    }
+  }
   if (ctx->integrator == RDG_INTEGRATOR_LSRK54)
     return ctx->esz == 4 ? enqueue_lsrk_step<float>(ctx, base, dt, fresh, keep)
                          : enqueue_lsrk_step<double>(ctx, base, dt, fresh, keep);
@@ -1197,7 +1232,7 @@ int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double
 }
 
 int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta) {
-  return enqueue_face_stage(ctx, u, nullptr, rhs, 0, 0.0f, ta, nullptr, 0.0f, 0.0f, -1, true, false);
+  return enqueue_face_stage(ctx, u, nullptr, rhs, 0, 0.0f, ta, nullptr, 0.0f, 0.0f, -1, true, false, 0);
 }
 
 }  // namespace rdg

@@ -58,9 +58,11 @@ struct rdg_ctx {
   int32_t* d_f12 = nullptr;         // per edge f1 | f2 << 2
   // face form (FP32, element-wise D): parameters, two alternating record buffers, ghost data's parts
   bool face = false;
-  float4 *d_fpar = nullptr, *d_gpar = nullptr;
-  float2* d_rec[2] = {nullptr, nullptr};
+  rdg::FaceTables face_tab{};       // p4 heads one allocation that also holds p2, p1 and nbr
+  float* d_rec[2] = {nullptr, nullptr};
   float* d_gpart = nullptr;
+  float* d_tau = nullptr;           // forcing factors of a replayed chunk's stages (launch_face_tau)
+  int tau_step = 0;                 // step of the chunk being enqueued
   int rec_cur = 0;                  // buffer holding the records of the current stage input
   TimeState* d_time = nullptr;
   int* d_err = nullptr;            // device error bits (kernel self-checks)

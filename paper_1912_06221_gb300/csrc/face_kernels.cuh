@@ -5,9 +5,12 @@
 //  face_stage_kernel  volume term of the stage input, fluxes from the own and the neighbours' parts,
 //                     LIFT, sources, the stage update, and the new values' parts for the next stage
 //
-// Face records (the parts and the element's reference value) are planes of float2 [3 RP][K], so a
-// warp stores and reads its own elements' records in whole sectors; two buffers alternate between
-// stages, since a block reads its neighbours' records while others already write the next stage's.
+// A warp owns 32 consecutive elements and never waits for another warp: its rows go through a slice
+// of shared memory of its own (cp.async in, 16-byte stores out).  A face record is the N + 1 components of
+// the part; records lie in planes [3][K] of 4, 2 and 1 floats (N = 4: a plane of float4 and one of
+// float), then one plane [K] of the reference values, so a warp stores and reads its own elements'
+// records in whole sectors and each record costs one or two loads.  Two buffers alternate between
+// stages, since a warp reads its neighbours' records while others already write the next stage's.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -18,13 +21,66 @@
 namespace rdg {
 namespace dev {
 
-template <int N>
-__host__ __device__ constexpr int face_block() {
-  return 128;
+constexpr int kFaceWarps = 4;
+constexpr int kFaceBlock = 32 * kFaceWarps;
+
+// How face_stage_kernel is built for a range of sizes (launch_stage in face_order.cu chooses).
+//  early: bit 0, the own and the neighbours' records, bit 1, the face parameters are held in registers
+//         from before the volume term; otherwise each is loaded where it is used;
+//  blocks: resident blocks of 4 warps per SM asked of the compiler;
+//  roll: the three faces in a loop over one copy of the code (the values rotate from face to face).
+// Few tiles (small): one warp per scheduler hides no latency by itself, so everything is loaded early;
+// at orders 5 and 6 a lone warp waits for instructions (70 KB of straight-line code at order 6), so
+// the loop is faster there (order 6, 20402 elements: 7.9 against 8.9 us per stage; order 4 no gain).
+// More tiles than those warps (large): all tiles resident at once beats two uneven waves.  131072
+// elements, small / large: order 1 4.2 / 3.4 us, 2 5.5 / 4.5, 3 7.2 / 6.1, 4 10.8 / 9.2; 65522
+// elements: order 5 10.9 / 9.2, 6 14.7 / 13.5.
+struct FaceBuild {
+  int early, blocks;
+  bool roll;
+};
+template <int N, bool LARGE>
+__host__ __device__ constexpr FaceBuild face_build() {
+  if (!LARGE) return N <= 3 ? FaceBuild{3, 5, false} : N == 4 ? FaceBuild{3, 4, false} : FaceBuild{3, N == 5 ? 3 : 2, true};
+  return N <= 2 ? FaceBuild{1, 7, false} : N <= 4 ? FaceBuild{0, 7, false} : FaceBuild{N == 5 ? 3 : 0, 4, N == 5};
 }
+// Resident four-warp blocks per SM of face_team_kernel.
 template <int N>
-__host__ __device__ constexpr int face_min_blocks() {
-  return N <= 2 ? 6 : (N <= 4 ? 4 : (N == 5 ? 3 : 2));
+__host__ __device__ constexpr int team_blocks() {
+  return N == 4 ? 6 : (N == 5 ? 5 : 4);
+}
+
+// Rows of a warp's elements (n values from a 16-byte aligned start) into its shared slice.
+template <int NP>
+__device__ __forceinline__ void rows_in(float* sh, const float* g, int n, int lane) {
+  const int nv = n / 4;
+#pragma unroll
+  for (int it = 0; it < (NP + 3) / 4; ++it) {
+    const int i = lane + 32 * it;
+    if (i < nv)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(sh + 4 * i)),
+                   "l"(g + 4 * i)
+                   : "memory");
+  }
+  const int i = nv * 4 + lane;
+  if (i < n) sh[i] = g[i];
+}
+template <int NP>
+__device__ __forceinline__ void rows_out(float* g, const float* sh, int n, int lane) {
+  const int nv = n / 4;
+#pragma unroll
+  for (int it = 0; it < (NP + 3) / 4; ++it) {
+    const int i = lane + 32 * it;
+    if (i < nv) reinterpret_cast<float4*>(g)[i] = reinterpret_cast<const float4*>(sh)[i];
+  }
+  const int i = nv * 4 + lane;
+  if (i < n) g[i] = sh[i];
+}
+__device__ __forceinline__ void rows_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void rows_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+  __syncwarp();
 }
 
 // Row of NP values in shared memory, read or written with the widest aligned access (NP = 6, 10: 8
@@ -62,65 +118,136 @@ __device__ __forceinline__ void row_put(float* p, const float (&v)[NP]) {
   }
 }
 
-// A face's parameters: {c, h, A, B}, {C, D, s, neighbour}.
-__device__ __forceinline__ face::Par<float> face_par(float4 a, float4 b) {
-  return face::Par<float>{a.x, a.y, a.z, a.w, b.x, b.y, b.z};
+// Element k's face parameters: {c, h, A, B}, s and, where the caller's warp has a jump of D, {C, D}.
+__device__ __forceinline__ face::Par<float> face_par(const FaceArgs& a, int f, unsigned k, bool diff) {
+  const float4 p = __ldg(a.p4 + (size_t)f * a.K + k);
+  const float2 q = diff ? __ldg(a.p2 + (size_t)f * a.K + k) : make_float2(0.f, 0.f);
+  return face::Par<float>{p.x, p.y, p.z, p.w, q.x, q.y, __ldg(a.p1 + (size_t)f * a.K + k)};
+}
+
+// The own-minus-neighbour weights are zero wherever D does not jump; the face's neighbour word says so,
+// and a warp without a jump skips their loads and products.
+template <bool ALG1>
+__device__ __forceinline__ bool jump_in_warp(unsigned nbr) {
+  return ALG1 && __any_sync(0xffffffffu, (nbr & kFaceJump) != 0);
+}
+
+// Record r of a buffer of 3 K records: planes of 4, 2 and 1 floats.
+template <int NG>
+__device__ __forceinline__ void record_get(const float* buf, size_t K3, unsigned r, float (&v)[NG]) {
+  constexpr int N4 = NG / 4 * 4, N2 = N4 + (NG - N4) / 2 * 2;
+  if constexpr (NG >= 4) {
+    const float4 t = reinterpret_cast<const float4*>(buf)[r];
+    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+  }
+  if constexpr (N2 > N4) {
+    const float2 t = reinterpret_cast<const float2*>(buf + N4 * K3)[r];
+    v[N4] = t.x, v[N4 + 1] = t.y;
+  }
+  if constexpr (NG > N2) v[N2] = (buf + N2 * K3)[r];
+}
+// The neighbour's record (word r of the neighbour table) and its reference value; of a boundary edge,
+// whose data ghost_get supplies, or a corrupt table, any valid one.
+template <int NG>
+__device__ __forceinline__ void neighbour_get(const FaceArgs& a, unsigned r, unsigned k, float (&v)[NG + 1]) {
+  const unsigned K = (unsigned)a.K, K3 = 3u * K;
+  if (r >= K3) {
+    if (r >= K3 + (unsigned)a.B) report(a.err, kErrBadIndex);
+    r = k;
+  }
+  float g[NG];
+  record_get<NG>(a.fin, K3, r, g);
+#pragma unroll
+  for (int c = 0; c < NG; ++c) v[c] = g[c];
+  r -= r >= K ? K : 0u;
+  r -= r >= K ? K : 0u;
+  v[NG] = (a.fin + (size_t)NG * K3)[r];
+}
+__device__ __forceinline__ float stage_tau(const FaceArgs& a, int m) { return a.tau_row ? a.tau_row[m] : a.tau[m]; }
+// Dirichlet: the ghost data's parts at the stage time.
+template <int NG>
+__device__ __forceinline__ void ghost_get(const FaceArgs& a, unsigned b, float (&v)[NG + 1]) {
+#pragma unroll
+  for (int c = 0; c <= NG; ++c) v[c] = 0.f;
+  if (b >= (unsigned)a.B) return;
+  for (int m = 0; m < a.nghost; ++m) {
+    const float* gp = a.gpart + ((int64_t)m * a.B + b) * (NG + 1);
+    const float tm = stage_tau(a, RDG_MAX_FORCING_TERMS + m);
+#pragma unroll
+    for (int c = 0; c <= NG; ++c) v[c] = fmaf(tm, gp[c], v[c]);
+  }
+}
+template <int NG>
+__device__ __forceinline__ void record_put(float* buf, size_t K3, unsigned r, const float (&v)[NG]) {
+  constexpr int N4 = NG / 4 * 4, N2 = N4 + (NG - N4) / 2 * 2;
+  if constexpr (NG >= 4) reinterpret_cast<float4*>(buf)[r] = make_float4(v[0], v[1], v[2], v[3]);
+  if constexpr (N2 > N4) reinterpret_cast<float2*>(buf + N4 * K3)[r] = make_float2(v[N4], v[N4 + 1]);
+  if constexpr (NG > N2) (buf + N2 * K3)[r] = v[N2];
 }
 
 // Parts of element k (values v) through its three faces into the record planes.
-template <int N, bool ALG1>
-__device__ __forceinline__ void store_parts(const float (&v)[np_of(N)], const float4 (&pa)[3], const float4 (&pb)[3],
-                                            float2* out, int64_t K, int64_t k, bool active) {
-  using O = face::Ops<N>;
-  constexpr int NP = np_of(N), RP = face::rec_pairs(N), G = O::GE + O::GO;
+template <int N, bool ALG1, bool ROLL>
+__device__ __forceinline__ void store_parts(const FaceArgs& a, const float (&v)[np_of(N)], const face::Par<float> (&par)[3],
+                                            const bool (&diff)[3], unsigned k, bool active) {
+  constexpr int NP = np_of(N), NG = N + 1;
+  const size_t K3 = 3 * (size_t)a.K;
   float d[NP];
 #pragma unroll
   for (int j = 0; j < NP; ++j) d[j] = v[j] - v[0];
   auto one = [&](auto face_c) {
     constexpr int F = decltype(face_c)::value;
-    float g[2 * RP];
-    // the own-minus-neighbour weights are zero wherever D does not jump: skipped for whole warps
-    const bool diff = ALG1 && __any_sync(0xffffffffu, pb[F].x != 0.f || pb[F].y != 0.f);
-    face::face_part<float, N, F, ALG1>(d, face_par(pa[F], pb[F]), diff, g);
-    g[G] = v[0];
-    if constexpr (G + 1 < 2 * RP) g[G + 1] = 0.f;
-    if (active) {
-#pragma unroll
-      for (int c = 0; c < RP; ++c) out[(int64_t)(F * RP + c) * K + k] = make_float2(g[2 * c], g[2 * c + 1]);
-    }
+    float g[NG];
+    face::face_part<float, N, F, ALG1>(d, par[F], diff[F], g);
+    if (active) record_put<NG>(a.fout, K3, (unsigned)F * (unsigned)a.K + k, g);
   };
-  one(std::integral_constant<int, 0>{});
-  one(std::integral_constant<int, 1>{});
-  one(std::integral_constant<int, 2>{});
+  if constexpr (ROLL) {
+    face::Par<float> p = par[1];
+    bool df = diff[1];
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+      const int f = i == 2 ? 0 : i + 1;
+      float g[NG];
+      face::face_part<float, N, 1, ALG1>(d, p, df, g);
+      if (active) record_put<NG>(a.fout, K3, (unsigned)f * (unsigned)a.K + k, g);
+      face::Ops<N>::rotate(d);
+      p = i == 0 ? par[2] : par[0];
+      df = i == 0 ? diff[2] : diff[0];
+    }
+  } else {
+    one(std::integral_constant<int, 0>{});
+    one(std::integral_constant<int, 1>{});
+    one(std::integral_constant<int, 2>{});
+  }
+  if (active) (a.fout + NG * K3)[k] = v[0];
 }
 
-// Parts of the stage input's elements [a.k_begin, a.K) (k_begin a multiple of 4: 16-byte rows).
+// Parts of the stage input's elements [k_begin, k_end) (k_begin a multiple of 4: 16-byte rows).
 template <int N, bool ALG1>
-__global__ void __launch_bounds__(face_block<N>(), face_min_blocks<N>()) face_parts_kernel(FaceArgs a) {
-  constexpr int NP = np_of(N), BLK = face_block<N>();
-  __shared__ __align__(16) float shs[BLK * NP];
-  const int64_t k0 = a.k_begin + (int64_t)blockIdx.x * BLK;
-  const int nk = (int)min((int64_t)BLK, a.k_end - k0);
-  const int tid = threadIdx.x;
-  const bool active = tid < nk;
-  const int64_t k = k0 + (active ? tid : nk - 1);
-  float4 pa[3], pb[3];
+__global__ void __launch_bounds__(kFaceBlock, face_build<N, false>().blocks) face_parts_kernel(const __grid_constant__ FaceArgs a) {
+  constexpr int NP = np_of(N);
+  __shared__ __align__(16) float shs[kFaceWarps][32 * NP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t k0 = a.k_begin + ((int64_t)blockIdx.x * kFaceWarps + warp) * 32;
+  const int nk = (int)min((int64_t)32, a.k_end - k0);
+  if (nk <= 0) return;
+  const bool active = lane < nk;
+  const int row = active ? lane : nk - 1;
+  const unsigned k = (unsigned)(k0 + row);
+  face::Par<float> par[3];
+  bool diff[3];
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
-    pa[f] = __ldg(a.par + (int64_t)(2 * f) * a.K + k);
-    pb[f] = __ldg(a.par + (int64_t)(2 * f + 1) * a.K + k);
+    diff[f] = jump_in_warp<ALG1>(__ldg(a.nbr + (size_t)f * a.K + k));
+    par[f] = face_par(a, f, k, diff[f]);
   }
   wait_for_predecessor();
   allow_dependents();
-  {
-    Staged<float, BLK, NP> gs;
-    gs.load(a.us + k0 * NP, nk * NP);
-    gs.store(shs, nk * NP);
-  }
-  __syncthreads();
+  rows_in<NP>(shs[warp], a.us + k0 * NP, nk * NP, lane);
+  rows_commit();
+  rows_wait<0>();
   float v[NP];
-  row_get<NP>(shs + (active ? tid : nk - 1) * NP, v);
-  store_parts<N, ALG1>(v, pa, pb, a.fout, a.K, k, active);
+  row_get<NP>(shs[warp] + row * NP, v);
+  store_parts<N, ALG1, face_build<N, false>().roll>(a, v, par, diff, k, active);
 }
 
 // Parts of the Dirichlet ghosts' data, one thread per forcing term and boundary edge: the flux is
@@ -128,177 +255,352 @@ __global__ void __launch_bounds__(face_block<N>(), face_min_blocks<N>()) face_pa
 // ghost's shared face is its second, whose node order is the element's own.
 template <int N, bool ALG1>
 __global__ void __launch_bounds__(128) face_ghost_kernel(const float* G, const float4* gpar, int64_t B, int64_t n, float* out) {
-  using O = face::Ops<N>;
-  constexpr int NP = np_of(N), RP = face::rec_pairs(N), NG = O::GE + O::GO;
+  constexpr int NP = np_of(N), NG = N + 1;
   const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (i >= n) return;
   const int64_t b = i % B;
-  float d[NP], g[2 * RP];
+  float d[NP], g[NG];
   const float v0 = G[i * NP];
 #pragma unroll
   for (int j = 0; j < NP; ++j) d[j] = G[i * NP + j] - v0;
-  face::face_part<float, N, 1, ALG1>(d, face_par(gpar[2 * b], gpar[2 * b + 1]), true, g);
-  g[NG] = v0;
-  if constexpr (NG + 1 < 2 * RP) g[NG + 1] = 0.f;
+  const float4 p = gpar[2 * b], q = gpar[2 * b + 1];
+  face::face_part<float, N, 1, ALG1>(d, face::Par<float>{p.x, p.y, p.z, p.w, q.x, q.y, q.z}, true, g);
 #pragma unroll
-  for (int c = 0; c < 2 * RP; ++c) out[i * 2 * RP + c] = g[c];
+  for (int c = 0; c < NG; ++c) out[i * (NG + 1) + c] = g[c];
+  out[i * (NG + 1) + NG] = v0;
 }
 
-template <int N, bool ALG1>
-__global__ void __launch_bounds__(face_block<N>(), face_min_blocks<N>()) face_stage_kernel(FaceArgs a) {
+template <int N, bool ALG1, bool LARGE>
+__global__ void __launch_bounds__(kFaceBlock, face_build<N, LARGE>().blocks)
+    face_stage_kernel(const __grid_constant__ FaceArgs a) {
   using O = face::Ops<N>;
-  constexpr int NP = np_of(N), BLK = face_block<N>(), RP = face::rec_pairs(N), NG = O::GE + O::GO;
-  __shared__ __align__(16) float shs[BLK * NP];
-  __shared__ __align__(16) float shn[BLK * NP];
-  __shared__ float tau_s[RDG_MAX_FORCING_TERMS], tau_g[RDG_MAX_FORCING_TERMS];
-  const int64_t k0 = (int64_t)blockIdx.x * BLK;
-  const int nk = (int)min((int64_t)BLK, a.K - k0);
-  const int tid = threadIdx.x;
-  const bool active = tid < nk;
-  const int row = active ? tid : nk - 1;
-  const int64_t k = k0 + row;
-  // the parameters and coefficients are written by no stage: loaded before the dependency wait
-  float4 pa[3], pb[3];
+  constexpr FaceBuild build = face_build<N, LARGE>();
+  constexpr bool RECS = build.early & 1, PARS = build.early & 2;
+  constexpr int NP = np_of(N), NG = N + 1;
+  static_assert(NG == O::GE + O::GO, "record size");
+  __shared__ __align__(16) float shs_all[kFaceWarps][32 * NP];
+  __shared__ __align__(16) float shn_all[kFaceWarps][32 * NP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float *shs = shs_all[warp], *shn = shn_all[warp];
+  for (int64_t tile = (int64_t)blockIdx.x * kFaceWarps + warp; tile * 32 < a.K; tile += (int64_t)gridDim.x * kFaceWarps) {
+    const int64_t k0 = tile * 32;
+    const int nk = (int)min((int64_t)32, a.K - k0);
+    const bool active = lane < nk;
+    const int row = active ? lane : nk - 1;
+    const unsigned k = (unsigned)(k0 + row), K3 = 3u * (unsigned)a.K;
+    // neighbours, coefficients and parameters are written by no stage: loaded before the dependency wait
+    unsigned nbr[3];
 #pragma unroll
-  for (int f = 0; f < 3; ++f) {
-    pa[f] = __ldg(a.par + (int64_t)(2 * f) * a.K + k);
-    pb[f] = __ldg(a.par + (int64_t)(2 * f + 1) * a.K + k);
+    for (int f = 0; f < 3; ++f) nbr[f] = __ldg(a.nbr + (size_t)f * a.K + k);
+    float geo[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) geo[c] = __ldg(a.geo + (size_t)c * a.K + k);
+    bool diff[3];
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      diff[f] = jump_in_warp<ALG1>(nbr[f]);
+      nbr[f] &= ~kFaceJump;
+    }
+    face::Par<float> par[3];
+    if constexpr (PARS) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) par[f] = face_par(a, f, k, diff[f]);
+    }
+    const bool need_un = a.mode == 2 || a.mode == 3 || (a.mode == 4 && a.rka != 0.f);
+    wait_for_predecessor();
+    allow_dependents();
+    rows_in<NP>(shs, a.us + k0 * NP, nk * NP, lane);
+    rows_commit();
+    if (need_un) rows_in<NP>(shn, a.un + k0 * NP, nk * NP, lane);
+    rows_commit();
+    float own[RECS ? 3 : 1][NG], nb[RECS ? 3 : 1][NG + 1];
+    auto records = [&](int f, float (&og)[NG], float (&ng)[NG + 1]) {
+      record_get<NG>(a.fin, K3, (unsigned)f * (unsigned)a.K + k, og);
+      neighbour_get<NG>(a, nbr[f], k, ng);
+    };
+    if constexpr (RECS) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) records(f, own[f], nb[f]);
+    }
+    rows_wait<1>();
+    float rhs[NP], u0;
+    {
+      float ve[O::NE], vo[O::NO];
+      {
+        float d[NP];
+        row_get<NP>(shs + row * NP, d);
+        u0 = d[0];
+#pragma unroll
+        for (int j = 0; j < NP; ++j) d[j] -= u0;
+        face::volume_parts<float, N>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      }
+      auto flux = [&](int f, float (&ge)[O::GE], float (&go)[O::GO]) {
+        float (&og)[NG] = own[RECS ? f : 0], (&ng)[NG + 1] = nb[RECS ? f : 0];
+        if constexpr (!RECS) records(f, og, ng);
+        const face::Par<float> p = PARS ? par[f] : face_par(a, f, k, diff[f]);
+        if (nbr[f] >= K3) ghost_get<NG>(a, nbr[f] - K3, ng);
+#pragma unroll
+        for (int q = 0; q < O::GE; ++q) ge[q] = og[q];
+#pragma unroll
+        for (int q = 0; q < O::GO; ++q) go[q] = og[O::GE + q];
+        face::face_flux<float, N, ALG1>(p, diff[f], u0, ng[NG], ng, ge, go);
+        const float mj = -geo[5];
+#pragma unroll
+        for (int q = 0; q < O::GE; ++q) ge[q] *= mj;
+#pragma unroll
+        for (int q = 0; q < O::GO; ++q) go[q] *= mj;
+      };
+      float ge[O::GE], go[O::GO];
+      if constexpr (build.roll) {
+        O::nodes(ve, vo, rhs);
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) {
+          if (i == 0) flux(1, ge, go);
+          else if (i == 1) flux(2, ge, go);
+          else flux(0, ge, go);
+#pragma unroll
+          for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+#pragma unroll
+          for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+          O::lift_even(ge, ve);
+          O::lift_odd(go, vo);
+          O::join1(ve, vo, rhs);
+          O::rotate(rhs);
+        }
+      } else {
+      flux(1, ge, go);              // the second face's order is the element's own
+      O::lift_even(ge, ve);
+      O::lift_odd(go, vo);
+      O::nodes(ve, vo, rhs);
+#pragma unroll
+      for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+#pragma unroll
+      for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+      flux(0, ge, go);
+      O::lift_even(ge, ve);
+      O::lift_odd(go, vo);
+      O::join0(ve, vo, rhs);
+#pragma unroll
+      for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+#pragma unroll
+      for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+      flux(2, ge, go);
+      O::lift_even(ge, ve);
+      O::lift_odd(go, vo);
+      O::join2(ve, vo, rhs);
+      }
+    }
+    for (int m = 0; m < a.nsrc; ++m) {
+      float S[NP];
+      row_get<NP>(a.S + ((int64_t)m * a.K + k) * NP, S);
+      const float tm = stage_tau(a, m);
+#pragma unroll
+      for (int i = 0; i < NP; ++i) rhs[i] = fmaf(tm, S[i], rhs[i]);
+    }
+    rows_wait<0>();
+    if (a.mode >= 1) {
+      float us[NP], un[NP];
+      row_get<NP>(shs + row * NP, us);
+      if (a.mode == 4) {
+        // low-storage stage: du' = rka du + dt L, u' = u + rkb du'
+        if (need_un) {
+          row_get<NP>(shn + row * NP, un);
+#pragma unroll
+          for (int i = 0; i < NP; ++i) un[i] = fmaf(a.rka, un[i], a.dt * rhs[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < NP; ++i) un[i] = a.dt * rhs[i];
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.rkb, un[i], us[i]);
+        __syncwarp();
+        if (active) row_put<NP>(shn + lane * NP, un);
+      } else {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.dt, rhs[i], us[i]);
+        if (need_un) {
+          const float c = a.mode == 2 ? 0.25f : (float)(2.0 / 3.0);   // see rk_combine
+          row_get<NP>(shn + row * NP, un);
+#pragma unroll
+          for (int i = 0; i < NP; ++i) rhs[i] = fmaf(c, rhs[i] - un[i], un[i]);
+        }
+      }
+    }
+    __syncwarp();
+    if (active) row_put<NP>(shs + lane * NP, rhs);
+    __syncwarp();
+    rows_out<NP>(a.out + k0 * NP, shs, nk * NP, lane);
+    if (a.mode == 4) rows_out<NP>(a.out2 + k0 * NP, shn, nk * NP, lane);
+    if (a.fout) {
+      if constexpr (!PARS) {
+#pragma unroll
+        for (int f = 0; f < 3; ++f) par[f] = face_par(a, f, k, diff[f]);
+      }
+      store_parts<N, ALG1, build.roll>(a, rhs, par, diff, k, active);
+    }
+    __syncwarp();
+  }
+}
+
+// The same stage with four warps on 32 elements: each warp takes a quarter of the volume term, and
+// the last three one face each (flux and LIFT before the update, the new parts after it).  A thread of
+// face_stage_kernel walks the whole chain alone (N = 4: 1900 instructions, about 1.8 us for a lone
+// warp), which sets the stage time where there are few warps per scheduler; here the chain is about a
+// third as long.
+template <int N, bool ALG1>
+__global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const __grid_constant__ FaceArgs a) {
+  using O = face::Ops<N>;
+  constexpr int NP = np_of(N), NG = N + 1, V4 = (NP * 8 + 127) / 128;
+  __shared__ __align__(16) float su[32 * NP];
+  __shared__ __align__(16) float sp[4][32 * NP];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t k0 = (int64_t)blockIdx.x * 32;
+  const int nk = (int)min((int64_t)32, a.K - k0), n = nk * NP, nv = n / 4;
+  const bool active = lane < nk;
+  const int row = active ? lane : nk - 1;
+  const unsigned k = (unsigned)(k0 + row), K = (unsigned)a.K, K3 = 3u * K;
+  const int f = warp - 1;               // this warp's face (none for warp 0)
+  unsigned nbr = 0;
+  bool diff = false;
+  face::Par<float> par{};
+  if (f >= 0) {
+    nbr = __ldg(a.nbr + (size_t)f * K + k);
+    diff = jump_in_warp<ALG1>(nbr);
+    nbr &= ~kFaceJump;
+    par = face_par(a, f, k, diff);
   }
   float geo[6];
 #pragma unroll
-  for (int c = 0; c < 6; ++c) geo[c] = __ldg(a.geo + c * a.K + k);
+  for (int c = 0; c < 6; ++c) geo[c] = __ldg(a.geo + (size_t)c * K + k);
   const bool need_un = a.mode == 2 || a.mode == 3 || (a.mode == 4 && a.rka != 0.f);
   wait_for_predecessor();
   allow_dependents();
-  float2 own[3][RP], nb[3][RP];
-  {
-    Staged<float, BLK, NP> gs, gn;
-    gs.load(a.us + k0 * NP, nk * NP);
-    if (need_un) gn.load(a.un + k0 * NP, nk * NP);
+  const float4* us4 = reinterpret_cast<const float4*>(a.us + k0 * NP);
+  float4 un4[V4];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
-#pragma unroll
-      for (int c = 0; c < RP; ++c) own[f][c] = a.fin[(int64_t)(f * RP + c) * a.K + k];
-      const unsigned r = __float_as_uint(pb[f].w), fn = r & 3u;
-      int64_t kn = r >> 2;
-      if (fn != 3u && kn >= a.K) {   // self-check: record and read the own record instead
-        report(a.err, kErrBadIndex);
-        kn = k;
-      }
-#pragma unroll
-      for (int c = 0; c < RP; ++c)
-        nb[f][c] = fn != 3u ? a.fin[(int64_t)(fn * RP + c) * a.K + kn] : make_float2(0.f, 0.f);
-    }
-    gs.store(shs, nk * NP);
-    if (need_un) gn.store(shn, nk * NP);
+  for (int j = 0; j < V4; ++j) {
+    const int i = tid + 128 * j;
+    if (i < nv)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(su + 4 * i)),
+                   "l"(us4 + i)
+                   : "memory");
+    un4[j] = need_un && i < nv ? reinterpret_cast<const float4*>(a.un + k0 * NP)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  if (tid < a.frc.nsrc) tau_s[tid] = (float)tau_of(a.frc.kind[tid], a.frc.omega[tid], stage_time(a.time));
-  if (tid < a.frc.nghost) tau_g[tid] = (float)tau_of(a.frc.gkind[tid], a.frc.gomega[tid], stage_time(a.time));
+  if (nv * 4 + tid < n) su[nv * 4 + tid] = a.us[k0 * NP + nv * 4 + tid];
+  rows_commit();
+  float own[NG], nb[NG + 1];
+  if (f >= 0) {
+    record_get<NG>(a.fin, K3, (unsigned)f * K + k, own);
+    neighbour_get<NG>(a, nbr, k, nb);
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  float rhs[NP], u0;
   {
-    float ve[O::NE], vo[O::NO];
-    {
-      float d[NP];
-      row_get<NP>(shs + row * NP, d);
-      u0 = d[0];
+    float d[NP], rhs[NP], ve[O::NE], vo[O::NO], ge[O::GE], go[O::GO];
+    row_get<NP>(su + row * NP, d);
+    const float u0 = d[0];
 #pragma unroll
-      for (int j = 0; j < NP; ++j) d[j] -= u0;
-      face::volume_parts<float, N>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
-    }
-    auto flux = [&](int f, float (&ge)[O::GE], float (&go)[O::GO]) {
-      float ng[2 * RP], og[2 * RP];
+    for (int j = 0; j < NP; ++j) d[j] -= u0;
+    auto flux = [&]() {
+      if (nbr >= K3) ghost_get<NG>(a, nbr - K3, nb);
 #pragma unroll
-      for (int c = 0; c < RP; ++c) {
-        og[2 * c] = own[f][c].x, og[2 * c + 1] = own[f][c].y;
-        ng[2 * c] = nb[f][c].x, ng[2 * c + 1] = nb[f][c].y;
-      }
-      const unsigned r = __float_as_uint(pb[f].w);
-      if ((r & 3u) == 3u && a.frc.nghost > 0) {   // Dirichlet: the ghost data's parts at the stage time
-        const int64_t b = r >> 2;
-        if (b < a.B) {
-          for (int m = 0; m < a.frc.nghost; ++m) {
-            const float* gp = a.gpart + ((int64_t)m * a.B + b) * 2 * RP;
-            const float tm = tau_g[m];
+      for (int q = 0; q < O::GE; ++q) ge[q] = own[q];
 #pragma unroll
-            for (int c = 0; c <= NG; ++c) ng[c] = fmaf(tm, gp[c], ng[c]);
-          }
-        } else {
-          report(a.err, kErrBadIndex);
-        }
-      }
+      for (int q = 0; q < O::GO; ++q) go[q] = own[O::GE + q];
+      face::face_flux<float, N, ALG1>(par, diff, u0, nb[NG], nb, ge, go);
 #pragma unroll
-      for (int q = 0; q < O::GE; ++q) ge[q] = og[q];
+      for (int q = 0; q < O::GE; ++q) ge[q] *= -geo[5];
 #pragma unroll
-      for (int q = 0; q < O::GO; ++q) go[q] = og[O::GE + q];
-      face::face_flux<float, N, ALG1>(face_par(pa[f], pb[f]), u0, ng[NG], ng, ge, go);
-      const float mj = -geo[5];
-#pragma unroll
-      for (int q = 0; q < O::GE; ++q) ge[q] *= mj;
-#pragma unroll
-      for (int q = 0; q < O::GO; ++q) go[q] *= mj;
+      for (int q = 0; q < O::GO; ++q) go[q] *= -geo[5];
     };
-    float ge[O::GE], go[O::GO];
-    flux(1, ge, go);              // the second face's order is the element's own
-    O::lift_even(ge, ve);
-    O::lift_odd(go, vo);
-    O::nodes(ve, vo, rhs);
+    auto clear = [&]() {
 #pragma unroll
-    for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+      for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
 #pragma unroll
-    for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
-    flux(0, ge, go);
-    O::lift_even(ge, ve);
-    O::lift_odd(go, vo);
-    O::join0(ve, vo, rhs);
-#pragma unroll
-    for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
-#pragma unroll
-    for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
-    flux(2, ge, go);
-    O::lift_even(ge, ve);
-    O::lift_odd(go, vo);
-    O::join2(ve, vo, rhs);
+      for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+    };
+    auto lift = [&]() {
+      O::lift_even(ge, ve);
+      O::lift_odd(go, vo);
+    };
+    if (warp == 0) {
+      face::volume_parts<float, N, 0>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      O::nodes(ve, vo, rhs);
+    } else if (warp == 1) {
+      face::volume_parts<float, N, 1>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      O::nodes(ve, vo, rhs);
+      flux();
+      clear();
+      lift();
+      O::join0(ve, vo, rhs);
+    } else if (warp == 2) {
+      face::volume_parts<float, N, 2>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      flux();
+      lift();                           // the second face's order is the element's own
+      O::nodes(ve, vo, rhs);
+    } else {
+      face::volume_parts<float, N, 3>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      O::nodes(ve, vo, rhs);
+      flux();
+      clear();
+      lift();
+      O::join2(ve, vo, rhs);
+    }
+    if (active) row_put<NP>(sp[warp] + lane * NP, rhs);
   }
-  for (int m = 0; m < a.frc.nsrc; ++m) {
-    float S[NP];
-    row_get<NP>(a.S + ((int64_t)m * a.K + k) * NP, S);
-    const float tm = tau_s[m];
-#pragma unroll
-    for (int i = 0; i < NP; ++i) rhs[i] = fmaf(tm, S[i], rhs[i]);
-  }
-  if (a.mode >= 1) {
-    float us[NP], un[NP];
-    row_get<NP>(shs + row * NP, us);
+  __syncthreads();
+  // the update, value by value: any thread, any value of the tile
+  const int64_t g0 = k0 * NP;
+  auto update = [&](int i, float un, float& du) {
+    float v = (sp[0][i] + sp[1][i]) + (sp[2][i] + sp[3][i]);
+    for (int m = 0; m < a.nsrc; ++m) v = fmaf(stage_tau(a, m), a.S[(int64_t)m * a.K * NP + g0 + i], v);
+    if (a.mode == 0) return v;
+    const float us = su[i];
     if (a.mode == 4) {
       // low-storage stage: du' = rka du + dt L, u' = u + rkb du'
-      if (need_un) {
-        row_get<NP>(shn + row * NP, un);
+      du = need_un ? fmaf(a.rka, un, a.dt * v) : a.dt * v;
+      return fmaf(a.rkb, du, us);
+    }
+    v = fmaf(a.dt, v, us);
+    return need_un ? fmaf(a.mode == 2 ? 0.25f : (float)(2.0 / 3.0), v - un, un) : v;   // see rk_combine
+  };
 #pragma unroll
-        for (int i = 0; i < NP; ++i) un[i] = fmaf(a.rka, un[i], a.dt * rhs[i]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) un[i] = a.dt * rhs[i];
-      }
-#pragma unroll
-      for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.rkb, un[i], us[i]);
-      if (active) row_put<NP>(shn + tid * NP, un);
-    } else {
-#pragma unroll
-      for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.dt, rhs[i], us[i]);
-      if (need_un) {
-        const float c = a.mode == 2 ? 0.25f : (float)(2.0 / 3.0);   // see rk_combine
-        row_get<NP>(shn + row * NP, un);
-#pragma unroll
-        for (int i = 0; i < NP; ++i) rhs[i] = fmaf(c, rhs[i] - un[i], un[i]);
-      }
+  for (int j = 0; j < V4; ++j) {
+    const int i = tid + 128 * j;
+    if (i < nv) {
+      float4 v, du;
+      v.x = update(4 * i, un4[j].x, du.x);
+      v.y = update(4 * i + 1, un4[j].y, du.y);
+      v.z = update(4 * i + 2, un4[j].z, du.z);
+      v.w = update(4 * i + 3, un4[j].w, du.w);
+      reinterpret_cast<float4*>(su)[i] = v;
+      reinterpret_cast<float4*>(a.out + g0)[i] = v;
+      if (a.mode == 4) reinterpret_cast<float4*>(a.out2 + g0)[i] = du;
     }
   }
-  if (active) row_put<NP>(shs + tid * NP, rhs);   // a thread rewrites only its own row
+  if (nv * 4 + tid < n) {
+    const int i = nv * 4 + tid;
+    float du = 0.f;
+    const float v = update(i, need_un ? a.un[g0 + i] : 0.f, du);
+    su[i] = v;
+    a.out[g0 + i] = v;
+    if (a.mode == 4) a.out2[g0 + i] = du;
+  }
+  if (!a.fout) return;
   __syncthreads();
-  stage_out(a.out + k0 * NP, shs, nk * NP);
-  if (a.mode == 4) stage_out(a.out2 + k0 * NP, shn, nk * NP);
-  if (a.fout) store_parts<N, ALG1>(rhs, pa, pb, a.fout, a.K, k, active);
+  if (f >= 0) {
+    float d[NP], g[NG];
+    row_get<NP>(su + row * NP, d);
+    const float v0 = d[0];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) d[j] -= v0;
+    if (f == 0) face::face_part<float, N, 0, ALG1>(d, par, diff, g);
+    else if (f == 1) face::face_part<float, N, 1, ALG1>(d, par, diff, g);
+    else face::face_part<float, N, 2, ALG1>(d, par, diff, g);
+    if (active) record_put<NG>(a.fout, K3, (unsigned)f * K + k, g);
+  } else if (active) {
+    (a.fout + (size_t)NG * K3)[k] = su[lane * NP];
+  }
 }
 
 }  // namespace dev

@@ -31,9 +31,6 @@ namespace face {
 template <int N>
 struct Ops;
 
-// Values of one face record: even and odd flux parts and u_0, padded to pairs.
-RDG_HD constexpr int rec_pairs(int N) { return (N + 3) / 2; }
-
 template <typename T>
 struct Par {
   T c, h, A, B, C, D, s;
@@ -96,7 +93,7 @@ RDG_HD __forceinline__ void face_part(const T* d, const Par<T>& p, bool diff, T*
 // Flux out of the own element from both sides' parts: on return ge, go hold its even and odd
 // components.  u0, n0: the two sides' reference values; ng: the neighbour's part.
 template <typename T, int N, bool ALG1>
-RDG_HD __forceinline__ void face_flux(const Par<T>& p, T u0, T n0, const T* ng, T* ge, T* go) {
+RDG_HD __forceinline__ void face_flux(const Par<T>& p, bool diff, T u0, T n0, const T* ng, T* ge, T* go) {
   using O = Ops<N>;
   const T jump = u0 - n0, base = p.s * (p.s > T(0) ? u0 : n0);
   T z[O::GE];
@@ -106,27 +103,32 @@ RDG_HD __forceinline__ void face_flux(const Par<T>& p, T u0, T n0, const T* ng, 
   else O::alg2_jump_a(p.A, z);
 #pragma unroll
   for (int q = 0; q < O::GE; ++q) ge[q] = (ge[q] - ng[q]) + fma(z[q], jump, base);
-  if constexpr (ALG1) {
+#pragma unroll
+  for (int q = 0; q < O::GO; ++q) go[q] += ng[O::GE + q];
+  if (ALG1 && diff) {
 #pragma unroll
     for (int q = 0; q < O::GO; ++q) z[q] = T(0);
     O::alg1_jump_d(p.D, z);
 #pragma unroll
-    for (int q = 0; q < O::GO; ++q) go[q] = fma(z[q], jump, go[q] + ng[O::GE + q]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < O::GO; ++q) go[q] += ng[O::GE + q];
+    for (int q = 0; q < O::GO; ++q) go[q] = fma(z[q], jump, go[q]);
   }
 }
 
 // Volume term in mirror components (halves: node = e + o, mirror node = e - o) from the element's
 // coefficients a_r, a_s, g_rr, g_rs, g_ss.
-template <typename T, int N>
+// SHARE 0..3: one of four nearly equal parts of the sum, -1: all of it.
+template <typename T, int N, int SHARE = -1>
 RDG_HD __forceinline__ void volume_parts(const T* d, T u0, T ar, T as, T grr, T grs, T gss, T* ve, T* vo) {
   using O = Ops<N>;
   T e[O::NE], o[O::NO];
   O::split1(d, e, o);
   const T gm = T(0.5) * (grr + gss);
-  O::volume(e, o, u0, ar + as, ar - as, gm + grs, T(0.5) * (grr - gss), gm - grs, ve, vo);
+  const T al = ar + as, am = ar - as, be = gm + grs, ga = T(0.5) * (grr - gss), de = gm - grs;
+  if constexpr (SHARE < 0) O::volume(e, o, u0, al, am, be, ga, de, ve, vo);
+  else if constexpr (SHARE == 0) O::volume0(e, o, u0, al, am, be, ga, de, ve, vo);
+  else if constexpr (SHARE == 1) O::volume1(e, o, u0, al, am, be, ga, de, ve, vo);
+  else if constexpr (SHARE == 2) O::volume2(e, o, u0, al, am, be, ga, de, ve, vo);
+  else O::volume3(e, o, u0, al, am, be, ga, de, ve, vo);
 }
 
 }  // namespace face

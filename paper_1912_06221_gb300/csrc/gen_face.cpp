@@ -195,6 +195,15 @@ struct Gen {
       }
       close();
     }
+    // the element's values in the next face's order: faces 1, 2, 0 (and back to 1) in turn
+    for (int l = 0; l < Np; ++l)
+      if (P[2][P[2][l]] != P[0][l] || P[2][P[0][l]] != l) { std::fprintf(stderr, "face orderings are not a rotation\n"); std::exit(1); }
+    open("rotate(T* v)");
+    for (int l = 0; l < Np; ++l) {   // cycles of three
+      const int b = P[2][l], c = P[2][b];
+      if (l < b && l < c) std::printf("    { const T t = v[%d]; v[%d] = v[%d]; v[%d] = v[%d]; v[%d] = t; }\n", l, l, b, b, c, c);
+    }
+    close();
     open("nodes(const T* e, const T* o, T* v)");
     for (int c = 0; c < NE; ++c) {
       const int i = er[c], j = mir[er[c]];
@@ -350,49 +359,72 @@ struct Gen {
     Mat Wp = add(o->Wr, o->Ws, 1), Wm = add(o->Wr, o->Ws, -1);
     for (auto& v : Wp) v *= 0.5;
     for (auto& v : Wm) v *= 0.5;
-    open("volume(const T* e, const T* o, T u0, T al, T am, T be, T ga, T de, T* ve, T* vo)");
-    bool bege = false, bego = false;
-    for (int odd = 0; odd < 2; ++odd) {
-      const Mat Rp = comp(Dp, !odd, !odd, false), Rm = comp(Dm, !odd, odd, false);
-      const Mat Cp = comp(Wp, !odd, !odd, true), Cm = comp(Wm, odd, !odd, true);
-      const int n = odd ? NO : NE, mo = odd ? NE : NO;   // this parity's components, the other's
-      for (int q = 0; q < n; ++q) {
-        std::printf("    {\n      T p, m;\n");
-        auto row = [&](const Mat& R, int cols, const char* x, const char* y, bool skip0) {
-          double top = 0;
-          for (double v : R) top = std::max(top, std::fabs(v));
-          bool begun = false;
-          for (int c = 0; c < cols; ++c) {
-            const double v = R[(size_t)q * cols + c];
-            if ((skip0 && c == zero) || std::fabs(v) <= 1e-13 * top) continue;   // d at node 0 is zero
-            if (begun) std::printf("      %s = fma(%s, %s[%d], %s);\n", y, lit(v).c_str(), x, c, y);
-            else std::printf("      %s = %s * %s[%d];\n", y, lit(v).c_str(), x, c);
-            begun = true;
-          }
-          if (!begun) std::printf("      %s = T(0);\n", y);
-        };
-        row(Rp, n, odd ? "o" : "e", "p", !odd);
-        row(Rm, mo, odd ? "e" : "o", "m", odd);
-        if (odd) std::printf("      const T u = T(0.5) * o[%d];\n", q);
-        else if (mir[er[q]] == er[q]) std::printf("      const T u = e[%d] + u0;\n", q);
-        else std::printf("      const T u = fma(T(0.5), e[%d], u0);\n", q);
-        std::printf("      const T fp = al * u - (be * p + ga * m), fm = am * u - (ga * p + de * m);\n");
-        auto col = [&](const Mat& C, int rows, const char* f, const char* y, bool& begun) {
-          double top = 0;
-          for (double v : C) top = std::max(top, std::fabs(v));
-          for (int i = 0; i < rows; ++i) {
-            const double v = C[(size_t)i * n + q];
-            if (!begun) std::printf("      %s[%d] = %s * %s;\n", y, i, lit(v).c_str(), f);
-            else if (std::fabs(v) > 1e-13 * top) std::printf("      %s[%d] = fma(%s, %s, %s[%d]);\n", y, i, lit(v).c_str(), f, y, i);
-          }
-          begun = true;
-        };
-        col(Cp, n, "fp", odd ? "vo" : "ve", odd ? bego : bege);
-        col(Cm, mo, "fm", odd ? "ve" : "vo", odd ? bege : bego);
-        std::printf("    }\n");
+    // volume: all components; volume0..3: the components' products split into four nearly equal shares
+    // for four warps that work on the same elements, the last three also having a face's flux and LIFT
+    std::vector<int> share(NE + NO, 0);
+    {
+      std::vector<double> load = {0.0, 1, 1, 1};
+      const double face = 3.0 * GE + 3.0 * GO + NE * GE + NO * GO + NE + 2.0 * NO + 8;
+      for (int w = 1; w < 4; ++w) load[w] = face;
+      for (int q = 0; q < NE + NO; ++q) {
+        int best = 0;
+        for (int w = 1; w < 4; ++w)
+          if (load[w] < load[best]) best = w;
+        share[q] = best;
+        load[best] += 2.0 * Np + 7;
       }
     }
-    close();
+    for (int part = -1; part < 4; ++part) {
+      char sig[160];
+      std::snprintf(sig, sizeof sig, "volume%s(const T* e, const T* o, T u0, T al, T am, T be, T ga, T de, T* ve, T* vo)",
+                    part < 0 ? "" : std::to_string(part).c_str());
+      open(sig);
+      bool bege = false, bego = false;
+      for (int odd = 0; odd < 2; ++odd) {
+        const Mat Rp = comp(Dp, !odd, !odd, false), Rm = comp(Dm, !odd, odd, false);
+        const Mat Cp = comp(Wp, !odd, !odd, true), Cm = comp(Wm, odd, !odd, true);
+        const int n = odd ? NO : NE, mo = odd ? NE : NO;   // this parity's components, the other's
+        for (int q = 0; q < n; ++q) {
+          if (part >= 0 && share[odd * NE + q] != part) continue;
+          std::printf("    {\n      T p, m;\n");
+          auto row = [&](const Mat& R, int cols, const char* x, const char* y, bool skip0) {
+            double top = 0;
+            for (double v : R) top = std::max(top, std::fabs(v));
+            bool begun = false;
+            for (int c = 0; c < cols; ++c) {
+              const double v = R[(size_t)q * cols + c];
+              if ((skip0 && c == zero) || std::fabs(v) <= 1e-13 * top) continue;   // d at node 0 is zero
+              if (begun) std::printf("      %s = fma(%s, %s[%d], %s);\n", y, lit(v).c_str(), x, c, y);
+              else std::printf("      %s = %s * %s[%d];\n", y, lit(v).c_str(), x, c);
+              begun = true;
+            }
+            if (!begun) std::printf("      %s = T(0);\n", y);
+          };
+          row(Rp, n, odd ? "o" : "e", "p", !odd);
+          row(Rm, mo, odd ? "e" : "o", "m", odd);
+          if (odd) std::printf("      const T u = T(0.5) * o[%d];\n", q);
+          else if (mir[er[q]] == er[q]) std::printf("      const T u = e[%d] + u0;\n", q);
+          else std::printf("      const T u = fma(T(0.5), e[%d], u0);\n", q);
+          std::printf("      const T fp = al * u - (be * p + ga * m), fm = am * u - (ga * p + de * m);\n");
+          auto col = [&](const Mat& C, int rows, const char* f, const char* y, bool& begun) {
+            double top = 0;
+            for (double v : C) top = std::max(top, std::fabs(v));
+            for (int i = 0; i < rows; ++i) {
+              const double v = C[(size_t)i * n + q];
+              if (!begun) std::printf("      %s[%d] = %s * %s;\n", y, i, lit(v).c_str(), f);
+              else if (std::fabs(v) > 1e-13 * top) std::printf("      %s[%d] = fma(%s, %s, %s[%d]);\n", y, i, lit(v).c_str(), f, y, i);
+            }
+            begun = true;
+          };
+          col(Cp, n, "fp", odd ? "vo" : "ve", odd ? bego : bege);
+          col(Cm, mo, "fm", odd ? "ve" : "vo", odd ? bege : bego);
+          std::printf("    }\n");
+        }
+      }
+      for (int i = 0; i < NE && !bege; ++i) std::printf("    ve[%d] = T(0);\n", i);
+      for (int i = 0; i < NO && !bego; ++i) std::printf("    vo[%d] = T(0);\n", i);
+      close();
+    }
     std::printf("};\n");
   }
 };

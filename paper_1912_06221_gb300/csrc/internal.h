@@ -95,23 +95,31 @@ struct ElemArgs {
   T rka, rkb;
 };
 
+constexpr unsigned kFaceJump = 0x80000000u;
 // Face form of a stage (face_kernels.cuh): FP32, element-wise D.
 struct FaceArgs {
   const float* us;        // stage input
   const float* un;        // step start, or the low-storage residual register
   float* out;
   float* out2;            // low-storage stage: the residual register written
-  const float2* fin;      // face records of the stage input, planes [3 RP][K]
-  float2* fout;           // records of the stage's result, or null: not wanted
-  const float4* par;      // face parameters [3][2][K]: {c, h, A, B}, {C, D, s, neighbour}; neighbour =
-                          // 4 element + face, or 4 boundary edge + 3
+  const float* fin;       // face records of the stage input (face_kernels.cuh)
+  float* fout;            // records of the stage's result, or null: not wanted
+  // face parameters, each [3][K]: {c, h, A, B}; {C, D}; s; the neighbour's record, face K + element,
+  // or 3 K + boundary edge, with kFaceJump set where C or D is not zero
+  const float4* p4;
+  const float2* p2;
+  const float* p1;
+  const unsigned* nbr;
   const float* geo;       // [6][K]
   const float* S;         // [nsrc][K][Np]
-  const float* gpart;     // parts of the ghost data [nghost][B][2 RP]
+  const float* gpart;     // parts of the ghost data and its reference value [nghost][B][N + 2]
   int64_t K, B;
   int64_t k_begin, k_end; // parts kernel: elements of this launch
-  Forcing frc;
-  TimeArg time;
+  // the stage's tau_m(t): nsrc source and nghost ghost terms (at +RDG_MAX_FORCING_TERMS), given here or,
+  // in replayed chunks, in a device row that launch_face_tau fills
+  int nsrc, nghost;
+  const float* tau_row;
+  float tau[2 * RDG_MAX_FORCING_TERMS];
   int* err;               // device error word; may be null
   int mode;               // as below
   float dt, rka, rkb;
@@ -148,7 +156,15 @@ int launch_edge_only64(int N, const EdgeArgs<double>& a, cudaStream_t s);
 int launch_face_parts(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
 int launch_face_stage(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
 int launch_face_ghost(int N, bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out, cudaStream_t s);
-inline int face_rec_pairs(int N) { return (N + 3) / 2; }   // float2 words of a face record
+// Rows of tau values for kTauSteps steps from step n of the replay: row (step, stage) of kTauStages
+// stage offsets, 2 RDG_MAX_FORCING_TERMS floats each.
+constexpr int kTauSteps = 16, kTauStages = 5, kTauRow = 2 * RDG_MAX_FORCING_TERMS;
+struct StageOffsets {
+  double c[kTauStages];
+};
+int launch_face_tau(const Forcing& f, const TimeArg& base, const StageOffsets& off, float* rows, cudaStream_t s);
+double host_tau(int kind, double omega, double t);
+inline int64_t face_rec_floats(int N, int64_t K) { return (3 * (N + 1) + 1) * K; }   // a record buffer
 int gemm_param_words(int N);   // 16-byte words of an edge's parameter record
 
 // ---- setup (FP64) -------------------------------------------------------------------
@@ -174,8 +190,17 @@ struct EdgeSetupIn {
 // (W_dense), and/or the GEMM-form parameter record (P_tiled, FP32); any may be null.
 int setup_edges(int N, const EdgeSetupIn& in, void* W_tiled, int elem_bytes, double* W_dense, float* P_tiled,
                 cudaStream_t s);
-// Face parameters of the face form, FP64 arithmetic: par [3][2][K] and the ghosts' gpar [B][2].
-int setup_faces(const EdgeSetupIn& in, int64_t K, float4* par, float4* gpar, cudaStream_t s);
+// Face parameters of the face form, FP64 arithmetic (layouts of FaceArgs), and the ghosts' [B][2].
+struct FaceTables {
+  float4* p4;
+  float2* p2;
+  float* p1;
+  unsigned* nbr;
+  float4* gpar;
+};
+// Largest mesh of the face form: a record's byte offset in a plane fits 32 bits.
+constexpr int64_t kMaxFaceElements = (int64_t)1 << 27;
+int setup_faces(const EdgeSetupIn& in, int64_t K, const FaceTables& t, cudaStream_t s);
 int setup_elements(int64_t K, const double* xy, const double* D, const double* Dy, double vx, double vy, void* geo,
                    int elem_bytes,
                    cudaStream_t s);

@@ -716,19 +716,6 @@ __global__ void __launch_bounds__(kElemBlock, (N == 1 ? 8 : 1)) elem_fused_kerne
 }  // namespace dev
 
 // Host-side launch helpers instantiated by the including translation unit.
-inline int sm_count() {
-  static int cached[64] = {0};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) return 1;
-  if (!cached[dev]) {
-    int n = 0;
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cached[dev] = n > 0 ? n : 1;
-  }
-  return cached[dev];
-}
-
 template <typename T, int N, bool VOL = false>
 inline int launch_edge_t(const EdgeArgs<T>& a, cudaStream_t s) {
   const int64_t kv = a.Kvol > 0 ? a.Kvol : a.K;

@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(32 * setup_warps<N>()) edge_setup_kernel(EdgeS
 // (w_oR + w_oS + w_nR + w_nS)/4, B = (w_oR - w_oS + w_nR - w_nS)/4, C = (w_oR + w_oS - w_nR - w_nS)/4,
 // D = (w_oR - w_oS - w_nR + w_nS)/4 for own side o and neighbour n (Algorithm 1); the one-coefficient
 // rules use A = (w_R + w_S)/2, B = (w_R - w_S)/2.
-__global__ void __launch_bounds__(128) face_setup_kernel(EdgeSetupIn in, int64_t K, float4* par, float4* gpar) {
+__global__ void __launch_bounds__(128) face_setup_kernel(EdgeSetupIn in, int64_t K, FaceTables t) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= in.E) return;
   const int fb[3] = {1, 2, 0}, fc[3] = {2, 0, 1};
@@ -506,17 +506,22 @@ __global__ void __launch_bounds__(128) face_setup_kernel(EdgeSetupIn in, int64_t
   const float c[2] = {(float)(0.5 * (be[0] - al[0])), (float)(0.5 * (be[1] - al[1]))};
   const float h[2] = {(float)(-0.5 * (al[0] + be[0])), (float)(-0.5 * (al[1] + be[1]))};
   const int64_t bb = -1 - (int64_t)k2;
-  const unsigned r1 = k2 >= 0 ? 4u * (unsigned)k2 + (unsigned)f2 : 4u * (unsigned)bb + 3u;
-  par[(int64_t)(2 * f1) * K + k1] = make_float4(c[0], h[0], A, B);
-  par[(int64_t)(2 * f1 + 1) * K + k1] = make_float4(C, D, s, __uint_as_float(r1));
-  const float4 a2 = make_float4(c[1], h[1], A, B);
-  const float4 b2 = make_float4(-C, -D, -s, __uint_as_float(4u * (unsigned)k1 + (unsigned)f1));
+  const int64_t i1 = (int64_t)f1 * K + k1;
+  const unsigned jump = (C != 0.f || D != 0.f) ? kFaceJump : 0u;
+  t.p4[i1] = make_float4(c[0], h[0], A, B);
+  t.p2[i1] = make_float2(C, D);
+  t.p1[i1] = s;
   if (k2 >= 0) {
-    par[(int64_t)(2 * f2) * K + k2] = a2;
-    par[(int64_t)(2 * f2 + 1) * K + k2] = b2;
+    const int64_t i2 = (int64_t)f2 * K + k2;
+    t.nbr[i1] = (unsigned)i2 | jump;
+    t.p4[i2] = make_float4(c[1], h[1], A, B);
+    t.p2[i2] = make_float2(-C, -D);
+    t.p1[i2] = -s;
+    t.nbr[i2] = (unsigned)i1 | jump;
   } else {
-    gpar[2 * bb] = a2;
-    gpar[2 * bb + 1] = b2;
+    t.nbr[i1] = (unsigned)(3 * K + bb) | jump;
+    t.gpar[2 * bb] = make_float4(c[1], h[1], A, B);
+    t.gpar[2 * bb + 1] = make_float4(-C, -D, -s, 0.f);
   }
 }
 
@@ -551,7 +556,30 @@ __global__ void set_time_kernel(TimeState* ts, double t0) {
   ts->n = 0;
 }
 
+// The double-precision sines and cosines of a chunk's stages, all at once: evaluated inside every
+// stage kernel they cost about 3 us of its 6 (an FP64 warp instruction issues over 64 cycles here).
+__global__ void __launch_bounds__(kTauSteps * kTauStages * kTauRow) face_tau_kernel(Forcing f, TimeArg base, StageOffsets off,
+                                                                                  float* rows) {
+  const int m = threadIdx.x % kTauRow, st = threadIdx.x / kTauRow % kTauStages, step = threadIdx.x / (kTauRow * kTauStages);
+  const bool src = m < RDG_MAX_FORCING_TERMS;
+  const int i = src ? m : m - RDG_MAX_FORCING_TERMS;
+  if (i >= (src ? f.nsrc : f.nghost)) return;
+  const double t = base.ts->t0 + ((double)base.ts->n + (base.off + step + off.c[st])) * base.dt;
+  const int kind = src ? f.kind[i] : f.gkind[i];
+  const double w = src ? f.omega[i] : f.gomega[i];
+  rows[threadIdx.x] = (float)(kind == RDG_TAU_COS ? cos(w * t) : (kind == RDG_TAU_SIN ? sin(w * t) : 1.0));
+}
+
 }  // namespace
+
+int launch_face_tau(const Forcing& f, const TimeArg& base, const StageOffsets& off, float* rows, cudaStream_t s) {
+  face_tau_kernel<<<1, kTauSteps * kTauStages * kTauRow, 0, s>>>(f, base, off, rows);
+  return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
+}
+
+double host_tau(int kind, double omega, double t) {
+  return kind == RDG_TAU_COS ? std::cos(omega * t) : (kind == RDG_TAU_SIN ? std::sin(omega * t) : 1.0);
+}
 
 template <int N>
 int launch_setup(const EdgeSetupIn& in, void* W_tiled, int elem_bytes, double* W_dense, float* P_tiled,
@@ -577,9 +605,9 @@ int setup_edges(int N, const EdgeSetupIn& in, void* W_tiled, int elem_bytes, dou
   }
 }
 
-int setup_faces(const EdgeSetupIn& in, int64_t K, float4* par, float4* gpar, cudaStream_t s) {
+int setup_faces(const EdgeSetupIn& in, int64_t K, const FaceTables& t, cudaStream_t s) {
   if (in.E == 0) return RDG_OK;
-  face_setup_kernel<<<(unsigned)((in.E + 127) / 128), 128, 0, s>>>(in, K, par, gpar);
+  face_setup_kernel<<<(unsigned)((in.E + 127) / 128), 128, 0, s>>>(in, K, t);
   return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
 }
 

@@ -41,7 +41,7 @@ void rhs(int64_t K, const T* u, const double* par, const int64_t* nbr, const dou
       T ge[O::GE], go[O::GO];
       for (int q = 0; q < O::GE; ++q) ge[q] = own[q];
       for (int q = 0; q < O::GO; ++q) go[q] = own[O::GE + q];
-      face::face_flux<T, N, ALG1>(P(k, f), u0, nb[G], nb, ge, go);
+      face::face_flux<T, N, ALG1>(P(k, f), true, u0, nb[G], nb, ge, go);
       for (int q = 0; q < O::GE; ++q) ge[q] *= -(T)g[5];
       for (int q = 0; q < O::GO; ++q) go[q] *= -(T)g[5];
       O::lift_even(ge, ve);

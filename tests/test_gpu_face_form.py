@@ -55,3 +55,19 @@ def test_face_form_matches_fp64(N, m, kind, iface, bc, integ):
     want = _run(N, m, rdg.FP64, kind, iface, bc, integ)
     for a, b in zip(got, want):
         assert parity_err(a, b) < 1e-5
+
+
+# one size per kernel choice beyond the tiny meshes above: more than one tile per SM, and more tiles
+# than the small build holds at once (ragged last tiles)
+LARGE_M = {1: 225, 2: 225, 3: 225, 4: 225, 5: 181, 6: 150}
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("large", [False, True])
+@pytest.mark.parametrize("integ", [rdg.SSP_RK3, rdg.LSRK54])
+def test_face_form_kernel_choice_matches_fp64(N, large, integ):
+    m = LARGE_M[N] if large else 75
+    got = _run(N, m, rdg.FP32, "jump", rdg.IFACE_ALG1, rdg.BC_DIRICHLET, integ)
+    want = _run(N, m, rdg.FP64, "jump", rdg.IFACE_ALG1, rdg.BC_DIRICHLET, integ)
+    for a, b in zip(got, want):
+        assert parity_err(a, b) < 1e-5
