@@ -409,23 +409,21 @@ int rdg_batch_synchronize(rdg_batch* b);
 /* Form of a batch step.  RDG_BATCH_GRAPH: the members' own stage launches as parallel
  * branches of one CUDA graph.  RDG_BATCH_PERSISTENT: one persistent launch per chunk of steps
  * for all members (captured in the CUDA graph like the branches): blocks take work items
- * (member, stage, part, tile) from a ticket counter in stage order; part A of a stage (edge
- * fluxes, volume terms) starts once the member's previous stage is done, part B (surface
- * terms and stage update per element) once the member's part A is done; every wait is
- * bounded (see rdg_batch_set_wait_limit).  It needs every member FP32 with stored operators and the
- * SSP-RK3 integrator (order 6 then forms its volume term on the CUDA cores).  RDG_BATCH_AUTO
- * (the default): persistent when every member fits, else the graph.  The persistent form
- * takes each member's set-up (forcing, dt, tiles) when the membership last changed.
+ * (member, stage, elements) from one ticket counter per order in stage order; a stage of a
+ * member starts once the member's previous stage is done; every wait is bounded (see
+ * rdg_batch_set_wait_limit).  It needs every member FP32 with an element-wise D and the
+ * SSP-RK3 integrator.  RDG_BATCH_AUTO (the default): persistent when every member fits, else
+ * the graph.  The persistent form takes each member's set-up (forcing, dt, tiles) when the
+ * membership last changed.
  * Errors: RDG_EINVAL (unknown mode, or RDG_BATCH_PERSISTENT with a member that does not fit). */
 enum { RDG_BATCH_AUTO = 0, RDG_BATCH_GRAPH = 1, RDG_BATCH_PERSISTENT = 2 };
 int rdg_batch_set_mode(rdg_batch* b, int mode);
 /* The form the next step uses (RDG_BATCH_GRAPH or RDG_BATCH_PERSISTENT) into *mode. */
 int rdg_batch_get_mode(const rdg_batch* b, int* mode);
-/* Tile mapping of the persistent form for members of order N: edges_per_thread (1 or 2)
- * edges per thread of an edge tile (128 or 256 edges per tile; element tiles are 128
- * elements) and tiles_per_item (1, 2 or 4) consecutive tiles per work item, which amortises
- * an item's dependency check over more work.  Chosen per order by the autotuner.  Errors:
- * RDG_EINVAL. */
+/* Tile mapping of the persistent form for members of order N: edges_per_thread (1 or 2) times
+ * tiles_per_item (1, 2 or 4) consecutive tiles per work item (a tile is 128 elements, or 32
+ * for the smaller members of orders 4..6), which amortises an item's dependency check over
+ * more work.  Chosen per order by the autotuner.  Errors: RDG_EINVAL. */
 int rdg_batch_set_tiles(rdg_batch* b, int N, int edges_per_thread, int tiles_per_item);
 /* Bound on every dependency wait of the persistent kernel (default 1 s; (0, 60]): a wait that
  * runs out records the timeout, and the launch ends without finishing its work. */

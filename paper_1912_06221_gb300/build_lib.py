@@ -20,7 +20,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = [("refops.cpp", "refops", []), ("api.cpp", "api", []), ("rhs_dispatch.cpp", "rhs_dispatch", []),
            ("setup.cu", "setup", []), ("rhs_static.cu", "rhs_static", []), ("batch.cpp", "batch", []),
            ("measure.cu", "measure", []), ("halo.cu", "halo", []),
-           ("batch_kernel.cu", "batch_kernel", [])]
+           ("batch_kernel.cu", "batch_kernel", ["-I", os.path.join(OUT, "gen")])]
 for _n in range(1, 7):
     for _t, _tag in (("float", "f"), ("double", "d")):
         SOURCES.append(("rhs_order.cu", "rhs_%s%d" % (_tag, _n),

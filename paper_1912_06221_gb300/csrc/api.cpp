@@ -963,14 +963,14 @@ FaceArgs face_args(const rdg_ctx* ctx, const float* us) {
   a.K = ctx->K;
   a.B = ctx->B;
   a.err = ctx->d_err;
+  a.nsrc = ctx->frc.nsrc;
+  a.nghost = ctx->frc.nghost;
   return a;
 }
 
 // The forcing factors at stage time ta: a row of the replayed chunk's table, or evaluated here.
 void face_forcing(const rdg_ctx* ctx, const TimeArg& ta, int stage, FaceArgs& a) {
   const Forcing& f = ctx->frc;
-  a.nsrc = f.nsrc;
-  a.nghost = f.nghost;
   if (f.nsrc + f.nghost == 0) return;
   if (ta.ts) {
     // offsets within a replayed chunk count whole steps; the stage's own offset is in its row
@@ -1230,6 +1230,8 @@ int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double
   ctx->capturing = was;
   return rc;
 }
+
+FaceArgs face_member_args(const rdg_ctx* ctx) { return face_args(ctx, nullptr); }
 
 int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta) {
   return enqueue_face_stage(ctx, u, nullptr, rhs, 0, 0.0f, ta, nullptr, 0.0f, 0.0f, -1, true, false, 0);

@@ -37,16 +37,14 @@ struct rdg_batch {
   int g_chunk = 0;
   // persistent form: one launch per chunk of steps of every member
   int mode = RDG_BATCH_AUTO;
-  int ept[7] = {1, 1, 1, 1, 1, 1, 1};   // edges per thread of an edge tile, per order
   int tpi[7] = {1, 1, 1, 1, 1, 1, 1};   // tiles per work item, per order
   double wait_s = 1.0;                  // bound on every dependency wait of the kernel
   int hold_member = -1;                 // test hook: this member's phase hold_phase never starts
   int64_t hold_phase = -1;
   bool dirty = true;                    // descriptors to rebuild before the next launch
   rdg::BMember* d_members = nullptr;
-  unsigned long long* d_ticket = nullptr;   // ticket, then one count per member
+  unsigned long long* d_ticket = nullptr;   // tickets and claims per list, counts per member, a cache line each
   int* d_flags = nullptr;               // abort flag, error word
-  float* d_tabs = nullptr;
   int nm_alloc = 0;
   rdg::BatchArgs args{};
   int grid = 0;
@@ -85,11 +83,12 @@ void release_member(rdg_batch::Member& m) {
   if (m.branch) cudaStreamDestroy(m.branch);
 }
 
-// The persistent form applies when every member is FP32 with stored operators and SSP-RK3.
+// The persistent form applies when every member is FP32 with an element-wise D (the face form) and
+// SSP-RK3.
 bool persistent_fits(const rdg_batch* b) {
   for (const auto& m : b->members) {
     const rdg_ctx* c = m.ctx;
-    if (c->esz != 4 || c->gemm || c->integrator != RDG_INTEGRATOR_SSP_RK3 || c->d_Dn) return false;
+    if (!c->face || c->integrator != RDG_INTEGRATOR_SSP_RK3) return false;
   }
   return !b->members.empty();
 }
@@ -103,11 +102,9 @@ void free_persistent(rdg_batch* b) {
   cudaFree(b->d_members);
   cudaFree(b->d_ticket);
   cudaFree(b->d_flags);
-  cudaFree(b->d_tabs);
   b->d_members = nullptr;
   b->d_ticket = nullptr;
   b->d_flags = nullptr;
-  b->d_tabs = nullptr;
   b->nm_alloc = 0;
   b->dirty = true;
 }
@@ -118,85 +115,83 @@ int prepare_persistent(rdg_batch* b) {
   free_persistent(b);
   const int nm = (int)b->members.size();
   std::vector<rdg::BMember> hm(nm);
-  bool orders[7] = {false, false, false, false, false, false, false};
-  int64_t off = 0, offb = 0;
-  for (int i = 0; i < nm; ++i) {
-    rdg_ctx* c = b->members[i].ctx;
-    int rc = rdg::ensure_edge_form(c);
-    if (rc != RDG_OK) return bfail(b, rc, std::string("member: ") + rdg_last_error(c));
-    rdg::BMember& d = hm[i];
-    d.W = c->d_W;
-    d.k1 = c->d_k1;
-    d.k2 = c->d_k2;
-    d.f12 = c->d_f12;
+  // by order: each order's members are one list of items
+  std::vector<int> by(nm);
+  for (int i = 0; i < nm; ++i) by[i] = i;
+  std::stable_sort(by.begin(), by.end(), [&](int x, int y) { return b->members[x].ctx->N < b->members[y].ctx->N; });
+  rdg::BatchArgs& a = b->args;
+  a = rdg::BatchArgs{};
+  // instructions of one element's stage in thousands: by a thread, by a team's thread
+  static const double kCost[7] = {0, 0.3, 0.6, 1.2, 1.9, 3.0, 4.7}, kTeam[7] = {0, 0, 0, 0, 0.8, 1.1, 1.4};
+  double weight[6] = {}, total = 0;
+  int64_t items = 0;
+  for (int j = 0; j < nm; ++j) {
+    const int i = by[j];
+    const rdg_ctx* c = b->members[i].ctx;
+    if (a.nlist == 0 || hm[j - 1].N != c->N) {
+      a.list[a.nlist].m0 = j;
+      ++a.nlist;
+    }
+    rdg::BatchList& l = a.list[a.nlist - 1];
+    rdg::BMember& d = hm[j];
+    d.base = rdg::face_member_args(c);
     d.u = (float*)c->d_u;
     d.u1 = (float*)c->d_u1;
     d.u2 = (float*)c->d_u2;
-    d.vol = (float*)c->d_vol;
-    d.fb = (float*)c->d_fb;
-    d.geo = (const float*)c->d_geo;
-    d.S = (const float*)c->d_S;
-    d.G = (const float*)c->d_G;
-    d.err = c->d_err;
+    d.rec[0] = c->d_rec[0];
+    d.rec[1] = c->d_rec[1];
     d.ts = c->d_time;
-    d.K = c->K;
-    d.E = c->E;
-    d.B = c->B;
     d.frc = c->frc;
     d.dt = b->members[i].dt;
-    d.dt32 = (float)b->members[i].dt;
+    d.base.dt = (float)d.dt;
     d.N = c->N;
-    d.ept = b->ept[c->N];
-    d.ntile_v = (c->K + rdg::kStageBlock - 1) / rdg::kStageBlock;
-    const int64_t per_tile = (int64_t)rdg::kStageBlock * d.ept;
-    d.ntile_e = (c->E + per_tile - 1) / per_tile;
-    d.ntile_u = d.ntile_v;
-    d.tpi = b->tpi[c->N];
-    d.nitem_a = (d.ntile_e + d.ntile_v + d.tpi - 1) / d.tpi;
-    d.nitem_b = (d.ntile_u + d.tpi - 1) / d.tpi;
-    d.off_a = off;
-    d.off_b = offb;
-    d.hold_phase = i == b->hold_member ? b->hold_phase : -1;
-    off += d.nitem_a;
-    offb += d.nitem_b;
-    orders[c->N] = true;
+    d.alg1 = c->iface == RDG_IFACE_ALG1;
+    d.team = c->N >= 4 && (c->K + 31) / 32 <= rdg::batch_sms();
+    d.per_item = (d.team ? 32 : 128) * b->tpi[c->N];
+    d.nitem = (c->K + d.per_item - 1) / d.per_item;
+    d.off = l.per_phase;
+    d.hold_phase = i == b->hold_member && b->hold_phase >= 0 ? b->hold_phase + 1 : -1;
+    l.per_phase += d.nitem;
+    l.m1 = j + 1;
+    items += d.nitem;
+    const double w = (double)d.nitem * (d.team ? kTeam[c->N] : kCost[c->N]);
+    weight[a.nlist - 1] += w;
+    total += w;
   }
-  std::vector<float> tabs;
-  int toff[7];
-  int rc = rdg::batch_tables(orders, tabs, toff);
-  if (rc != RDG_OK) return bfail(b, rc, "reference tables");
+  double upto = 0;
+  for (int l = 0; l < a.nlist; ++l) {
+    upto += weight[l];
+    a.list[l].sm_end = std::max((int)(rdg::batch_sms() * upto / total + 0.5), l > 0 ? a.list[l - 1].sm_end + 1 : 1);
+  }
   cudaError_t e;
   if ((e = cudaMalloc(&b->d_members, nm * sizeof(rdg::BMember))) != cudaSuccess ||
-      (e = cudaMalloc(&b->d_ticket, (2 * nm + 1) * sizeof(unsigned long long))) != cudaSuccess ||
-      (e = cudaMalloc(&b->d_flags, 2 * sizeof(int))) != cudaSuccess ||
-      (e = cudaMalloc(&b->d_tabs, std::max<size_t>(tabs.size(), 4) * sizeof(float))) != cudaSuccess) {
+      (e = cudaMalloc(&b->d_ticket, (nm + 12) * rdg::kCountStride * sizeof(unsigned long long))) != cudaSuccess ||
+      (e = cudaMalloc(&b->d_flags, 2 * sizeof(int))) != cudaSuccess) {
     free_persistent(b);
     return bcuda(b, e, "persistent batch buffers");
   }
   if ((e = cudaMemcpy(b->d_members, hm.data(), nm * sizeof(rdg::BMember), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(b->d_tabs, tabs.data(), tabs.size() * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemset(b->d_flags, 0, 2 * sizeof(int))) != cudaSuccess) {
     free_persistent(b);
     return bcuda(b, e, "persistent batch upload");
   }
-  rdg::BatchArgs& a = b->args;
   a.m = b->d_members;
   a.nm = nm;
-  a.items_a = off;
-  a.per_phase = off + offb;
   a.ticket = b->d_ticket;
-  a.done = b->d_ticket + 1;
+  a.claim = b->d_ticket + 6 * rdg::kCountStride;
+  a.done = b->d_ticket + 12 * rdg::kCountStride;
   a.abort = b->d_flags;
   a.err = b->d_flags + 1;
-  a.tabs = b->d_tabs;
-  a.tab_floats = (int)tabs.size();
   a.wait_ns = (uint64_t)(b->wait_s * 1e9);
-  b->smem = rdg::batch_smem_bytes(a.tab_floats, nm);
+  b->smem = rdg::batch_smem_bytes(nm);
   b->grid = rdg::batch_grid(b->smem);
   if (b->grid <= 0) {
     free_persistent(b);
     return bfail(b, RDG_ECUDA, "persistent batch kernel occupancy");
   }
+  // blocks beyond one phase's items would only poll
+  b->grid = (int)std::min<int64_t>(b->grid, std::max<int64_t>(1, items));
+  for (int l = 0; l < a.nlist; ++l) a.list[l].blocks = (int)((a.list[l].per_phase * b->grid + items - 1) / items);
   b->nm_alloc = nm;
   b->dirty = false;
   return RDG_OK;
@@ -204,11 +199,11 @@ int prepare_persistent(rdg_batch* b) {
 
 // nsteps steps of every member in one persistent launch on `root`, then the time origins.
 int enqueue_persistent(rdg_batch* b, cudaStream_t root, int nsteps) {
-  cudaError_t e = cudaMemsetAsync(b->d_ticket, 0, (2 * b->nm_alloc + 1) * sizeof(unsigned long long), root);
+  cudaError_t e = cudaMemsetAsync(b->d_ticket, 0, (b->nm_alloc + 12) * rdg::kCountStride * sizeof(unsigned long long), root);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_flags, 0, sizeof(int), root);   // abort flag only
   if (e != cudaSuccess) return bcuda(b, e, "cudaMemsetAsync");
   rdg::BatchArgs a = b->args;
-  a.nphase = 3 * nsteps;
+  a.nphase = 1 + 3 * nsteps;
   int rc = rdg::launch_batch_persistent(a, b->grid, b->smem, root);
   if (rc == RDG_OK) rc = rdg::launch_batch_advance(b->d_members, b->nm_alloc, nsteps, root);
   return rc == RDG_OK ? RDG_OK : bfail(b, rc, "kernel launch failed");
@@ -323,11 +318,6 @@ int rdg_batch_add(rdg_batch* b, rdg_ctx* ctx, double t0, double dt) {
   for (auto& m : b->members)
     if (m.ctx == ctx) return bfail(b, RDG_EINVAL, "context is already in the batch");
   DevGuard g(b->device);
-  // the persistent launch streams per-edge operators: built here, not in the first step
-  if (b->mode != RDG_BATCH_GRAPH && ctx->face && ctx->integrator == RDG_INTEGRATOR_SSP_RK3) {
-    int rc = rdg::ensure_edge_form(ctx);
-    if (rc != RDG_OK) return bfail(b, rc, std::string("member: ") + rdg_last_error(ctx));
-  }
   rdg_batch::Member m{ctx, dt, nullptr, nullptr, nullptr};
   bool ok = cudaEventCreateWithFlags(&m.ev_in, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&m.ev_join, cudaEventDisableTiming) == cudaSuccess &&
@@ -446,7 +436,7 @@ int rdg_batch_set_mode(rdg_batch* b, int mode) {
   if (mode != RDG_BATCH_AUTO && mode != RDG_BATCH_GRAPH && mode != RDG_BATCH_PERSISTENT)
     return bfail(b, RDG_EINVAL, "mode must be RDG_BATCH_AUTO, RDG_BATCH_GRAPH or RDG_BATCH_PERSISTENT");
   if (mode == RDG_BATCH_PERSISTENT && !b->members.empty() && !persistent_fits(b))
-    return bfail(b, RDG_EINVAL, "the persistent form needs FP32 members with stored operators and SSP-RK3");
+    return bfail(b, RDG_EINVAL, "the persistent form needs FP32 members with an element-wise D and SSP-RK3");
   DevGuard g(b->device);
   cudaStreamSynchronize(b->stream);
   b->mode = mode;
@@ -467,8 +457,7 @@ int rdg_batch_set_tiles(rdg_batch* b, int N, int edges_per_thread, int tiles_per
     return bfail(b, RDG_EINVAL, "N must be in 1..6, edges_per_thread 1 or 2, tiles_per_item 1, 2 or 4");
   DevGuard g(b->device);
   cudaStreamSynchronize(b->stream);
-  b->ept[N] = edges_per_thread;
-  b->tpi[N] = tiles_per_item;
+  b->tpi[N] = edges_per_thread * tiles_per_item;
   b->dirty = true;
   drop_graph(b);
   return RDG_OK;

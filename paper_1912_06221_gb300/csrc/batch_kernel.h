@@ -4,67 +4,55 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <vector>
-
 #include "internal.h"
 
 namespace rdg {
 
-// One member problem as the persistent kernel sees it (FP32, stored operators, SSP-RK3).
-// A stage of a member is two parts of work items: part A, its edge tiles (fluxes into the
-// face slots) and element tiles (volume terms); part B, its element tiles again (surface
-// terms and the stage update).
+// One member problem as the persistent kernel sees it (face form, SSP-RK3).  Its work of one phase is
+// a row of items, each `per_item` elements: in phase 0 the face records of its state, in phase p >= 1
+// stage p - 1 of the launch.
 struct BMember {
-  const void* W;             // tiled per-edge operators
-  const int32_t* k1;
-  const int32_t* k2;
-  const int32_t* f12;
+  FaceArgs base;             // everything a stage takes that does not change from stage to stage
   float *u, *u1, *u2;        // state and the two stage buffers
-  float *vol, *fb;           // volume terms, face slots
-  const float* geo;
-  const float* S;            // sources [nsrc][K][Np]
-  const float* G;            // Dirichlet ghost data [nghost][B][Np]
-  int* err;                  // the member's device error word
+  float* rec[2];             // the two record buffers
   TimeState* ts;             // time origin and steps done before this launch
-  int64_t K, E, B;
   Forcing frc;
   double dt;
-  float dt32;
   int N;
-  int ept;                   // edges per thread in an edge tile (1 or 2)
-  int tpi;                   // tiles per work item (1, 2 or 4)
-  int64_t ntile_e, ntile_v;  // part A: edge and element tiles per stage
-  int64_t ntile_u;           // part B: element tiles per stage
-  int64_t nitem_a, nitem_b;  // work items of part A / part B per stage (tiles / tpi, rounded up)
-  int64_t off_a, off_b;      // first item of this member within part A / part B of a stage
-  int64_t hold_phase;        // a stage whose part A is never released (test hook), or -1
+  bool alg1, team;           // team: items of 32-element tiles, four warps to a tile
+  int64_t per_item, nitem;   // elements per item, items per phase
+  int64_t off;               // first item of this member within a phase of its list
+  int64_t hold_phase;        // a phase that is never released (test hook), or -1
+};
+
+// The members of one order: a list of items of its own.  Blocks prefer the list of their SM, until as
+// many as the list wants have come.
+struct BatchList {
+  int m0, m1;                // members [m0, m1) of the descriptor array
+  int sm_end;                // SMs up to here (exclusive, from the previous list's end) prefer this list
+  int blocks;                // blocks wanted
+  int64_t per_phase;         // items of one phase, all members of the list
 };
 
 struct BatchArgs {
-  const BMember* m;          // device array [nm], ascending off_a and off_b
-  int nm;
-  int64_t items_a;           // part-A items of all members in one stage
-  int64_t per_phase;         // items of one stage: every member's part A, then every part B
-  int nphase;                // stages of this launch (3 x steps)
-  unsigned long long* ticket;
-  unsigned long long* done;  // [2 nm]: part-A items finished per member, then part-B items
+  const BMember* m;          // device array [nm], by ascending order and, within it, ascending off
+  int nm, nlist;
+  BatchList list[6];
+  int nphase;                // 1 + stages of this launch (3 x steps)
+  unsigned long long* ticket;  // per list, kCountStride apart (a cache line each)
+  unsigned long long* claim;   // blocks that came to each list, likewise
+  unsigned long long* done;    // items finished per member, likewise
   int* abort;
   int* err;                  // the batch's device error word
-  const float* tabs;         // order 6's volume tables for shared memory (batch_tables), if present
-  int tab_floats;
   uint64_t wait_ns;          // bound on every dependency wait
 };
 
-// Uploads every order's reference matrices to the kernel's constant banks (once per device)
-// and returns the shared-memory tables the kernel stages (order 6's volume matrices, when
-// orders[6]); off is unused (all zero).
-int batch_tables(const bool orders[7], std::vector<float>& tabs, int off[7]);
-// Dynamic shared memory of the kernel: the tables, a volume tile's rows, and the member
-// descriptors when there are at most kSmemMembers of them.
-constexpr int kSmemMembers = 64;
-size_t batch_smem_bytes(int tab_floats, int nm);
-int batch_grid(size_t smem);   // resident blocks of the persistent kernel (-1 on error)
+constexpr int kCountStride = 16;
+constexpr int kSmemMembers = 64;   // descriptors kept in shared memory up to this many
+size_t batch_smem_bytes(int nm);
+int batch_grid(size_t smem);       // resident blocks of the persistent kernel (-1 on error)
 int launch_batch_persistent(const BatchArgs& a, int grid, size_t smem, cudaStream_t s);
 int launch_batch_advance(BMember* m, int nm, long long steps, cudaStream_t s);
+int batch_sms();                   // SMs of the current device
 
 }  // namespace rdg

@@ -81,14 +81,16 @@ struct rdg_ctx {
 };
 
 namespace rdg {
-// Whether stages run in the face form, and building what the per-edge forms need beside it (the
-// persistent batch launch, an explicitly set stage form).
+// Whether stages run in the face form, and building what the per-edge forms need beside it (an
+// explicitly set stage form).
 bool use_face(const rdg_ctx* ctx);
 int ensure_edge_form(rdg_ctx* ctx);
 // One step of ctx's resident state with every launch on stream s (which may be capturing); used by
 // the batch, whose member steps run on per-member branch streams.  fresh: the face records of the
 // state are formed first; keep: the last stage leaves the records of its result.
 int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double dt, bool fresh, bool keep);
+// What every stage of ctx's face form takes, without the stage's own buffers, mode and forcing factors.
+FaceArgs face_member_args(const rdg_ctx* ctx);
 // Right-hand side of u in the face form (two launches, no allocation).
 int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta);
 // Row gather (dst[i] = src[idx[i]]) or scatter (dst[idx[i]] = src[i]) of np-value rows of

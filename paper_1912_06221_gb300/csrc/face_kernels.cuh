@@ -50,8 +50,16 @@ __host__ __device__ constexpr int team_blocks() {
   return N == 4 ? 6 : (N == 5 ? 5 : 4);
 }
 
+// Load of stage data.  LIVE: written by other blocks of the same launch (the persistent batch kernel),
+// so it is read through L2; otherwise by an earlier kernel.
+template <bool LIVE, typename V>
+__device__ __forceinline__ V ld_stage(const V* p) {
+  if constexpr (LIVE) return __ldcg(p);
+  else return *p;
+}
+
 // Rows of a warp's elements (n values from a 16-byte aligned start) into its shared slice.
-template <int NP>
+template <int NP, bool LIVE = false>
 __device__ __forceinline__ void rows_in(float* sh, const float* g, int n, int lane) {
   const int nv = n / 4;
 #pragma unroll
@@ -63,7 +71,7 @@ __device__ __forceinline__ void rows_in(float* sh, const float* g, int n, int la
                    : "memory");
   }
   const int i = nv * 4 + lane;
-  if (i < n) sh[i] = g[i];
+  if (i < n) sh[i] = ld_stage<LIVE>(g + i);
 }
 template <int NP>
 __device__ __forceinline__ void rows_out(float* g, const float* sh, int n, int lane) {
@@ -133,22 +141,22 @@ __device__ __forceinline__ bool jump_in_warp(unsigned nbr) {
 }
 
 // Record r of a buffer of 3 K records: planes of 4, 2 and 1 floats.
-template <int NG>
+template <int NG, bool LIVE>
 __device__ __forceinline__ void record_get(const float* buf, size_t K3, unsigned r, float (&v)[NG]) {
   constexpr int N4 = NG / 4 * 4, N2 = N4 + (NG - N4) / 2 * 2;
   if constexpr (NG >= 4) {
-    const float4 t = reinterpret_cast<const float4*>(buf)[r];
+    const float4 t = ld_stage<LIVE>(reinterpret_cast<const float4*>(buf) + r);
     v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
   }
   if constexpr (N2 > N4) {
-    const float2 t = reinterpret_cast<const float2*>(buf + N4 * K3)[r];
+    const float2 t = ld_stage<LIVE>(reinterpret_cast<const float2*>(buf + N4 * K3) + r);
     v[N4] = t.x, v[N4 + 1] = t.y;
   }
-  if constexpr (NG > N2) v[N2] = (buf + N2 * K3)[r];
+  if constexpr (NG > N2) v[N2] = ld_stage<LIVE>(buf + N2 * K3 + r);
 }
 // The neighbour's record (word r of the neighbour table) and its reference value; of a boundary edge,
 // whose data ghost_get supplies, or a corrupt table, any valid one.
-template <int NG>
+template <int NG, bool LIVE>
 __device__ __forceinline__ void neighbour_get(const FaceArgs& a, unsigned r, unsigned k, float (&v)[NG + 1]) {
   const unsigned K = (unsigned)a.K, K3 = 3u * K;
   if (r >= K3) {
@@ -156,12 +164,12 @@ __device__ __forceinline__ void neighbour_get(const FaceArgs& a, unsigned r, uns
     r = k;
   }
   float g[NG];
-  record_get<NG>(a.fin, K3, r, g);
+  record_get<NG, LIVE>(a.fin, K3, r, g);
 #pragma unroll
   for (int c = 0; c < NG; ++c) v[c] = g[c];
   r -= r >= K ? K : 0u;
   r -= r >= K ? K : 0u;
-  v[NG] = (a.fin + (size_t)NG * K3)[r];
+  v[NG] = ld_stage<LIVE>(a.fin + (size_t)NG * K3 + r);
 }
 __device__ __forceinline__ float stage_tau(const FaceArgs& a, int m) { return a.tau_row ? a.tau_row[m] : a.tau[m]; }
 // Dirichlet: the ghost data's parts at the stage time.
@@ -221,15 +229,11 @@ __device__ __forceinline__ void store_parts(const FaceArgs& a, const float (&v)[
   if (active) (a.fout + NG * K3)[k] = v[0];
 }
 
-// Parts of the stage input's elements [k_begin, k_end) (k_begin a multiple of 4: 16-byte rows).
-template <int N, bool ALG1>
-__global__ void __launch_bounds__(kFaceBlock, face_build<N, false>().blocks) face_parts_kernel(const __grid_constant__ FaceArgs a) {
+// Parts of the nk (>= 1) stage input elements from k0 on, by one warp; sh: 32 rows.
+template <int N, bool ALG1, bool ROLL, bool LIVE>
+__device__ __forceinline__ void parts_tile(const FaceArgs& a, int64_t k0, int nk, float* sh) {
   constexpr int NP = np_of(N);
-  __shared__ __align__(16) float shs[kFaceWarps][32 * NP];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t k0 = a.k_begin + ((int64_t)blockIdx.x * kFaceWarps + warp) * 32;
-  const int nk = (int)min((int64_t)32, a.k_end - k0);
-  if (nk <= 0) return;
+  const int lane = threadIdx.x & 31;
   const bool active = lane < nk;
   const int row = active ? lane : nk - 1;
   const unsigned k = (unsigned)(k0 + row);
@@ -240,14 +244,27 @@ __global__ void __launch_bounds__(kFaceBlock, face_build<N, false>().blocks) fac
     diff[f] = jump_in_warp<ALG1>(__ldg(a.nbr + (size_t)f * a.K + k));
     par[f] = face_par(a, f, k, diff[f]);
   }
-  wait_for_predecessor();
-  allow_dependents();
-  rows_in<NP>(shs[warp], a.us + k0 * NP, nk * NP, lane);
+  if constexpr (!LIVE) {
+    wait_for_predecessor();
+    allow_dependents();
+  }
+  rows_in<NP, LIVE>(sh, a.us + k0 * NP, nk * NP, lane);
   rows_commit();
   rows_wait<0>();
   float v[NP];
-  row_get<NP>(shs[warp] + row * NP, v);
-  store_parts<N, ALG1, face_build<N, false>().roll>(a, v, par, diff, k, active);
+  row_get<NP>(sh + row * NP, v);
+  store_parts<N, ALG1, ROLL>(a, v, par, diff, k, active);
+}
+
+// Parts of the stage input's elements [k_begin, k_end) (k_begin a multiple of 4: 16-byte rows).
+template <int N, bool ALG1>
+__global__ void __launch_bounds__(kFaceBlock, face_build<N, false>().blocks)
+    face_parts_kernel(const __grid_constant__ FaceArgs a) {
+  __shared__ __align__(16) float sh[kFaceWarps][32 * np_of(N)];
+  const int warp = threadIdx.x >> 5;
+  const int64_t k0 = a.k_begin + ((int64_t)blockIdx.x * kFaceWarps + warp) * 32;
+  const int nk = (int)min((int64_t)32, a.k_end - k0);
+  if (nk > 0) parts_tile<N, ALG1, face_build<N, false>().roll, false>(a, k0, nk, sh[warp]);
 }
 
 // Parts of the Dirichlet ghosts' data, one thread per forcing term and boundary edge: the flux is
@@ -270,175 +287,183 @@ __global__ void __launch_bounds__(128) face_ghost_kernel(const float* G, const f
   out[i * (NG + 1) + NG] = v0;
 }
 
-template <int N, bool ALG1, bool LARGE>
-__global__ void __launch_bounds__(kFaceBlock, face_build<N, LARGE>().blocks)
-    face_stage_kernel(const __grid_constant__ FaceArgs a) {
+// One stage of the nk (>= 1) elements from k0 on, by one warp; shs, shn: 32 rows each.  EARLY, ROLL: see
+// FaceBuild.
+template <int N, bool ALG1, int EARLY, bool ROLL, bool LIVE>
+__device__ __forceinline__ void stage_tile(const FaceArgs& a, int64_t k0, int nk, float* shs, float* shn) {
   using O = face::Ops<N>;
-  constexpr FaceBuild build = face_build<N, LARGE>();
-  constexpr bool RECS = build.early & 1, PARS = build.early & 2;
+  constexpr bool RECS = EARLY & 1, PARS = EARLY & 2;
   constexpr int NP = np_of(N), NG = N + 1;
   static_assert(NG == O::GE + O::GO, "record size");
-  __shared__ __align__(16) float shs_all[kFaceWarps][32 * NP];
-  __shared__ __align__(16) float shn_all[kFaceWarps][32 * NP];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float *shs = shs_all[warp], *shn = shn_all[warp];
-  for (int64_t tile = (int64_t)blockIdx.x * kFaceWarps + warp; tile * 32 < a.K; tile += (int64_t)gridDim.x * kFaceWarps) {
-    const int64_t k0 = tile * 32;
-    const int nk = (int)min((int64_t)32, a.K - k0);
-    const bool active = lane < nk;
-    const int row = active ? lane : nk - 1;
-    const unsigned k = (unsigned)(k0 + row), K3 = 3u * (unsigned)a.K;
-    // neighbours, coefficients and parameters are written by no stage: loaded before the dependency wait
-    unsigned nbr[3];
+  const int lane = threadIdx.x & 31;
+  const bool active = lane < nk;
+  const int row = active ? lane : nk - 1;
+  const unsigned k = (unsigned)(k0 + row), K3 = 3u * (unsigned)a.K;
+  // neighbours, coefficients and parameters are written by no stage: loaded before the dependency wait
+  unsigned nbr[3];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) nbr[f] = __ldg(a.nbr + (size_t)f * a.K + k);
-    float geo[6];
+  for (int f = 0; f < 3; ++f) nbr[f] = __ldg(a.nbr + (size_t)f * a.K + k);
+  float geo[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) geo[c] = __ldg(a.geo + (size_t)c * a.K + k);
-    bool diff[3];
+  for (int c = 0; c < 6; ++c) geo[c] = __ldg(a.geo + (size_t)c * a.K + k);
+  bool diff[3];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      diff[f] = jump_in_warp<ALG1>(nbr[f]);
-      nbr[f] &= ~kFaceJump;
+  for (int f = 0; f < 3; ++f) {
+    diff[f] = jump_in_warp<ALG1>(nbr[f]);
+    nbr[f] &= ~kFaceJump;
+  }
+  face::Par<float> par[3] = {};
+  if constexpr (PARS) {
+#pragma unroll
+    for (int f = 0; f < 3; ++f) par[f] = face_par(a, f, k, diff[f]);
+  }
+  const bool need_un = a.mode == 2 || a.mode == 3 || (a.mode == 4 && a.rka != 0.f);
+  if constexpr (!LIVE) {
+    wait_for_predecessor();
+    allow_dependents();
+  }
+  rows_in<NP, LIVE>(shs, a.us + k0 * NP, nk * NP, lane);
+  rows_commit();
+  if (need_un) rows_in<NP, LIVE>(shn, a.un + k0 * NP, nk * NP, lane);
+  rows_commit();
+  float own[RECS ? 3 : 1][NG], nb[RECS ? 3 : 1][NG + 1];
+  auto records = [&](int f, float (&og)[NG], float (&ng)[NG + 1]) {
+    record_get<NG, LIVE>(a.fin, K3, (unsigned)f * (unsigned)a.K + k, og);
+    neighbour_get<NG, LIVE>(a, nbr[f], k, ng);
+  };
+  if constexpr (RECS) {
+#pragma unroll
+    for (int f = 0; f < 3; ++f) records(f, own[f], nb[f]);
+  }
+  rows_wait<1>();
+  float rhs[NP], u0;
+  {
+    float ve[O::NE], vo[O::NO];
+    {
+      float d[NP];
+      row_get<NP>(shs + row * NP, d);
+      u0 = d[0];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) d[j] -= u0;
+      face::volume_parts<float, N>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
     }
-    face::Par<float> par[3];
-    if constexpr (PARS) {
+    auto flux = [&](int f, float (&ge)[O::GE], float (&go)[O::GO]) {
+      float (&og)[NG] = own[RECS ? f : 0], (&ng)[NG + 1] = nb[RECS ? f : 0];
+      if constexpr (!RECS) records(f, og, ng);
+      const face::Par<float> p = PARS ? par[f] : face_par(a, f, k, diff[f]);
+      if (nbr[f] >= K3) ghost_get<NG>(a, nbr[f] - K3, ng);
+#pragma unroll
+      for (int q = 0; q < O::GE; ++q) ge[q] = og[q];
+#pragma unroll
+      for (int q = 0; q < O::GO; ++q) go[q] = og[O::GE + q];
+      face::face_flux<float, N, ALG1>(p, diff[f], u0, ng[NG], ng, ge, go);
+      const float mj = -geo[5];
+#pragma unroll
+      for (int q = 0; q < O::GE; ++q) ge[q] *= mj;
+#pragma unroll
+      for (int q = 0; q < O::GO; ++q) go[q] *= mj;
+    };
+    float ge[O::GE], go[O::GO];
+    if constexpr (ROLL) {
+      O::nodes(ve, vo, rhs);
+#pragma unroll 1
+      for (int i = 0; i < 3; ++i) {
+        if (i == 0) flux(1, ge, go);
+        else if (i == 1) flux(2, ge, go);
+        else flux(0, ge, go);
+#pragma unroll
+        for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+#pragma unroll
+        for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+        O::lift_even(ge, ve);
+        O::lift_odd(go, vo);
+        O::join1(ve, vo, rhs);
+        O::rotate(rhs);
+      }
+    } else {
+    flux(1, ge, go);              // the second face's order is the element's own
+    O::lift_even(ge, ve);
+    O::lift_odd(go, vo);
+    O::nodes(ve, vo, rhs);
+#pragma unroll
+    for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+#pragma unroll
+    for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+    flux(0, ge, go);
+    O::lift_even(ge, ve);
+    O::lift_odd(go, vo);
+    O::join0(ve, vo, rhs);
+#pragma unroll
+    for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+#pragma unroll
+    for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+    flux(2, ge, go);
+    O::lift_even(ge, ve);
+    O::lift_odd(go, vo);
+    O::join2(ve, vo, rhs);
+    }
+  }
+  for (int m = 0; m < a.nsrc; ++m) {
+    float S[NP];
+    row_get<NP>(a.S + ((int64_t)m * a.K + k) * NP, S);
+    const float tm = stage_tau(a, m);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) rhs[i] = fmaf(tm, S[i], rhs[i]);
+  }
+  rows_wait<0>();
+  if (a.mode >= 1) {
+    float us[NP], un[NP];
+    row_get<NP>(shs + row * NP, us);
+    if (a.mode == 4) {
+      // low-storage stage: du' = rka du + dt L, u' = u + rkb du'
+      if (need_un) {
+        row_get<NP>(shn + row * NP, un);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) un[i] = fmaf(a.rka, un[i], a.dt * rhs[i]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) un[i] = a.dt * rhs[i];
+      }
+#pragma unroll
+      for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.rkb, un[i], us[i]);
+      __syncwarp();
+      if (active) row_put<NP>(shn + lane * NP, un);
+    } else {
+#pragma unroll
+      for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.dt, rhs[i], us[i]);
+      if (need_un) {
+        const float c = a.mode == 2 ? 0.25f : (float)(2.0 / 3.0);   // see rk_combine
+        row_get<NP>(shn + row * NP, un);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) rhs[i] = fmaf(c, rhs[i] - un[i], un[i]);
+      }
+    }
+  }
+  __syncwarp();
+  if (active) row_put<NP>(shs + lane * NP, rhs);
+  __syncwarp();
+  rows_out<NP>(a.out + k0 * NP, shs, nk * NP, lane);
+  if (a.mode == 4) rows_out<NP>(a.out2 + k0 * NP, shn, nk * NP, lane);
+  if (a.fout) {
+    if constexpr (!PARS) {
 #pragma unroll
       for (int f = 0; f < 3; ++f) par[f] = face_par(a, f, k, diff[f]);
     }
-    const bool need_un = a.mode == 2 || a.mode == 3 || (a.mode == 4 && a.rka != 0.f);
-    wait_for_predecessor();
-    allow_dependents();
-    rows_in<NP>(shs, a.us + k0 * NP, nk * NP, lane);
-    rows_commit();
-    if (need_un) rows_in<NP>(shn, a.un + k0 * NP, nk * NP, lane);
-    rows_commit();
-    float own[RECS ? 3 : 1][NG], nb[RECS ? 3 : 1][NG + 1];
-    auto records = [&](int f, float (&og)[NG], float (&ng)[NG + 1]) {
-      record_get<NG>(a.fin, K3, (unsigned)f * (unsigned)a.K + k, og);
-      neighbour_get<NG>(a, nbr[f], k, ng);
-    };
-    if constexpr (RECS) {
-#pragma unroll
-      for (int f = 0; f < 3; ++f) records(f, own[f], nb[f]);
-    }
-    rows_wait<1>();
-    float rhs[NP], u0;
-    {
-      float ve[O::NE], vo[O::NO];
-      {
-        float d[NP];
-        row_get<NP>(shs + row * NP, d);
-        u0 = d[0];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) d[j] -= u0;
-        face::volume_parts<float, N>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
-      }
-      auto flux = [&](int f, float (&ge)[O::GE], float (&go)[O::GO]) {
-        float (&og)[NG] = own[RECS ? f : 0], (&ng)[NG + 1] = nb[RECS ? f : 0];
-        if constexpr (!RECS) records(f, og, ng);
-        const face::Par<float> p = PARS ? par[f] : face_par(a, f, k, diff[f]);
-        if (nbr[f] >= K3) ghost_get<NG>(a, nbr[f] - K3, ng);
-#pragma unroll
-        for (int q = 0; q < O::GE; ++q) ge[q] = og[q];
-#pragma unroll
-        for (int q = 0; q < O::GO; ++q) go[q] = og[O::GE + q];
-        face::face_flux<float, N, ALG1>(p, diff[f], u0, ng[NG], ng, ge, go);
-        const float mj = -geo[5];
-#pragma unroll
-        for (int q = 0; q < O::GE; ++q) ge[q] *= mj;
-#pragma unroll
-        for (int q = 0; q < O::GO; ++q) go[q] *= mj;
-      };
-      float ge[O::GE], go[O::GO];
-      if constexpr (build.roll) {
-        O::nodes(ve, vo, rhs);
-#pragma unroll 1
-        for (int i = 0; i < 3; ++i) {
-          if (i == 0) flux(1, ge, go);
-          else if (i == 1) flux(2, ge, go);
-          else flux(0, ge, go);
-#pragma unroll
-          for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
-#pragma unroll
-          for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
-          O::lift_even(ge, ve);
-          O::lift_odd(go, vo);
-          O::join1(ve, vo, rhs);
-          O::rotate(rhs);
-        }
-      } else {
-      flux(1, ge, go);              // the second face's order is the element's own
-      O::lift_even(ge, ve);
-      O::lift_odd(go, vo);
-      O::nodes(ve, vo, rhs);
-#pragma unroll
-      for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
-#pragma unroll
-      for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
-      flux(0, ge, go);
-      O::lift_even(ge, ve);
-      O::lift_odd(go, vo);
-      O::join0(ve, vo, rhs);
-#pragma unroll
-      for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
-#pragma unroll
-      for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
-      flux(2, ge, go);
-      O::lift_even(ge, ve);
-      O::lift_odd(go, vo);
-      O::join2(ve, vo, rhs);
-      }
-    }
-    for (int m = 0; m < a.nsrc; ++m) {
-      float S[NP];
-      row_get<NP>(a.S + ((int64_t)m * a.K + k) * NP, S);
-      const float tm = stage_tau(a, m);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) rhs[i] = fmaf(tm, S[i], rhs[i]);
-    }
-    rows_wait<0>();
-    if (a.mode >= 1) {
-      float us[NP], un[NP];
-      row_get<NP>(shs + row * NP, us);
-      if (a.mode == 4) {
-        // low-storage stage: du' = rka du + dt L, u' = u + rkb du'
-        if (need_un) {
-          row_get<NP>(shn + row * NP, un);
-#pragma unroll
-          for (int i = 0; i < NP; ++i) un[i] = fmaf(a.rka, un[i], a.dt * rhs[i]);
-        } else {
-#pragma unroll
-          for (int i = 0; i < NP; ++i) un[i] = a.dt * rhs[i];
-        }
-#pragma unroll
-        for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.rkb, un[i], us[i]);
-        __syncwarp();
-        if (active) row_put<NP>(shn + lane * NP, un);
-      } else {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) rhs[i] = fmaf(a.dt, rhs[i], us[i]);
-        if (need_un) {
-          const float c = a.mode == 2 ? 0.25f : (float)(2.0 / 3.0);   // see rk_combine
-          row_get<NP>(shn + row * NP, un);
-#pragma unroll
-          for (int i = 0; i < NP; ++i) rhs[i] = fmaf(c, rhs[i] - un[i], un[i]);
-        }
-      }
-    }
-    __syncwarp();
-    if (active) row_put<NP>(shs + lane * NP, rhs);
-    __syncwarp();
-    rows_out<NP>(a.out + k0 * NP, shs, nk * NP, lane);
-    if (a.mode == 4) rows_out<NP>(a.out2 + k0 * NP, shn, nk * NP, lane);
-    if (a.fout) {
-      if constexpr (!PARS) {
-#pragma unroll
-        for (int f = 0; f < 3; ++f) par[f] = face_par(a, f, k, diff[f]);
-      }
-      store_parts<N, ALG1, build.roll>(a, rhs, par, diff, k, active);
-    }
-    __syncwarp();
+    store_parts<N, ALG1, ROLL>(a, rhs, par, diff, k, active);
+  }
+}
+
+template <int N, bool ALG1, bool LARGE>
+__global__ void __launch_bounds__(kFaceBlock, face_build<N, LARGE>().blocks)
+    face_stage_kernel(const __grid_constant__ FaceArgs a) {
+  constexpr FaceBuild build = face_build<N, LARGE>();
+  __shared__ __align__(16) float shs[kFaceWarps][32 * np_of(N)];
+  __shared__ __align__(16) float shn[kFaceWarps][32 * np_of(N)];
+  const int warp = threadIdx.x >> 5;
+  for (int64_t tile = (int64_t)blockIdx.x * kFaceWarps + warp; tile * 32 < a.K; tile += (int64_t)gridDim.x * kFaceWarps) {
+    stage_tile<N, ALG1, build.early, build.roll, false>(a, tile * 32, (int)min((int64_t)32, a.K - tile * 32), shs[warp],
+                                                       shn[warp]);
+    __syncwarp();   // the rows before the next tile's
   }
 }
 
@@ -447,15 +472,12 @@ __global__ void __launch_bounds__(kFaceBlock, face_build<N, LARGE>().blocks)
 // face_stage_kernel walks the whole chain alone (N = 4: 1900 instructions, about 1.8 us for a lone
 // warp), which sets the stage time where there are few warps per scheduler; here the chain is about a
 // third as long.
-template <int N, bool ALG1>
-__global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const __grid_constant__ FaceArgs a) {
+template <int N, bool ALG1, bool LIVE>
+__device__ __forceinline__ void team_tile(const FaceArgs& a, int64_t k0, int nk, float* su, float (*sp)[32 * np_of(N)]) {
   using O = face::Ops<N>;
   constexpr int NP = np_of(N), NG = N + 1, V4 = (NP * 8 + 127) / 128;
-  __shared__ __align__(16) float su[32 * NP];
-  __shared__ __align__(16) float sp[4][32 * NP];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t k0 = (int64_t)blockIdx.x * 32;
-  const int nk = (int)min((int64_t)32, a.K - k0), n = nk * NP, nv = n / 4;
+  const int n = nk * NP, nv = n / 4;
   const bool active = lane < nk;
   const int row = active ? lane : nk - 1;
   const unsigned k = (unsigned)(k0 + row), K = (unsigned)a.K, K3 = 3u * K;
@@ -473,8 +495,10 @@ __global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const 
 #pragma unroll
   for (int c = 0; c < 6; ++c) geo[c] = __ldg(a.geo + (size_t)c * K + k);
   const bool need_un = a.mode == 2 || a.mode == 3 || (a.mode == 4 && a.rka != 0.f);
-  wait_for_predecessor();
-  allow_dependents();
+  if constexpr (!LIVE) {
+    wait_for_predecessor();
+    allow_dependents();
+  }
   const float4* us4 = reinterpret_cast<const float4*>(a.us + k0 * NP);
   float4 un4[V4];
 #pragma unroll
@@ -484,14 +508,15 @@ __global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const 
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(su + 4 * i)),
                    "l"(us4 + i)
                    : "memory");
-    un4[j] = need_un && i < nv ? reinterpret_cast<const float4*>(a.un + k0 * NP)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    un4[j] = need_un && i < nv ? ld_stage<LIVE>(reinterpret_cast<const float4*>(a.un + k0 * NP) + i)
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  if (nv * 4 + tid < n) su[nv * 4 + tid] = a.us[k0 * NP + nv * 4 + tid];
+  if (nv * 4 + tid < n) su[nv * 4 + tid] = ld_stage<LIVE>(a.us + k0 * NP + nv * 4 + tid);
   rows_commit();
   float own[NG], nb[NG + 1];
   if (f >= 0) {
-    record_get<NG>(a.fin, K3, (unsigned)f * K + k, own);
-    neighbour_get<NG>(a, nbr, k, nb);
+    record_get<NG, LIVE>(a.fin, K3, (unsigned)f * K + k, own);
+    neighbour_get<NG, LIVE>(a, nbr, k, nb);
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
@@ -581,7 +606,7 @@ __global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const 
   if (nv * 4 + tid < n) {
     const int i = nv * 4 + tid;
     float du = 0.f;
-    const float v = update(i, need_un ? a.un[g0 + i] : 0.f, du);
+    const float v = update(i, need_un ? ld_stage<LIVE>(a.un + g0 + i) : 0.f, du);
     su[i] = v;
     a.out[g0 + i] = v;
     if (a.mode == 4) a.out2[g0 + i] = du;
@@ -601,6 +626,14 @@ __global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const 
   } else if (active) {
     (a.fout + (size_t)NG * K3)[k] = su[lane * NP];
   }
+}
+
+template <int N, bool ALG1>
+__global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const __grid_constant__ FaceArgs a) {
+  __shared__ __align__(16) float su[32 * np_of(N)];
+  __shared__ __align__(16) float sp[4][32 * np_of(N)];
+  const int64_t k0 = (int64_t)blockIdx.x * 32;
+  team_tile<N, ALG1, false>(a, k0, (int)min((int64_t)32, a.K - k0), su, sp);
 }
 
 }  // namespace dev
