@@ -25,7 +25,7 @@ for _n in range(1, 7):
     for _t, _tag in (("float", "f"), ("double", "d")):
         SOURCES.append(("rhs_order.cu", "rhs_%s%d" % (_tag, _n),
                         ["-DRDG_ORDER=%d" % _n, "-DRDG_REAL=%s" % _t, "-DRDG_TAG=%s" % _tag,
-                         "-DRDG_TAG_IS_F=%d" % (_tag == "f")]))
+                         "-DRDG_TAG_IS_F=%d" % (_tag == "f"), "-I", os.path.join(OUT, "gen")]))
     # the face form: its order's operators are written into the build folder first (gen_face.cpp)
     SOURCES.append(("face_order.cu", "face_%d" % _n, ["-DRDG_ORDER=%d" % _n, "-I", os.path.join(OUT, "gen")]))
 

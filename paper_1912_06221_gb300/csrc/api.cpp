@@ -943,11 +943,21 @@ bool one_kernel_stage(const rdg_ctx* ctx) {
   return form == RDG_STAGE_ONE_KERNEL;
 }
 
+// Whether a stage runs as the FP64 kernel with a lane per (element, node) (rows_kernel.cuh): the
+// smaller meshes by default, up to where its doubled pipe time costs more than its short chains save
+// (us per stage, rows / two kernels: order 1 at 16200 triangles 7.0 / 8.9, order 2 at 8192 9.7 / 12.1,
+// order 3 at 8192 20 / 21, order 4 at 4608 17.7 / 31.3 and at 8192 37 / 35, order 5 at 4608 43 / 51,
+// order 6 at 4608 70 / 78; 512 triangles of order 2: 5.5 / 11.2).
+bool rows_stage(const rdg_ctx* ctx, int mode) {
+  static const int64_t kRows[kMaxN + 1] = {0, 16384, 8192, 8192, 6144, 4608, 4608};
+  return ctx->esz == 8 && mode <= 3 && ctx->stage_form == RDG_STAGE_AUTO && ctx->K <= kRows[ctx->N];
+}
+
 // Whether a stage of this context can run in two parts around a halo exchange (the stage
 // kernel and element kernel form on a split mesh).
 bool splittable_stage(const rdg_ctx* ctx, int mode) {
   return ctx->n_owned < ctx->K && !ctx->gemm && !(ctx->esz == 4 && split_volume32(ctx->N)) &&
-         !(mode <= 3 && one_kernel_stage(ctx));
+         !(mode <= 3 && one_kernel_stage(ctx)) && !rows_stage(ctx, mode);
 }
 
 FaceArgs face_args(const rdg_ctx* ctx, const float* us) {
@@ -1082,7 +1092,8 @@ int enqueue_stage(rdg_ctx* ctx, const void* us, const void* un, void* out, int m
   if (prof)
     for (auto& e : ev) e = take_event(ctx);
   int rc;
-  if (mode <= 3 && one_kernel_stage(ctx)) {
+  const bool rows = rows_stage(ctx, mode);
+  if (rows || (mode <= 3 && one_kernel_stage(ctx))) {
     // one launch: the edge part of the timing is empty
     if (prof) {
       cudaEventRecord(ev[0], st);
@@ -1090,7 +1101,7 @@ int enqueue_stage(rdg_ctx* ctx, const void* us, const void* un, void* out, int m
       cudaEventRecord(ev[2], st);
     }
     if constexpr (sizeof(T) == 4) rc = launch_fused32(ctx->N, mode, ea, la, st);
-    else rc = launch_fused64(ctx->N, mode, ea, la, st);
+    else rc = rows ? launch_rows64(ctx->N, mode, ea, la, st) : launch_fused64(ctx->N, mode, ea, la, st);
     if (prof) {
       cudaEventRecord(ev[3], st);
       ctx->ev_pending[0].push_back({ev[0], ev[1]});

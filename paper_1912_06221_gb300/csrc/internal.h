@@ -13,7 +13,11 @@ namespace rdg {
 
 constexpr int kTile = 32;            // edges per W tile (one warp, one edge per lane)
 constexpr int kElemBlock = 128;      // elements per element-kernel block
-constexpr int kStageBlock = 128;     // threads per block of the stage (edge/volume) kernel
+constexpr int kStageBlock = 128;     // threads per block of the FP32 stage (edge/volume) kernel
+// ... and of the FP64 one: the multiprocessor's one FP64 pipe is what the blocks share, and their work
+// per thread differs (order 4: an element's volume term 490 FP64 instructions, an edge 146), so
+// single-warp blocks even out the SMs (order 4, 32768 triangles: 75 us per stage, 88 with 128 threads).
+constexpr int kStageBlock64 = 32;
 
 // Stored values of one edge's flux operator in its difference form: per row, side 1's
 // columns 1..Np-1 and side 2's Np columns (2 Np - 1 values), then the one value J_f (v.n1)
@@ -139,6 +143,8 @@ int launch_elem_lite64(int N, int mode, const ElemArgs<double>& a, cudaStream_t 
 // One-kernel stage (elem_fused_kernel): modes 0..3.
 int launch_fused32(int N, int mode, const EdgeArgs<float>& ea, const ElemArgs<float>& a, cudaStream_t s);
 int launch_fused64(int N, int mode, const EdgeArgs<double>& ea, const ElemArgs<double>& a, cudaStream_t s);
+// One-kernel FP64 stage with a lane per (element, node), for small meshes: modes 0..3.
+int launch_rows64(int N, int mode, const EdgeArgs<double>& ea, const ElemArgs<double>& a, cudaStream_t s);
 int upload_elem_tables(int device);
 // GEMM form of the edge flux (FP32 state, tcgen05 split 3xTF32), orders 1..kMaxGemmN: the
 // edge kernel reads per-edge parameter records (EdgeArgs::W) and also computes the volume

@@ -75,6 +75,14 @@ int launch_volume32(int N, const EdgeArgs<float>& a, cudaStream_t s) {
   return N == 6 ? launch_volume_f6(a, s) : RDG_EINVAL;
 }
 
+#define RDG_ROWS_DECL(n) \
+  int launch_rows_##n(int mode, const EdgeArgs<double>& ea, const ElemArgs<double>& a, cudaStream_t s);
+RDG_ROWS_DECL(1) RDG_ROWS_DECL(2) RDG_ROWS_DECL(3) RDG_ROWS_DECL(4) RDG_ROWS_DECL(5) RDG_ROWS_DECL(6)
+#define CALL_ROWS(tag, n) launch_rows_##n(mode, ea, a, s)
+int launch_rows64(int N, int mode, const EdgeArgs<double>& ea, const ElemArgs<double>& a, cudaStream_t s) {
+  RDG_SWITCH(d, CALL_ROWS)
+}
+
 #define RDG_FACE_DECL(n)                                                                               \
   int launch_face_parts_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                             \
   int launch_face_stage_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                             \

@@ -16,6 +16,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
+#include "face_ops.h"
 #include "internal.h"
 #include "kernel_common.cuh"
 
@@ -70,15 +72,25 @@ __device__ __forceinline__ double2 ld_keep(const double2* p, uint64_t pol) {
 // u - u_0 and vol are live: 2 Np values instead of 5 Np.
 //
 // NODAL: D given at the nodes (dn, the element's Np values; the coefficients g_rr, g_rs, g_ss
-// then hold the metric alone), F_r = a_r u - D_j (g_rr u_r + g_rs u_s) node by node.
+// then hold the metric alone), F_r = a_r u - D_j (g_rr u_r + g_rs u_s) node by node.  Without it the
+// products run on the mirror-even and mirror-odd halves (face_ops.h), half the multiply-adds: FP64,
+// whose pipe issues one warp instruction in 64 cycles, is bound by their number.
 template <typename T, int N, bool NODAL = false>
 __device__ __forceinline__ void volume_row(const T (&u)[np_of(N)], T ar, T as, T grr, T grs, T gss,
                                            T (&vol)[np_of(N)], const T* __restrict__ dn = nullptr) {
   constexpr int NP = np_of(N);
   constexpr int ODR = 0, ODS = NP * NP, OWR = 2 * NP * NP, OWS = 3 * NP * NP;
   T du[NP];
+  du[0] = T(0);
 #pragma unroll
   for (int j = 1; j < NP; ++j) du[j] = u[j] - u[0];
+  if constexpr (!NODAL) {
+    using O = face::Ops<N>;
+    T ve[O::NE], vo[O::NO];
+    face::volume_parts<T, N>(du, u[0], ar, as, grr, grs, gss, ve, vo);
+    O::nodes(ve, vo, vol);
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < NP; ++i) vol[i] = T(0);
 #pragma unroll
@@ -90,21 +102,45 @@ __device__ __forceinline__ void volume_row(const T (&u)[np_of(N)], T ar, T as, T
       us = fma((T)RDG_TAB[ODS + j * NP + k], du[k], us);
     }
     const T uj = j == 0 ? u[0] : du[j] + u[0];
-    T fr, fs;
-    if constexpr (NODAL) {
-      const T dj = __ldg(dn + j);
-      fr = ar * uj - dj * (grr * ur + grs * us);
-      fs = as * uj - dj * (grs * ur + gss * us);
-    } else {
-      fr = ar * uj - (grr * ur + grs * us);
-      fs = as * uj - (grs * ur + gss * us);
-    }
+    const T dj = NODAL ? __ldg(dn + j) : T(1);
+    const T fr = ar * uj - dj * (grr * ur + grs * us);
+    const T fs = as * uj - dj * (grs * ur + gss * us);
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       vol[i] = fma((T)RDG_TAB[OWR + i * NP + j], fr, vol[i]);
       vol[i] = fma((T)RDG_TAB[OWS + i * NP + j], fs, vol[i]);
     }
   }
+}
+
+// rhs -= (1/J) LIFT_F q for face F's fluxes q in the element's face order, on mirror halves.
+template <typename T, int N, int F>
+__device__ __forceinline__ void lift_face(const T* q, T ij, T* rhs) {
+  using O = face::Ops<N>;
+  T ge[O::GE], go[O::GO], ve[O::NE], vo[O::NO];
+  const T h = T(-0.5) * ij;
+#pragma unroll
+  for (int c = 0; c < O::GO; ++c) {
+    ge[c] = h * (q[c] + q[N - c]);
+    go[c] = h * (q[c] - q[N - c]);
+  }
+  if constexpr (O::GE > O::GO) ge[O::GE - 1] = -ij * q[N / 2];
+#pragma unroll
+  for (int i = 0; i < O::NE; ++i) ve[i] = T(0);
+#pragma unroll
+  for (int i = 0; i < O::NO; ++i) vo[i] = T(0);
+  O::lift_even(ge, ve);
+  O::lift_odd(go, vo);
+  if constexpr (F == 0) O::join0(ve, vo, rhs);
+  else if constexpr (F == 1) O::join1(ve, vo, rhs);
+  else O::join2(ve, vo, rhs);
+}
+// Calls f with the face numbers 0, 1, 2 as compile-time constants.
+template <typename F>
+__device__ __forceinline__ void for_faces(F&& f) {
+  f(std::integral_constant<int, 0>{});
+  f(std::integral_constant<int, 1>{});
+  f(std::integral_constant<int, 2>{});
 }
 
 // The same volume term for the largest order, with the four reference matrices staged in
@@ -177,16 +213,21 @@ __device__ __forceinline__ void stage_in(T* sh, const T* g, int n) {
 // Volume role of the stage kernel: element tile v (one thread per element, rows staged
 // through shared memory), vol = M^{-1} S^T . F written to a.vol.  Kept out of line so its
 // register demand does not set the edge role's.
+template <typename T>
+__host__ __device__ constexpr int stage_block() {
+  return sizeof(T) == 8 ? kStageBlock64 : kStageBlock;
+}
+
 template <typename T, int N, bool NODAL = false>
 __device__ __noinline__ void stage_volume_tile(const EdgeArgs<T>& a, int64_t v, T* sh) {
   constexpr int NP = np_of(N);
   constexpr bool SMEM_TAB = N >= 6 && sizeof(T) == 4;   // (FP64: 25 KB of tables, and FP64-bound anyway)
   __shared__ __align__(16) T tab[SMEM_TAB ? VolTab<T, N>::SIZE : 4];
   const int tid = threadIdx.x;
-  const int64_t k0 = v * kStageBlock;
-  const int nk = (int)min((int64_t)kStageBlock, (a.Kvol > 0 ? a.Kvol : a.K) - k0);
+  const int64_t k0 = v * stage_block<T>();
+  const int nk = (int)min((int64_t)stage_block<T>(), (a.Kvol > 0 ? a.Kvol : a.K) - k0);
   {
-    Staged<T, kStageBlock, NP> g;
+    Staged<T, stage_block<T>(), NP> g;
     g.load(a.u + k0 * NP, nk * NP);
     if constexpr (SMEM_TAB) {
       constexpr int NV = VolTab<T, N>::SIZE * (int)sizeof(T) / 16;
@@ -361,7 +402,7 @@ constexpr int kEdgeOnlyBlocks[7] = {0, 5, 5, 5, 5, 4, 3};
 template <typename T, int N, int KIND = 1>
 constexpr int stage_min_blocks() {
   if (KIND == 2 && sizeof(T) == 4) return kEdgeOnlyBlocks[N];
-  return sizeof(T) == 4 ? (N <= 4 ? 5 : 6) : (N <= 3 ? 4 : 3);
+  return sizeof(T) == 4 ? (N <= 4 ? 5 : 6) : (N <= 3 ? 4 : 3) * 128 / kStageBlock64;
 }
 
 // Operator stream kinds: 0 edge blocks only, fluxes to the per-edge buffer (allocation-free
@@ -369,18 +410,20 @@ constexpr int stage_min_blocks() {
 // slots); 2 edge blocks only, fluxes to the face slots (the volume term from its own
 // kernel).
 template <typename T, int N, int KIND>
-__global__ void __launch_bounds__(kStageBlock, stage_min_blocks<T, N, KIND>()) edge_flux_kernel(EdgeArgs<T> a) {
+__global__ void __launch_bounds__(stage_block<T>(), stage_min_blocks<T, N, KIND>()) edge_flux_kernel(EdgeArgs<T> a) {
   constexpr int NP = np_of(N);
   wait_for_predecessor();
   // the element kernel may start its independent loads on SMs that the last wave leaves idle
   if constexpr (KIND != 0) allow_dependents();
   int64_t eblk = blockIdx.x;
   if constexpr (KIND == 1) {
-    __shared__ __align__(16) T sh[kStageBlock * NP];
+    __shared__ __align__(16) T sh[stage_block<T>() * NP];
     const int64_t nb = gridDim.x;
-    const int64_t nv = ((a.Kvol > 0 ? a.Kvol : a.K) + kStageBlock - 1) / kStageBlock;
+    const int64_t nv = ((a.Kvol > 0 ? a.Kvol : a.K) + stage_block<T>() - 1) / stage_block<T>();
     const int64_t b = blockIdx.x;
-    const int64_t v0 = (b * nv) / nb, v1 = ((b + 1) * nv) / nb;
+    // FP64: the long volume blocks first, so the short edge blocks even out the SMs
+    const int64_t v0 = sizeof(T) == 8 ? b : (b * nv) / nb;
+    const int64_t v1 = sizeof(T) == 8 ? min(b + 1, nv) : ((b + 1) * nv) / nb;
     if (v1 > v0) {
       if (a.Dn) stage_volume_tile<T, N, true>(a, v0, sh);    // D given at the nodes
       else stage_volume_tile<T, N, false>(a, v0, sh);
@@ -388,7 +431,7 @@ __global__ void __launch_bounds__(kStageBlock, stage_min_blocks<T, N, KIND>()) e
     }
     eblk = b - v1;    // edge blocks so far = blocks so far minus volume blocks so far
   }
-  const int64_t e = eblk * kStageBlock + threadIdx.x;
+  const int64_t e = eblk * stage_block<T>() + threadIdx.x;
   if (e < a.E) stage_edge<T, N, KIND != 0>(a, e);
 }
 
@@ -406,7 +449,6 @@ constexpr int elem_min_blocks() {
 template <typename T, int N, int MODE, bool VOLIN>
 __global__ void __launch_bounds__(kElemBlock, elem_min_blocks<T, N, VOLIN>()) elem_kernel(ElemArgs<T> a) {
   constexpr int NP = np_of(N), NFP = nfp_of(N);
-  constexpr int OLIFT = 4 * NP * NP;
   __shared__ __align__(16) T sh[kElemBlock * NP];
   __shared__ __align__(16) T shv[VOLIN ? kElemBlock * NP : 4];
   __shared__ T tau_s[RDG_MAX_FORCING_TERMS];
@@ -437,8 +479,8 @@ __global__ void __launch_bounds__(kElemBlock, elem_min_blocks<T, N, VOLIN>()) el
                        rhs);
     }
     // surface terms: side 1 takes J_f F*.n1 in its face order, side 2 the negated reverse
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
+    for_faces([&](auto face_c) {
+      constexpr int f = decltype(face_c)::value;
       int er = a.eref[(int64_t)f * a.K + k];
       if (er < 0 || (er >> 1) >= a.E) {     // self-check: record and read edge 0 instead
         report(a.err, kErrBadIndex);
@@ -451,14 +493,8 @@ __global__ void __launch_bounds__(kElemBlock, elem_min_blocks<T, N, VOLIN>()) el
       for (int i = 0; i < NFP; ++i) q[i] = fl[i];
 #pragma unroll
       for (int i = 0; i < NFP; ++i) qv[i] = side2 ? -q[NFP - 1 - i] : q[i];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        T acc = T(0);
-#pragma unroll
-        for (int c = 0; c < NFP; ++c) acc = fma((T)RDG_TAB[OLIFT + i * 3 * NFP + f * NFP + c], qv[c], acc);
-        rhs[i] -= ij * acc;
-      }
-    }
+      lift_face<T, N, f>(qv, ij, rhs);
+    });
     for (int m = 0; m < a.frc.nsrc; ++m) {
       const T* S = a.S + ((int64_t)m * a.K + k) * NP;
 #pragma unroll
@@ -493,6 +529,7 @@ __global__ void __launch_bounds__(kElemBlock, elem_min_blocks<T, N, VOLIN>()) el
 // rows of the volume term, face fluxes, stage input and step start in one round trip.
 template <typename T, int N>
 __host__ __device__ constexpr int lite_block() {
+  if (sizeof(T) == 8) return kStageBlock64;   // as the stage kernel's
   return 128 * (3 * np_of(N) + 3 * nfp_of(N)) * (int)sizeof(T) <= 46 * 1024
              ? 128
              : (64 * (3 * np_of(N) + 3 * nfp_of(N)) * (int)sizeof(T) <= 46 * 1024 ? 64 : 32);
@@ -501,7 +538,6 @@ __host__ __device__ constexpr int lite_block() {
 template <typename T, int N, int MODE>
 __global__ void __launch_bounds__(lite_block<T, N>(), elem_min_blocks<T, N, true>()) elem_lite_kernel(ElemArgs<T> a) {
   constexpr int NP = np_of(N), NFP = nfp_of(N), NQ = 3 * NFP;
-  constexpr int OLIFT = 4 * NP * NP;
   constexpr int BLK = lite_block<T, N>();
   __shared__ __align__(16) T shv[BLK * NP];
   __shared__ __align__(16) T shq[BLK * NQ];
@@ -540,19 +576,13 @@ __global__ void __launch_bounds__(lite_block<T, N>(), elem_min_blocks<T, N, true
   T rhs[NP];
 #pragma unroll
   for (int i = 0; i < NP; ++i) rhs[i] = shv[tid * NP + i];
-#pragma unroll
-  for (int f = 0; f < 3; ++f) {
+  for_faces([&](auto face_c) {
+    constexpr int f = decltype(face_c)::value;
     T q[NFP];
 #pragma unroll
     for (int c = 0; c < NFP; ++c) q[c] = shq[tid * NQ + f * NFP + c];
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      T acc = T(0);
-#pragma unroll
-      for (int c = 0; c < NFP; ++c) acc = fma((T)RDG_TAB[OLIFT + i * 3 * NFP + f * NFP + c], q[c], acc);
-      rhs[i] -= ij * acc;
-    }
-  }
+    lift_face<T, N, f>(q, ij, rhs);
+  });
   if (active) {
     for (int m = 0; m < a.frc.nsrc; ++m) {
       const T* S = a.S + ((int64_t)m * a.K + k) * NP;
@@ -616,7 +646,6 @@ template <typename T, int N, int MODE>
 __global__ void __launch_bounds__(kElemBlock, (N == 1 ? 8 : 1)) elem_fused_kernel(EdgeArgs<T> ea, ElemArgs<T> a) {
   static_assert(MODE >= 0 && MODE <= 3, "SSP-RK3 stages and the right-hand side only");
   constexpr int NP = np_of(N), NFP = nfp_of(N);
-  constexpr int OLIFT = 4 * NP * NP;
   constexpr int BLK = kElemBlock;
   constexpr bool NEED_UN = MODE == 2 || MODE == 3;
   __shared__ __align__(16) T shs[BLK * NP];
@@ -669,8 +698,8 @@ __global__ void __launch_bounds__(kElemBlock, (N == 1 ? 8 : 1)) elem_fused_kerne
     else
       volume_row<T, N>(u, a.geo[k], a.geo[a.K + k], a.geo[2 * a.K + k], a.geo[3 * a.K + k], a.geo[4 * a.K + k], rhs);
     const T ij = a.geo[5 * a.K + k];
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
+    for_faces([&](auto face_c) {
+      constexpr int f = decltype(face_c)::value;
       T acc[NFP], q[NFP], u1[NP], u2[NP];
       edge_rows<T, N>(ea, kk1[f], kk2[f], u1, u2);
       if constexpr (PRE) {
@@ -683,14 +712,8 @@ __global__ void __launch_bounds__(kElemBlock, (N == 1 ? 8 : 1)) elem_fused_kerne
       // negated and reversed
 #pragma unroll
       for (int c = 0; c < NFP; ++c) q[c] = (er[f] & 1) ? -acc[NFP - 1 - c] : acc[c];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        T s = T(0);
-#pragma unroll
-        for (int c = 0; c < NFP; ++c) s = fma((T)RDG_TAB[OLIFT + i * 3 * NFP + f * NFP + c], q[c], s);
-        rhs[i] -= ij * s;
-      }
-    }
+      lift_face<T, N, f>(q, ij, rhs);
+    });
     for (int m = 0; m < a.frc.nsrc; ++m) {
       const T* S = a.S + ((int64_t)m * a.K + k) * NP;
 #pragma unroll
@@ -716,13 +739,22 @@ __global__ void __launch_bounds__(kElemBlock, (N == 1 ? 8 : 1)) elem_fused_kerne
 }  // namespace dev
 
 // Host-side launch helpers instantiated by the including translation unit.
+// Programmatic launch in FP32.  In FP64 an ordinary one: dependent blocks that come early and wait take
+// the place of the running grid's (order 2, 8192 triangles: 24.1 us per stage against 12.1).
+template <typename T, typename... KArgs, typename... Args>
+inline int launch_stage_kernel(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t s, Args&&... args) {
+  if constexpr (sizeof(T) == 4) return launch_pdl(kernel, grid, block, s, std::forward<Args>(args)...);
+  kernel<<<grid, block, 0, s>>>(std::forward<Args>(args)...);
+  return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
+}
+
 template <typename T, int N, bool VOL = false>
 inline int launch_edge_t(const EdgeArgs<T>& a, cudaStream_t s) {
   const int64_t kv = a.Kvol > 0 ? a.Kvol : a.K;
   if (a.E == 0 && (!VOL || kv == 0)) return RDG_OK;
-  const int64_t ge = (a.E + kStageBlock - 1) / kStageBlock, gv = (kv + kStageBlock - 1) / kStageBlock;
-  if constexpr (VOL) return launch_pdl(dev::edge_flux_kernel<T, N, 1>, (unsigned)(ge + gv), kStageBlock, s, a);
-  dev::edge_flux_kernel<T, N, 0><<<(unsigned)ge, kStageBlock, 0, s>>>(a);
+  const int64_t ge = (a.E + dev::stage_block<T>() - 1) / dev::stage_block<T>(), gv = (kv + dev::stage_block<T>() - 1) / dev::stage_block<T>();
+  if constexpr (VOL) return launch_stage_kernel<T>(dev::edge_flux_kernel<T, N, 1>, (unsigned)(ge + gv), dev::stage_block<T>(), s, a);
+  dev::edge_flux_kernel<T, N, 0><<<(unsigned)ge, dev::stage_block<T>(), 0, s>>>(a);
   return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
 }
 
@@ -730,8 +762,8 @@ inline int launch_edge_t(const EdgeArgs<T>& a, cudaStream_t s) {
 template <typename T, int N>
 inline int launch_edge_fb_t(const EdgeArgs<T>& a, cudaStream_t s) {
   if (a.E == 0) return RDG_OK;
-  const int64_t ge = (a.E + kStageBlock - 1) / kStageBlock;
-  return launch_pdl(dev::edge_flux_kernel<T, N, 2>, (unsigned)ge, kStageBlock, s, a);
+  const int64_t ge = (a.E + dev::stage_block<T>() - 1) / dev::stage_block<T>();
+  return launch_stage_kernel<T>(dev::edge_flux_kernel<T, N, 2>, (unsigned)ge, dev::stage_block<T>(), s, a);
 }
 
 // One-kernel stage (elem_fused_kernel), programmatic launch.
@@ -756,11 +788,11 @@ inline int launch_elem_t(int mode, const ElemArgs<T>& a, cudaStream_t s) {
     constexpr int BLK = dev::lite_block<T, N>();
     const unsigned g2 = (unsigned)((a.K + BLK - 1) / BLK);
     switch (mode) {
-      case 0: return launch_pdl(dev::elem_lite_kernel<T, N, 0>, g2, BLK, s, a);
-      case 1: return launch_pdl(dev::elem_lite_kernel<T, N, 1>, g2, BLK, s, a);
-      case 2: return launch_pdl(dev::elem_lite_kernel<T, N, 2>, g2, BLK, s, a);
-      case 3: return launch_pdl(dev::elem_lite_kernel<T, N, 3>, g2, BLK, s, a);
-      case 4: return launch_pdl(dev::elem_lite_kernel<T, N, 4>, g2, BLK, s, a);
+      case 0: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 0>, g2, BLK, s, a);
+      case 1: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 1>, g2, BLK, s, a);
+      case 2: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 2>, g2, BLK, s, a);
+      case 3: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 3>, g2, BLK, s, a);
+      case 4: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 4>, g2, BLK, s, a);
       default: return RDG_EINVAL;
     }
   } else {

@@ -14,6 +14,16 @@
 
 #define RDG_CAT2(a, b) a##b
 #define RDG_CAT(a, b) RDG_CAT2(a, b)
+#define RDG_STR2(a) #a
+#define RDG_STR(a) RDG_STR2(a)
+
+// the order's mirror-split operators (gen_face.cpp)
+#include "face_ops.h"
+namespace rdg {
+namespace face {
+#include RDG_STR(RDG_CAT(face_ops_, RDG_ORDER).h)
+}  // namespace face
+}  // namespace rdg
 
 namespace {
 constexpr int kN = RDG_ORDER;
@@ -28,6 +38,15 @@ __device__ __align__(16) RDG_REAL g_voltab[4 * kNp * kNpp];
 #define RDG_TAB c_tab
 #define RDG_VOLTAB g_voltab
 #include "rhs_kernels.cuh"
+
+// FP64 objects also hold the small meshes' stage and its matrices, transposed (RowsShape).
+#define RDG_ROWS (!RDG_TAG_IS_F)
+#if RDG_ROWS
+#include "rows_kernel.cuh"
+namespace {
+__device__ __align__(16) double g_rowtab[rdg::dev::RowsShape<kN>::TAB];
+}  // namespace
+#endif
 
 // FP32 objects of orders 1..kMaxGemmN also hold the GEMM form of the edge flux.
 #define RDG_GEMM (RDG_TAG_IS_F && RDG_ORDER <= 5)
@@ -75,6 +94,20 @@ int RDG_CAT(upload_tab_, RDG_CAT(RDG_TAG, RDG_ORDER))() {
       }
     if (cudaMemcpyToSymbol(g_voltab, vt.data(), vt.size() * sizeof(RDG_REAL)) != cudaSuccess) return RDG_ECUDA;
   }
+#if RDG_ROWS
+  {
+    std::vector<double> rt;
+    for (int q = 0; q < 4; ++q)
+      for (int j = 0; j < kNp; ++j)
+        for (int i = 0; i < kNp; ++i) rt.push_back(t[(q * kNp + i) * kNp + j]);
+    const int nq = 3 * (kN + 1);
+    for (int j = 0; j < nq; ++j)
+      for (int i = 0; i < kNp; ++i) rt.push_back(t[4 * kNp * kNp + i * nq + j]);
+    if (rt.size() * sizeof(double) != sizeof(g_rowtab) ||
+        cudaMemcpyToSymbol(g_rowtab, rt.data(), sizeof(g_rowtab)) != cudaSuccess)
+      return RDG_ECUDA;
+  }
+#endif
 #if RDG_GEMM
   const RefOps* o = get_refops(kN, nullptr);
   if (!o) return RDG_EINVAL;
@@ -106,6 +139,14 @@ int RDG_CAT(launch_gemm_, RDG_CAT(RDG_TAG, RDG_ORDER))(const EdgeArgs<float>& a,
   if (cudaGetSymbolAddress(&xb, g_xb) != cudaSuccess || cudaGetSymbolAddress(&gt, g_gtab) != cudaSuccess)
     return RDG_ECUDA;
   return gemm::launch_gemm_t<kN>(a, static_cast<const float4*>(xb), static_cast<const int*>(gt), s);
+}
+#endif
+
+#if RDG_ROWS
+int RDG_CAT(launch_rows_, RDG_ORDER)(int mode, const EdgeArgs<double>& ea, const ElemArgs<double>& a, cudaStream_t s) {
+  void* tab = nullptr;
+  if (cudaGetSymbolAddress(&tab, g_rowtab) != cudaSuccess) return RDG_ECUDA;
+  return launch_rows_t<kN>(mode, ea, a, static_cast<const double*>(tab), s);
 }
 #endif
 
