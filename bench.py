@@ -139,8 +139,8 @@ class ClockSampler:
                 "reasons": sorted(reasons)}
 
 
-TRAFFIC_CSV = os.path.join(ROOT, "profiles", "stage_kernels_circle_pulse_N4_m256_fp32_dram.csv")
-STAGE_SOURCES = ("rhs_kernels.cuh", "rhs_order.cu")     # the stage and element kernels' code
+TRAFFIC_CSV = os.path.join(ROOT, "profiles", "face_stage_kernel_circle_pulse_N4_m256_fp32_dram.csv")
+STAGE_SOURCES = ("face_kernels.cuh", "face_ops.h", "gen_face.cpp", "face_order.cu")     # the stage kernel's code
 
 
 def stage_source_hash():
@@ -154,7 +154,7 @@ def stage_source_hash():
     return h.hexdigest()[:16]
 
 
-def profiled_traffic(args, kernel="edge_flux_kernel<float, 4, 1>"):
+def profiled_traffic(args, kernel="face_stage_kernel<4, 1"):
     """DRAM bytes (read + write) per launch of `kernel`, averaged over the launches of the
     committed ncu capture of this workload (steady state: no cache flush between launches),
     or None for another workload or when the kernels' sources changed after the capture
@@ -194,6 +194,15 @@ def alg_bytes_per_element(N, esz):
     edge/element ids.  Intermediates (face fluxes, volume term) are not counted."""
     Np, Nfp = (N + 1) * (N + 2) // 2, N + 1
     return esz * (3 * Np + 3 * Nfp * Np) + (56 if esz == 4 else 88)
+
+
+def face_bytes_per_element(N):
+    """Bytes per element per stage of the FP32 face form: stage input, step start (two of three
+    stages) and output rows, the own and the neighbours' face records read and the new ones
+    written, 24 bytes of parameters and neighbour per face and six element coefficients.  At
+    131072 triangles all of it stays in L2 between stages."""
+    Np, Nfp = (N + 1) * (N + 2) // 2, N + 1
+    return int(4 * ((2 + 2 / 3) * Np + 3 * Nfp + 3 * (Nfp + 1) + 3 * Nfp + 1)) + 3 * 24 + 24
 
 
 # ---------------------------------------------------------------------------------------
@@ -392,7 +401,7 @@ def run_ours(args):
     E, K, Np, Nfp = s.E, s.K, s.Np, s.Nfp
     # the algorithmic bytes of one stage (stored operators, state in and out,
     # coefficients and ids); the stage kernel is the dominant launch
-    stage_alg = alg_bytes_per_element(N_ORDER, 4) * K
+    stage_alg = (alg_bytes_per_element(N_ORDER, 4) if gemm else face_bytes_per_element(N_ORDER)) * K
     # the two kernels' own bytes, intermediates (volume term, face fluxes) included
     edge_bytes = E * ((Nfp * (2 * Np - 1) + 1) * 4 + 8 + Nfp * 4) + K * Np * 4 + K * Np * 4 + K * 5 * 4
     if gemm:   # parameter records (16-byte words) instead of operators, plus the face-pair word
@@ -401,22 +410,32 @@ def run_ours(args):
     peak, peak_kind = measured_peaks()
     edge_avg = edge_ms / edge_n
     elem_avg = elem_ms / elem_n
-    ach = stage_alg / (edge_avg / 1e3) / 1e9
-    traffic, traffic_src = (None, "GEMM form: no capture") if gemm else profiled_traffic(args)
-    kname = "edge_gemm_pipe_kernel<4>" if gemm else "edge_flux_kernel<float,4,VOL=1>"
-    roof = {"bound": "hbm", "kernel": kname,
-            "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-            "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % peak_kind, "traffic": traffic,
-            "traffic_source": traffic_src,
-            "alg_bytes_per_launch": stage_alg,
-            "alg_bytes_rule": "%d B per element per stage (stored operators, state in/out, coefficients, ids) x K"
-                              % alg_bytes_per_element(N_ORDER, 4),
-            "avg_launch_us": edge_avg * 1e3,
-            "share_of_kernel_time": edge_ms / (edge_ms + elem_ms),
-            "kernel_own_bytes": {"edge_and_volume_blocks": edge_bytes, "element_updates": elem_bytes,
-                                 "note": "reads and writes of the stage's two parts, volume-term and face-flux "
-                                         "round trips included (they mostly hit L2 in steady state)"},
-            "elem_kernel": {"name": "elem_lite_kernel<float,4,MODE>", "avg_launch_us": elem_avg * 1e3}}
+    p32, p64 = rdg.peak_fma(local, rdg.FP32), rdg.peak_fma(local, rdg.FP64)
+    # the method's dense products per stage: 8 Np^2 + 12 Np Nfp + 12 Np flops per element
+    flops_stage = (8 * Np * Np + 12 * Np * Nfp + 12 * Np) * K
+    if gemm:
+        ach = stage_alg / (edge_avg / 1e3) / 1e9
+        roof = {"bound": "hbm", "kernel": "edge_gemm_pipe_kernel<4>", "achieved": ach, "peak": peak, "unit": "GB/s",
+                "frac": ach / peak, "peak_source": "%s (MEASURED_PEAKS.json hbm_gbs)" % peak_kind,
+                "traffic": None, "traffic_source": "GEMM form: no capture", "alg_bytes_per_launch": stage_alg,
+                "avg_launch_us": edge_avg * 1e3, "share_of_kernel_time": edge_ms / (edge_ms + elem_ms),
+                "kernel_own_bytes": {"edge_and_volume_blocks": edge_bytes, "element_updates": elem_bytes,
+                                     "note": "reads and writes of the stage's two parts, volume-term and face-flux "
+                                             "round trips included (they mostly hit L2 in steady state)"},
+                "elem_kernel": {"name": "elem_lite_kernel<float,4,MODE>", "avg_launch_us": elem_avg * 1e3}}
+    else:
+        # one kernel per stage, bound by the rate at which instructions issue; the flops are the
+        # method's dense products (the kernel executes about half of them, split by symmetry)
+        ach = flops_stage / (elem_avg / 1e3) / 1e12
+        traffic, traffic_src = profiled_traffic(args)
+        roof = {"bound": "fp32 issue", "kernel": "face_stage_kernel<4>", "achieved": ach, "peak": p32 / 1e12,
+                "unit": "TFLOP/s", "frac": ach * 1e12 / p32, "peak_source": "measured (rdg_peak_fma)",
+                "traffic": traffic, "traffic_source": traffic_src, "alg_bytes_per_launch": stage_alg,
+                "alg_bytes_rule": "%d B per element per stage (rows, face records, parameters; L2-resident) x K"
+                                  % face_bytes_per_element(N_ORDER),
+                "avg_launch_us": elem_avg * 1e3, "share_of_kernel_time": elem_ms / (edge_ms + elem_ms),
+                "parts_kernel": {"name": "face_parts_kernel<4>", "avg_us_per_stage": edge_avg * 1e3,
+                                 "note": "once per solve; empty event brackets otherwise"}}
     # the whole stage inside the replayed graph (programmatic dependent launch): the same
     # algorithmic bytes over the timed solve's time per stage
     t_stage_s = t_ms / args.steps / (3 * nrk) / 1e3
@@ -424,29 +443,12 @@ def run_ours(args):
                                     "achieved_gbs": stage_alg / t_stage_s / 1e9,
                                     "frac": stage_alg / t_stage_s / 1e9 / peak}
 
-    # the compute side: measured FMA rates (in-process, this GPU at its current clocks) and
-    # the flops per element per stage, 8 Np^2 + 12 Np Nfp + 12 Np
-    p32, p64 = rdg.peak_fma(local, rdg.FP32), rdg.peak_fma(local, rdg.FP64)
-    flops_stage = (8 * Np * Np + 12 * Np * Nfp + 12 * Np) * K
     roof["rhs_roofline"] = {"t_bytes_us": stage_alg / (peak * 1e9) * 1e6, "t_flops_us": flops_stage / p32 * 1e6,
                             "bound": "hbm" if stage_alg / (peak * 1e9) >= flops_stage / p32 else "fp32",
                             "frac": max(stage_alg / (peak * 1e9), flops_stage / p32) / t_stage_s,
                             "flops_per_stage": flops_stage}
     compute_peaks = {"fp32_tflops": p32 / 1e12, "fp64_tflops": p64 / 1e12,
                      "how": "rdg_peak_fma: independent FMA chains on every SM, CUDA events, best of 4"}
-    # the size-matched bound: a plain streaming read of the stage's algorithmic bytes and of
-    # the operators alone, each a standalone launch (rdg_stream_read)
-    w_bytes = ((E + 31) // 32) * ((Nfp * (2 * Np - 1) + 1 + 3) // 4) * 32 * 16
-    t_rd_stage = rdg.stream_read_seconds(local, stage_alg)
-    t_rd_w = rdg.stream_read_seconds(local, w_bytes)
-    roof["size_matched_read"] = {"stage_alg_bytes": stage_alg, "read_us": t_rd_stage * 1e6,
-                                 "read_gbs": stage_alg / t_rd_stage / 1e9,
-                                 "operator_bytes": w_bytes, "operator_read_us": t_rd_w * 1e6,
-                                 "stage_us_in_graph": t_stage_s * 1e6,
-                                 "stage_time_over_read_time": t_stage_s / t_rd_stage,
-                                 "how": "rdg_stream_read: float4 evict-first grid-stride read, L2 flushed, "
-                                        "median of 8 standalone launches"}
-
     # end to end through the C ABI with host buffers (copies inside the timed region)
     e2e_t = []
     in_pinned = torch.from_numpy(u0_host).pin_memory()       # inputs in pinned host memory
@@ -594,7 +596,10 @@ def run_ours(args):
     if s64_head is not None:
         s64_head.close()
 
-    per_solve = (1 + (nrk // 16) * (16 * 6 + 1) if nrk >= 16 else 0) + (nrk % 16) * 6
+    if gemm:    # two kernels per stage
+        per_solve = (1 + (nrk // 16) * (16 * 6 + 1) if nrk >= 16 else 0) + (nrk % 16) * 6
+    else:       # the records of the state once, then one kernel per stage (and the chunk's time kernels)
+        per_solve = 1 + 3 * nrk + (1 + nrk // 16 if nrk >= 16 else 0)
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
@@ -947,15 +952,15 @@ def run_orders(args):
                     ts.append(a.elapsed_time(b) * 1e3 / per)
                 forms[fname] = float(np.median(ts))
             us = forms["default"]
-            default_form = "one_kernel" if s.stage_form == rdg.STAGE_ONE_KERNEL else "two_kernels"
+            default_form = "face" if esz == 4 else "two_kernels"
             E, K, Np, Nfp = s.E, s.K, s.Np, N + 1
             w_bytes = E * (Nfp * (2 * Np - 1) + 1) * esz
-            # the algorithmic bytes per element (stored operators, state in and out,
-            # coefficients, ids); beside them the two kernels' own bytes at this order and
-            # precision: edge pass (operators, edge ids, face fluxes, stage input, volume term,
+            # the algorithmic bytes per element (FP32: the face form's; FP64: stored operators, state
+            # in and out, coefficients, ids); beside them the two-kernel form's own bytes at this
+            # order and precision: edge pass (operators, edge ids, face fluxes, stage input, volume term,
             # element coefficients) and element pass (volume term, stage input, step start in
             # two of three stages, output, ids, 1/J, face fluxes)
-            alg = alg_bytes_per_element(N, esz) * K
+            alg = (face_bytes_per_element(N) if esz == 4 else alg_bytes_per_element(N, esz)) * K
             own = (E * ((Nfp * (2 * Np - 1) + 1) * esz + 8 + Nfp * esz) + 2 * K * Np * esz + K * 5 * esz
                    + int(K * ((3 + 2.0 / 3.0) * Np * esz + 12 + esz) + E * Nfp * esz))
             rows.append({"N": N, "precision": name, "stage_us": us, "stage_form": default_form,

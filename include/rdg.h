@@ -194,8 +194,9 @@ int rdg_rhs_eval(rdg_ctx* ctx, const void* u_dev, void* rhs_dev, double t);
  * evaluate the right-hand side (inside another component's CUDA-graph capture, in loops
  * that must not hit cudaMalloc's implicit synchronisation, or under a pool allocator that
  * owns all device memory).  It computes the same right-hand side as rdg_rhs_eval, to rounding,
- * with the unfused pair of kernels (per-edge fluxes, then an element kernel that forms the
- * volume term, LIFT and sources), and keeps the per-edge fluxes in one static device array
+ * with launches that allocate nothing: FP32 contexts run the face form in their own record
+ * buffers, the others the unfused pair of kernels (per-edge fluxes, then an element kernel that
+ * forms the volume term, LIFT and sources) with the per-edge fluxes in one static device array
  * compiled into the library, 8 MiB,
  * held by every GPU that loads the library until the process exits; it calls no allocating
  * routine.  Meshes needing more than 8 MiB of fluxes (n_edges x Nfp x element size) get
@@ -224,13 +225,19 @@ int rdg_set_integrator(rdg_ctx* ctx, int integrator);
  *                        volume terms) and an element kernel (LIFT, sources, stage update);
  * RDG_STAGE_ONE_KERNEL   one element kernel that also computes its three edges' fluxes (each
  *                        edge's operator read by both of its elements; one launch per stage);
- * RDG_STAGE_AUTO         (default) the form measured faster for the context's order and
- *                        precision on GB300 (one kernel for FP32 order 1, two otherwise).
+ * RDG_STAGE_AUTO         (default) the fastest on GB300: FP32 with an element-wise D runs the face
+ *                        form (no per-edge operators, one kernel per stage and integrator
+ *                        stage of any kind, a lone right-hand side in one or two), small FP64
+ *                        meshes one kernel with a lane per (element, node), everything else
+ *                        two kernels.
+ * Setting a per-edge form on an FP32 context builds its operators there and then (device memory
+ * as rdg_query_bytes says; RDG_ENOMEM if there is none).
  * The one-kernel form serves rdg_rhs_eval and SSP-RK3 stages of contexts with stored
  * operators; the low-storage integrator (which updates its input in place), the GEMM form
  * and FP32 order 6 (tensor-core volume term) keep two kernels whatever is set.  Errors:
  * RDG_EINVAL for another value.  rdg_get_stage_form reports the form in use for a
- * right-hand-side stage (RDG_STAGE_ONE_KERNEL or RDG_STAGE_TWO_KERNELS) in *form. */
+ * right-hand-side stage (RDG_STAGE_ONE_KERNEL or RDG_STAGE_TWO_KERNELS) in *form; under
+ * RDG_STAGE_AUTO it names the per-edge form (one kernel for FP32 order 1, two otherwise). */
 enum { RDG_STAGE_AUTO = 0, RDG_STAGE_TWO_KERNELS = 1, RDG_STAGE_ONE_KERNEL = 2 };
 int rdg_set_stage_form(rdg_ctx* ctx, int form);
 int rdg_get_stage_form(const rdg_ctx* ctx, int* form);
@@ -292,8 +299,8 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps);
 
 /* Bytes of the per-edge flux operators that every stage loads with an evict-last L2 policy,
  * so they stay L2-resident from one stage to the next instead of streaming from HBM again
- * (the rest is streamed evict-first).  -1 (the default) and 0 stream everything.  Affects
- * speed only, never results. */
+ * (the rest is streamed evict-first).  -1 (the default) and 0 stream everything; the face form
+ * has none.  Affects speed only, never results. */
 int rdg_set_l2_resident_bytes(rdg_ctx* ctx, int64_t bytes);
 
 /* Per-kernel timing.  With enable != 0 every later edge-flux and element-update kernel launch

@@ -1001,6 +1001,10 @@ int enqueue_face_parts(rdg_ctx* ctx, const float* us, int64_t k0, int64_t k1) {
   return launch_face_parts(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, ls(ctx));
 }
 
+// Elements up to which a lone right-hand side is one launch (8192 elements, us per call with the host side,
+// one launch / two: order 2 3.8 / 6.1, order 4 4.7 / 6.0; 19602: order 3 5.0 / 6.2, order 4 6.4 / 6.0).
+constexpr int64_t kDirectRhsMax[kMaxN + 1] = {0, 20000, 20000, 20000, 10000, 5000, 5000};
+
 // A stage in the face form.  fresh: the records of us are formed first (they are current only after
 // a stage that kept them, with nothing else having touched its result); keep: leave the records of
 // the result, in the other buffer.  On a split mesh, part 0: the owned elements' records (they read
@@ -1016,8 +1020,10 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
     cudaEventRecord(ev[0], st);
   }
   int rc = RDG_OK;
+  // a lone right-hand side of a small mesh needs no records
+  const bool direct = mode == 0 && part < 0 && fresh && !keep && ctx->K <= kDirectRhsMax[ctx->N];
   if (part == 1) rc = enqueue_face_parts(ctx, us, ctx->n_owned, ctx->K);
-  else if (fresh) rc = enqueue_face_parts(ctx, us, 0, ctx->K);
+  else if (fresh && !direct) rc = enqueue_face_parts(ctx, us, 0, ctx->K);
   if (prof) {
     cudaEventRecord(ev[1], st);
     cudaEventRecord(ev[2], st);
@@ -1033,7 +1039,9 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
   a.dt = dt;
   a.rka = rka;
   a.rkb = rkb;
-  if (rc == RDG_OK) rc = launch_face_stage(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st);
+  if (rc == RDG_OK)
+    rc = direct ? launch_face_rhs(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st)
+                : launch_face_stage(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st);
   if (rc == RDG_OK && keep) ctx->rec_cur ^= 1;
   if (prof) {
     cudaEventRecord(ev[3], st);

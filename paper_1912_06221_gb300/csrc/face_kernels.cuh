@@ -636,5 +636,114 @@ __global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const 
   team_tile<N, ALG1, false>(a, k0, (int)min((int64_t)32, a.K - k0), su, sp);
 }
 
+// A lone right-hand side of a small mesh in one launch: a thread evaluates its neighbours' parts beside
+// its own (the same arithmetic on the neighbour's row, so the same bits) instead of reading records of a
+// first launch.  Twice the parts' work, which is free while there is at most a warp per scheduler; what
+// bounds such a call is its launches (order 2, 512 triangles).
+template <int N, bool ALG1>
+__global__ void __launch_bounds__(kFaceBlock) face_rhs_kernel(const __grid_constant__ FaceArgs a) {
+  using O = face::Ops<N>;
+  constexpr int NP = np_of(N), NG = N + 1;
+  __shared__ __align__(16) float sh_all[kFaceWarps][32 * NP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* sh = sh_all[warp];
+  const int64_t k0 = ((int64_t)blockIdx.x * kFaceWarps + warp) * 32;
+  const int nk = (int)min((int64_t)32, a.K - k0);
+  if (nk <= 0) return;
+  const bool active = lane < nk;
+  const int row = active ? lane : nk - 1;
+  const unsigned k = (unsigned)(k0 + row), K = (unsigned)a.K, K3 = 3u * K;
+  unsigned nbr[3];
+  bool diff[3];
+  float geo[6];
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    nbr[f] = __ldg(a.nbr + (size_t)f * K + k);
+    diff[f] = jump_in_warp<ALG1>(nbr[f]);
+    nbr[f] &= ~kFaceJump;
+  }
+#pragma unroll
+  for (int c = 0; c < 6; ++c) geo[c] = __ldg(a.geo + (size_t)c * K + k);
+  wait_for_predecessor();
+  allow_dependents();
+  rows_in<NP>(sh, a.us + k0 * NP, nk * NP, lane);
+  rows_commit();
+  rows_wait<0>();
+  float d[NP], rhs[NP];
+  row_get<NP>(sh + row * NP, d);
+  const float u0 = d[0];
+#pragma unroll
+  for (int j = 0; j < NP; ++j) d[j] -= u0;
+  {
+    float ve[O::NE], vo[O::NO];
+    face::volume_parts<float, N>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+    O::nodes(ve, vo, rhs);
+  }
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) {         // faces 1, 2, 0: d and rhs rotate into the face's order
+    const int f = i == 2 ? 0 : i + 1;
+    const unsigned r = i == 0 ? nbr[1] : (i == 1 ? nbr[2] : nbr[0]);
+    const bool df = i == 0 ? diff[1] : (i == 1 ? diff[2] : diff[0]);
+    const face::Par<float> p = face_par(a, f, k, df);
+    float g[NG], ng[NG + 1];
+    face::face_part<float, N, 1, ALG1>(d, p, df, g);
+    {
+      unsigned q = r;
+      if (q >= K3) {
+        if (q >= K3 + (unsigned)a.B) report(a.err, kErrBadIndex);
+        q = k;
+      }
+      const int fn = q >= 2u * K ? 2 : (q >= K ? 1 : 0);
+      const unsigned kn = q - (unsigned)fn * K;
+      float v[NP], w[NP], n[NG];
+      row_get<NP>(a.us + (int64_t)kn * NP, v);
+      const float n0 = v[0];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) w[j] = v[j] -= n0;
+      O::rotate(w);
+#pragma unroll
+      for (int j = 0; j < NP; ++j) v[j] = fn == 1 ? v[j] : w[j];
+      O::rotate(w);
+#pragma unroll
+      for (int j = 0; j < NP; ++j) v[j] = fn == 0 ? w[j] : v[j];
+      face::face_part<float, N, 1, ALG1>(v, face_par(a, fn, kn, df), df, n);
+#pragma unroll
+      for (int c = 0; c < NG; ++c) ng[c] = n[c];
+      ng[NG] = n0;
+    }
+    if (r >= K3) ghost_get<NG>(a, r - K3, ng);
+    float ge[O::GE], go[O::GO], ve[O::NE], vo[O::NO];
+#pragma unroll
+    for (int q = 0; q < O::GE; ++q) ge[q] = g[q];
+#pragma unroll
+    for (int q = 0; q < O::GO; ++q) go[q] = g[O::GE + q];
+    face::face_flux<float, N, ALG1>(p, df, u0, ng[NG], ng, ge, go);
+#pragma unroll
+    for (int q = 0; q < O::GE; ++q) ge[q] *= -geo[5];
+#pragma unroll
+    for (int q = 0; q < O::GO; ++q) go[q] *= -geo[5];
+#pragma unroll
+    for (int q = 0; q < O::NE; ++q) ve[q] = 0.f;
+#pragma unroll
+    for (int q = 0; q < O::NO; ++q) vo[q] = 0.f;
+    O::lift_even(ge, ve);
+    O::lift_odd(go, vo);
+    O::join1(ve, vo, rhs);
+    O::rotate(rhs);
+    O::rotate(d);
+  }
+  for (int m = 0; m < a.nsrc; ++m) {
+    float S[NP];
+    row_get<NP>(a.S + ((int64_t)m * a.K + k) * NP, S);
+    const float tm = stage_tau(a, m);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) rhs[i] = fmaf(tm, S[i], rhs[i]);
+  }
+  __syncwarp();
+  if (active) row_put<NP>(sh + lane * NP, rhs);
+  __syncwarp();
+  rows_out<NP>(a.out + k0 * NP, sh, nk * NP, lane);
+}
+
 }  // namespace dev
 }  // namespace rdg

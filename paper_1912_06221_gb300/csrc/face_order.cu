@@ -71,6 +71,13 @@ int RDG_CAT(launch_face_stage_, RDG_ORDER)(bool alg1, const FaceArgs& a, cudaStr
   return alg1 ? launch_stage<true>(a, s) : launch_stage<false>(a, s);
 }
 
+int RDG_CAT(launch_face_rhs_, RDG_ORDER)(bool alg1, const FaceArgs& a, cudaStream_t s) {
+  if (a.K == 0) return RDG_OK;
+  const unsigned grid = (unsigned)((a.K + dev::kFaceBlock - 1) / dev::kFaceBlock);
+  return alg1 ? launch_pdl(dev::face_rhs_kernel<RDG_ORDER, true>, grid, dev::kFaceBlock, s, a)
+              : launch_pdl(dev::face_rhs_kernel<RDG_ORDER, false>, grid, dev::kFaceBlock, s, a);
+}
+
 int RDG_CAT(launch_face_ghost_, RDG_ORDER)(bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out,
                                            cudaStream_t s) {
   constexpr int N = RDG_ORDER;
