@@ -1344,6 +1344,9 @@ int rdg_rows_scatter(rdg_ctx* ctx, const void* src_dev, const int32_t* idx_dev, 
   return rc == RDG_OK ? RDG_OK : fail(ctx, rc, "kernel launch failed");
 }
 
+// Steps below which the first solve of a dt is not captured.
+static constexpr int64_t kDirectSteps = 128;
+
 int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
   if (!ctx) return RDG_EINVAL;
   if (!ctx->ops_ok) return fail(ctx, RDG_ESTATE, "rdg_operator_setup must come first");
@@ -1351,7 +1354,13 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
   if (nsteps == 0) return RDG_OK;
   DeviceGuard g(ctx->device);
   const int chunk = ctx->prof ? (int)(nsteps + 1) : 16;   // profiling steps without the graph
-  if (nsteps >= chunk && (!ctx->gexec || ctx->g_dt != dt)) {
+  // A graph of a chunk costs about 0.2 ms to capture and instantiate.  The first solve of a dt launches
+  // its steps directly where there are few (a launch costs less than a stage takes on all but tiny
+  // meshes, and the device starts at once); it is captured when the dt comes again or the solve is long.
+  const bool ready = ctx->gexec && ctx->g_dt == dt;
+  const bool replay = nsteps >= chunk && (ready || nsteps >= kDirectSteps || ctx->seen_dt == dt);
+  ctx->seen_dt = dt;
+  if (replay && !ready) {
     if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
     ctx->gexec = nullptr;
     cudaGraph_t graph;
@@ -1379,7 +1388,7 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
     ctx->g_chunk = chunk;
   }
   int64_t done = 0;
-  if (nsteps >= chunk) {
+  if (replay) {
     int rc = set_time(ctx->d_time, t0, ctx->stream);
     if (rc == RDG_OK && use_face(ctx)) {
       ctx->rec_cur = 0;

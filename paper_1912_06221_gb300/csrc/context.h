@@ -77,6 +77,7 @@ struct rdg_ctx {
   // graph of a chunk of steps for one dt
   cudaGraphExec_t gexec = nullptr;
   double g_dt = 0;
+  double seen_dt = 0;              // dt of the last solve (dt is positive)
   int g_chunk = 0;
 };
 

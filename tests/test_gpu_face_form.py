@@ -71,3 +71,31 @@ def test_face_form_kernel_choice_matches_fp64(N, large, integ):
     want = _run(N, m, rdg.FP64, "jump", rdg.IFACE_ALG1, rdg.BC_DIRICHLET, integ)
     for a, b in zip(got, want):
         assert parity_err(a, b) < 1e-5
+
+
+@pytest.mark.parametrize("prec,N,integ", [(rdg.FP32, 2, rdg.SSP_RK3), (rdg.FP32, 5, rdg.LSRK54), (rdg.FP64, 3, rdg.SSP_RK3),
+                                          (rdg.FP32_3XTF32, 4, rdg.SSP_RK3)])
+@pytest.mark.parametrize("forced", [False, True])
+def test_direct_and_replayed_solves_agree(prec, N, integ, forced):
+    """The first solve of a dt launches its steps directly, the next one replays a captured chunk (16
+    steps, then three more): the same kernels, so the same bits; with forcing the stage times are summed
+    in another order, 1e-6 in FP32 and 1e-13 in FP64."""
+    xy, tri = unit_square_mesh(11, 0.1, 3)
+    s = rdg.Solver(xy, tri, N, 0.4, v=(0.3, 0.2), precision=prec)
+    s.set_integrator(integ)
+    if forced:
+        x = s.node_coords()
+        s.set_forcing([(np.sin(3 * x[..., 0]) * x[..., 1], rdg.TAU_COS, 200.0)])
+    u = torch.tensor(random_nodal(s.K, s.Np, 7), dtype=s.dtype, device="cuda")
+    out = []
+    for _ in range(3):
+        s.set_state(u)
+        s.solve_to_time(0.2, 0.02 / 11 ** 2 / (N + 1) ** 4, 19)
+        out.append(s.get_state_host().astype(np.float64))
+    s.synchronize()
+    s.close()
+    assert np.array_equal(out[1], out[2])
+    if forced:
+        assert parity_err(out[0], out[1]) < (1e-13 if prec == rdg.FP64 else 1e-6)
+    else:
+        assert np.array_equal(out[0], out[1])
