@@ -250,8 +250,7 @@ static int mesh_upload_impl(rdg_ctx* ctx, int64_t nv, const double* xy, int64_t 
   ctx->K = nt;
   ctx->n_owned = n_owned;
   ctx->bc = bc;
-  ctx->exy.assign(nt * 6, 0.0);
-  double hmin = 1e300;
+  ctx->exy.resize(nt * 6);
   for (int64_t k = 0; k < nt; ++k) {
     for (int c = 0; c < 3; ++c) {
       int32_t v = tri[3 * k + c];
@@ -265,9 +264,7 @@ static int mesh_upload_impl(rdg_ctx* ctx, int64_t nv, const double* xy, int64_t 
                           (p[4] - p[2]) * (p[4] - p[2]) + (p[5] - p[3]) * (p[5] - p[3]),
                           (p[0] - p[4]) * (p[0] - p[4]) + (p[1] - p[5]) * (p[1] - p[5])});
     if (!(J > 1e-12 * l2)) return fail(ctx, RDG_EMESH, "triangle " + std::to_string(k) + " is clockwise or degenerate");
-    hmin = std::min(hmin, std::sqrt(l2));
   }
-  (void)hmin;
   // Faces are matched first by their vertex ids: a counting sort of the faces by their lower
   // vertex id, then equal upper ids within each (small) bucket.  The faces left over (domain
   // boundary, periodic images, vertices duplicated at one point) are matched by their
@@ -275,42 +272,41 @@ static int mesh_upload_impl(rdg_ctx* ctx, int64_t nv, const double* xy, int64_t 
   const int64_t nf = 3 * nt;
   std::vector<int64_t> partner(nf, -1);
   {
-    auto lo_hi = [&](int64_t i, int32_t* lo, int32_t* hi) {
-      const int32_t a = tri[3 * (i / 3) + kFaceA[i % 3]], b = tri[3 * (i / 3) + kFaceB[i % 3]];
-      *lo = std::min(a, b);
-      *hi = std::max(a, b);
-    };
+    // a face's vertex ids in one word, lower id above: equal words are the two sides of an edge
+    std::vector<uint64_t> key(nf);
     std::vector<int64_t> start(nv + 1, 0);
-    for (int64_t i = 0; i < nf; ++i) {
-      int32_t lo, hi;
-      lo_hi(i, &lo, &hi);
-      start[lo + 1]++;
-    }
-    for (int64_t v = 0; v < nv; ++v) start[v + 1] += start[v];
-    std::vector<int64_t> fill(start.begin(), start.end() - 1), bucket(nf);
-    for (int64_t i = 0; i < nf; ++i) {
-      int32_t lo, hi;
-      lo_hi(i, &lo, &hi);
-      bucket[fill[lo]++] = i;
-    }
-    std::vector<std::pair<int32_t, int64_t>> run;
-    for (int64_t v = 0; v < nv; ++v) {
-      const int64_t b0 = start[v], n = start[v + 1] - b0;
-      if (n < 2) continue;
-      run.clear();
-      for (int64_t j = 0; j < n; ++j) {
-        int32_t lo, hi;
-        lo_hi(bucket[b0 + j], &lo, &hi);
-        run.push_back({hi, bucket[b0 + j]});
+    for (int64_t k = 0; k < nt; ++k)
+      for (int f = 0; f < 3; ++f) {
+        const uint32_t a = (uint32_t)tri[3 * k + kFaceA[f]], b = (uint32_t)tri[3 * k + kFaceB[f]];
+        const uint32_t lo = std::min(a, b), hi = std::max(a, b);
+        key[3 * k + f] = (uint64_t)lo << 32 | hi;
+        start[lo + 1]++;
       }
-      std::sort(run.begin(), run.end());
+    for (int64_t v = 0; v < nv; ++v) start[v + 1] += start[v];
+    // bucket by lower id (in face order within each); start[v] becomes the end of bucket v
+    std::vector<int64_t> bucket(nf);
+    for (int64_t i = 0; i < nf; ++i) bucket[start[key[i] >> 32]++] = i;
+    for (int64_t v = 0; v < nv; ++v) {
+      const int64_t b0 = v > 0 ? start[v - 1] : 0, n = start[v] - b0;
+      if (n < 2) continue;
+      int64_t* run = &bucket[b0];
+      if (n > 32) {
+        std::stable_sort(run, run + n, [&](int64_t x, int64_t y) { return key[x] < key[y]; });
+      } else {                                  // a handful of faces: insertion sort by upper id
+        for (int64_t j = 1; j < n; ++j) {
+          const int64_t x = run[j];
+          int64_t q = j;
+          for (; q > 0 && key[run[q - 1]] > key[x]; --q) run[q] = run[q - 1];
+          run[q] = x;
+        }
+      }
       for (int64_t j = 0; j < n;) {
         int64_t q = j + 1;
-        while (q < n && run[q].first == run[j].first) ++q;
+        while (q < n && key[run[q]] == key[run[j]]) ++q;
         if (q - j > 2) return fail(ctx, RDG_EMESH, "non-manifold edge (shared by more than two faces)");
         if (q - j == 2) {
-          partner[run[j].second] = run[j + 1].second;
-          partner[run[j + 1].second] = run[j].second;
+          partner[run[j]] = run[j + 1];
+          partner[run[j + 1]] = run[j];
         }
         j = q;
       }
@@ -355,7 +351,8 @@ static int mesh_upload_impl(rdg_ctx* ctx, int64_t nv, const double* xy, int64_t 
   }
   // edges in the order of their first face (sorted by first element, for locality of the
   // neighbour gathers): interior edges, then boundary edges
-  std::vector<EdgeRec> inner, bnd;
+  std::vector<EdgeRec> &inner = ctx->edges, bnd;
+  inner.clear();
   inner.reserve(nf / 2 + 1);
   for (int64_t i = 0; i < nf; ++i) {
     const int64_t j = partner[i];
@@ -386,7 +383,6 @@ static int mesh_upload_impl(rdg_ctx* ctx, int64_t nv, const double* xy, int64_t 
     inner.push_back(r);
   }
   for (size_t b = 0; b < bnd.size(); ++b) bnd[b].k2 = -1 - (int32_t)b;
-  ctx->edges = inner;
   ctx->edges.insert(ctx->edges.end(), bnd.begin(), bnd.end());
   ctx->E = (int64_t)ctx->edges.size();
   ctx->B = (int64_t)bnd.size();
