@@ -194,8 +194,10 @@ int rdg_rhs_eval(rdg_ctx* ctx, const void* u_dev, void* rhs_dev, double t);
  * evaluate the right-hand side (inside another component's CUDA-graph capture, in loops
  * that must not hit cudaMalloc's implicit synchronisation, or under a pool allocator that
  * owns all device memory).  It computes the same right-hand side as rdg_rhs_eval, to rounding,
- * with launches that allocate nothing: FP32 contexts run the face form in their own record
- * buffers, the others the unfused pair of kernels (per-edge fluxes, then an element kernel that
+ * with launches that allocate nothing and write none of the context's buffers (a call between
+ * the two parts of a stage, or a replay of a captured one beside the context's own work, leaves
+ * that work alone): contexts in the face form (see rdg_set_stage_form) one launch without
+ * scratch, the others the unfused pair of kernels (per-edge fluxes, then an element kernel that
  * forms the volume term, LIFT and sources) with the per-edge fluxes in one static device array
  * compiled into the library, 8 MiB,
  * held by every GPU that loads the library until the process exits; it calls no allocating
@@ -205,7 +207,7 @@ int rdg_rhs_eval(rdg_ctx* ctx, const void* u_dev, void* rhs_dev, double t);
  * process, so the address is valid only while that device's primary context lives (not after
  * a cudaDeviceReset); make that first call before any stream capture.  Contexts using the
  * GEMM form of the edge flux (RDG_FP32_3XTF32 with N <= 5 and an interface rule other than
- * RDG_IFACE_ALG1) have no stored operators and get RDG_ESTATE.  All calls share the array, which keeps the last call's contents (every
+ * RDG_IFACE_ALG1) have no stored operators and get RDG_ESTATE.  All calls that use the array share it; it keeps the last call's contents (every
  * flux is rewritten before it is read, so nothing is cleared): calls whose GPU work
  * overlaps (different streams or devices' contexts sharing a device) race on it.  The paper
  * has no counterpart to this entry point. */

@@ -988,10 +988,10 @@ void face_forcing(const rdg_ctx* ctx, const TimeArg& ta, int stage, FaceArgs& a)
   for (int m = 0; m < f.nghost; ++m) a.tau[RDG_MAX_FORCING_TERMS + m] = (float)host_tau(f.gkind[m], f.gomega[m], t);
 }
 
-// Face records of elements [k0, k1) of us into the current buffer.
-int enqueue_face_parts(rdg_ctx* ctx, const float* us, int64_t k0, int64_t k1) {
+// Face records of elements [k0, k1) of us into buffer buf.
+int enqueue_face_parts(rdg_ctx* ctx, const float* us, int64_t k0, int64_t k1, int buf) {
   FaceArgs a = face_args(ctx, us);
-  a.fout = ctx->d_rec[ctx->rec_cur];
+  a.fout = ctx->d_rec[buf];
   a.k_begin = k0 & ~(int64_t)3;   // 16-byte rows; the few elements before k0 get the same records again
   a.k_end = k1;
   return launch_face_parts(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, ls(ctx));
@@ -1004,10 +1004,12 @@ constexpr int64_t kDirectRhsMax[kMaxN + 1] = {0, 20000, 20000, 20000, 10000, 500
 // A stage in the face form.  fresh: the records of us are formed first (they are current only after
 // a stage that kept them, with nothing else having touched its result); keep: leave the records of
 // the result, in the other buffer.  On a split mesh, part 0: the owned elements' records (they read
-// owned rows only), part 1: the halo elements' records, then the stage.
+// owned rows only), part 1: the halo elements' records, then the stage.  Between the two the current
+// buffer holds the pending stage's records, so a lone right-hand side forms its own in the other one.
 int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* out, int mode, float dt, const TimeArg& ta,
                        float* out2, float rka, float rkb, int part, bool fresh, bool keep, int stage) {
-  if (part == 0) return enqueue_face_parts(ctx, us, 0, ctx->n_owned);
+  const int buf = mode == 0 ? ctx->rec_cur ^ 1 : ctx->rec_cur;
+  if (part == 0) return enqueue_face_parts(ctx, us, 0, ctx->n_owned, buf);
   cudaStream_t st = ls(ctx);
   const bool prof = ctx->prof && !ctx->capturing;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -1018,8 +1020,8 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
   int rc = RDG_OK;
   // a lone right-hand side of a small mesh needs no records
   const bool direct = mode == 0 && part < 0 && fresh && !keep && ctx->K <= kDirectRhsMax[ctx->N];
-  if (part == 1) rc = enqueue_face_parts(ctx, us, ctx->n_owned, ctx->K);
-  else if (fresh && !direct) rc = enqueue_face_parts(ctx, us, 0, ctx->K);
+  if (part == 1) rc = enqueue_face_parts(ctx, us, ctx->n_owned, ctx->K, buf);
+  else if (fresh && !direct) rc = enqueue_face_parts(ctx, us, 0, ctx->K, buf);
   if (prof) {
     cudaEventRecord(ev[1], st);
     cudaEventRecord(ev[2], st);
@@ -1029,7 +1031,7 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
   a.un = un;
   a.out = out;
   a.out2 = out2;
-  a.fin = ctx->d_rec[ctx->rec_cur];
+  a.fin = ctx->d_rec[buf];
   a.fout = keep ? ctx->d_rec[ctx->rec_cur ^ 1] : nullptr;
   a.mode = mode;
   a.dt = dt;
@@ -1249,7 +1251,10 @@ int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double
 FaceArgs face_member_args(const rdg_ctx* ctx) { return face_args(ctx, nullptr); }
 
 int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta) {
-  return enqueue_face_stage(ctx, u, nullptr, rhs, 0, 0.0f, ta, nullptr, 0.0f, 0.0f, -1, true, false, 0);
+  FaceArgs a = face_args(ctx, u);
+  face_forcing(ctx, ta, 0, a);
+  a.out = rhs;
+  return launch_face_rhs(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, ctx->stream);
 }
 
 }  // namespace rdg
@@ -1388,7 +1393,7 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
     int rc = set_time(ctx->d_time, t0, ctx->stream);
     if (rc == RDG_OK && use_face(ctx)) {
       ctx->rec_cur = 0;
-      rc = enqueue_face_parts(ctx, (const float*)ctx->d_u, 0, ctx->K);
+      rc = enqueue_face_parts(ctx, (const float*)ctx->d_u, 0, ctx->K, 0);
     }
     if (rc != RDG_OK) return fail(ctx, rc, "kernel launch failed");
     for (; done + chunk <= nsteps; done += chunk) CK(cudaGraphLaunch(ctx->gexec, ctx->stream));

@@ -92,7 +92,7 @@ int ensure_edge_form(rdg_ctx* ctx);
 int enqueue_rk_step_on(rdg_ctx* ctx, cudaStream_t s, const TimeArg& base, double dt, bool fresh, bool keep);
 // What every stage of ctx's face form takes, without the stage's own buffers, mode and forcing factors.
 FaceArgs face_member_args(const rdg_ctx* ctx);
-// Right-hand side of u in the face form (two launches, no allocation).
+// Right-hand side of u in the face form in one launch that writes rhs and nothing of the context's.
 int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta);
 // Row gather (dst[i] = src[idx[i]]) or scatter (dst[idx[i]] = src[i]) of np-value rows of
 // esz-byte values; indices outside 0..nrows-1 are recorded in err and skipped.

@@ -8,7 +8,10 @@
 // point uses, instead, one fixed scratch array compiled into the library (kStaticFluxBytes)
 // and calls no allocating routine at all.  It runs the unfused pair of kernels (edge fluxes
 // into that array, then the element kernel with the volume term, LIFT and sources), not the
-// fused pair of rdg_rhs_eval; the two agree to rounding.  The paper has no counterpart to it.
+// fused pair of rdg_rhs_eval; the two agree to rounding.  In the face form (FP32, element-wise D) it
+// is one launch that recomputes the neighbours' parts (face_rhs_kernel) and needs no scratch at all:
+// the context's record buffers belong to its stages, one of which may be between its two parts or
+// running elsewhere when this is called or replayed.  The paper has no counterpart to it.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -76,7 +79,7 @@ extern "C" int rdg_rhs_eval_static(rdg_ctx* ctx, const void* u_dev, void* rhs_de
     // array needs no clearing between calls
     TimeArg ta{nullptr, t, 1.0, 0.0};
     if (use_face(ctx)) {
-      rc = enqueue_face_rhs(ctx, (const float*)u_dev, (float*)rhs_dev, ta);   // in the context's own records
+      rc = enqueue_face_rhs(ctx, (const float*)u_dev, (float*)rhs_dev, ta);
     } else if (ctx->esz == 4) {
       EdgeArgs<float> ea{ctx->d_k1, ctx->d_k2, ctx->d_W, (const float*)u_dev, (float*)flux, (const float*)ctx->d_G,
                          ctx->E, ctx->B, ctx->frc, ta, ctx->d_err, ctx->K};
