@@ -422,8 +422,8 @@ int rdg_batch_synchronize(rdg_batch* b);
  * member starts once the member's previous stage is done; every wait is bounded (see
  * rdg_batch_set_wait_limit).  It needs every member FP32 with an element-wise D and the
  * SSP-RK3 integrator.  RDG_BATCH_AUTO (the default): persistent when every member fits, else
- * the graph.  The persistent form takes each member's set-up (forcing, dt, tiles) when the
- * membership last changed.
+ * the graph.  A member's forcing, integrator, stage form or operators may change between steps: the
+ * next step takes its set-up anew (captures again), RDG_ESTATE if it has no operators.
  * Errors: RDG_EINVAL (unknown mode, or RDG_BATCH_PERSISTENT with a member that does not fit). */
 enum { RDG_BATCH_AUTO = 0, RDG_BATCH_GRAPH = 1, RDG_BATCH_PERSISTENT = 2 };
 int rdg_batch_set_mode(rdg_batch* b, int mode);

@@ -57,6 +57,7 @@ void dfree(T*& p, cudaStream_t s) {
 
 void free_ops(rdg_ctx* ctx) {
   cudaStream_t s = ctx->stream;
+  ++ctx->setup_gen;
   dfree(ctx->d_W, s);
   dfree(ctx->d_k1, s);
   dfree(ctx->d_k2, s);
@@ -813,6 +814,7 @@ int rdg_set_forcing(rdg_ctx* ctx, int nsrc, const double* S, const int32_t* src_
   DeviceGuard g(ctx->device);
   CK(cudaStreamSynchronize(ctx->stream));
   const int64_t Np = np_of(ctx->N);
+  ++ctx->setup_gen;   // the old arrays go, whatever follows
   int rc = upload_converted(ctx, &ctx->d_S, S, (int64_t)nsrc * ctx->K * Np);
   if (rc != RDG_OK) return rc;
   rc = upload_converted(ctx, &ctx->d_G, G, (int64_t)nghost * ctx->B * Np);
@@ -1411,6 +1413,7 @@ int rdg_set_integrator(rdg_ctx* ctx, int integrator) {
   if (integrator != RDG_INTEGRATOR_SSP_RK3 && integrator != RDG_INTEGRATOR_LSRK54)
     return fail(ctx, RDG_EINVAL, "integrator must be RDG_INTEGRATOR_SSP_RK3 or RDG_INTEGRATOR_LSRK54");
   ctx->integrator = integrator;
+  ++ctx->setup_gen;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
   return RDG_OK;
@@ -1426,6 +1429,7 @@ int rdg_set_stage_form(rdg_ctx* ctx, int form) {
     if (rc != RDG_OK) return rc;
   }
   ctx->stage_form = form;
+  ++ctx->setup_gen;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
   return RDG_OK;
@@ -1440,6 +1444,7 @@ int rdg_gemm_hold_tile(rdg_ctx* ctx, int64_t tile) {
     if (rc != RDG_OK) return rc;
   }
   ctx->gemm_hold = tile + 1;
+  ++ctx->setup_gen;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
   return RDG_OK;
@@ -1455,6 +1460,7 @@ int rdg_set_l2_resident_bytes(rdg_ctx* ctx, int64_t bytes) {
   if (!ctx) return RDG_EINVAL;
   if (bytes < -1) return fail(ctx, RDG_EINVAL, "bytes must be >= -1");
   ctx->l2_keep_bytes = bytes;
+  ++ctx->setup_gen;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
   return RDG_OK;

@@ -23,6 +23,7 @@ struct rdg_batch {
     cudaEvent_t ev_in;    // member stream -> batch stream (work enqueued on the member before a step)
     cudaEvent_t ev_join;  // branch -> fork stream
     cudaStream_t branch;
+    uint64_t gen;         // the context's setup_gen that descriptors and captured launches were taken at
   };
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -318,7 +319,7 @@ int rdg_batch_add(rdg_batch* b, rdg_ctx* ctx, double t0, double dt) {
   for (auto& m : b->members)
     if (m.ctx == ctx) return bfail(b, RDG_EINVAL, "context is already in the batch");
   DevGuard g(b->device);
-  rdg_batch::Member m{ctx, dt, nullptr, nullptr, nullptr};
+  rdg_batch::Member m{ctx, dt, nullptr, nullptr, nullptr, ctx->setup_gen};
   bool ok = cudaEventCreateWithFlags(&m.ev_in, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&m.ev_join, cudaEventDisableTiming) == cudaSuccess &&
             cudaStreamCreateWithFlags(&m.branch, cudaStreamNonBlocking) == cudaSuccess;
@@ -378,6 +379,18 @@ int rdg_batch_step(rdg_batch* b, int64_t nsteps) {
   if (nsteps == 0 || b->members.empty()) return RDG_OK;
   DevGuard g(b->device);
   cudaError_t e;
+  // a member whose set-up changed since its descriptors and launches were taken has other buffers
+  bool changed = false;
+  for (auto& m : b->members) {
+    if (!m.ctx->ops_ok) return bfail(b, RDG_ESTATE, "a member context has no operators (rdg_operator_setup first)");
+    changed = changed || m.gen != m.ctx->setup_gen;
+  }
+  if (changed) {
+    if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) return bcuda(b, e, "cudaStreamSynchronize");
+    drop_graph(b);
+    b->dirty = true;
+    for (auto& m : b->members) m.gen = m.ctx->setup_gen;
+  }
   // order after the work already enqueued on every member's own stream
   for (auto& m : b->members) {
     if ((e = cudaEventRecord(m.ev_in, m.ctx->stream)) != cudaSuccess) return bcuda(b, e, "cudaEventRecord");

@@ -38,6 +38,9 @@ struct rdg_ctx {
   std::vector<int32_t> eref;     // [3][K]
   // operators
   bool ops_ok = false;
+  // counts every change of what a stage launches: buffers, forcing, integrator, kernel form.  A batch
+  // compares it before each step and takes its member's descriptors and captured launches anew.
+  uint64_t setup_gen = 0;
   int N = 0, prec = RDG_FP32, esz = 4, iface = RDG_IFACE_ALG2;
   double vx = 0, vy = 0;
   std::vector<double> Dk;           // element diffusion (x diffusion when Dy is set)
