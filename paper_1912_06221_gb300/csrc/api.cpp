@@ -540,7 +540,8 @@ static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz,
   if (W_tiled || W_dense || P_tiled) rc = setup_edges(ctx->N, in, W_tiled, esz, W_dense, P_tiled, s);
   if (rc == RDG_OK && faces) rc = setup_faces(in, K, ctx->face_tab, s);
   if (rc == RDG_OK && ctx->d_geo && !W_dense)
-    rc = setup_elements(K, d_xy, nodal ? nullptr : d_D, d_Dy, ctx->vx, ctx->vy, ctx->d_geo, esz, s);
+    rc = setup_elements(K, d_xy, nodal ? nullptr : d_D, d_Dy, ctx->vx, ctx->vy, ctx->d_geo, esz, false, s);
+  if (rc == RDG_OK && faces) rc = setup_elements(K, d_xy, d_D, d_Dy, ctx->vx, ctx->vy, ctx->face_tab.geo, 4, true, s);
   e = cudaStreamSynchronize(s);
   cleanup();
   if (rc != RDG_OK) return fail(ctx, rc, "setup kernel launch failed");
@@ -579,6 +580,7 @@ int ensure_edge_form(rdg_ctx* ctx) {
                         {(void**)&ctx->d_k2, E * 4, k2.data()},
                         {(void**)&ctx->d_f12, E * 4, f12.data()},
                         {(void**)&ctx->d_eref, 3 * K * 4, ctx->eref.data()},
+                        {&ctx->d_geo, 6 * K * esz, nullptr},
                         {&ctx->d_flux, E * Nfp * esz, nullptr},
                         {&ctx->d_vol, K * Np * esz, nullptr},
                         {&ctx->d_fb, K * 3 * Nfp * esz, nullptr}};
@@ -640,16 +642,17 @@ static int operator_setup_impl(rdg_ctx* ctx, int N, const double* D_elem, const 
   const int64_t K = ctx->K, Np = o->Np, esz = ctx->esz;
   const int64_t stb = K * Np * esz;
   ctx->face = precision != RDG_FP64 && !ctx->gemm && !Dn && K <= kMaxFaceElements;
-  CK(dalloc(&ctx->d_geo, 6 * K * esz, ctx->stream));
   CK(dalloc(&ctx->d_u, stb, ctx->stream));
   CK(dalloc(&ctx->d_u1, stb, ctx->stream));
   CK(dalloc(&ctx->d_u2, stb, ctx->stream));
   if (ctx->face) {
     FaceTables& t = ctx->face_tab;
-    CK(dalloc(&t.p4, 3 * K * (sizeof(float4) + sizeof(float2) + sizeof(float) + sizeof(unsigned)), ctx->stream));
+    CK(dalloc(&t.p4, 3 * K * (sizeof(float4) + sizeof(float2) + sizeof(float) + sizeof(unsigned)) + 6 * K * sizeof(float),
+              ctx->stream));
     t.p2 = reinterpret_cast<float2*>(t.p4 + 3 * K);
     t.p1 = reinterpret_cast<float*>(t.p2 + 3 * K);
     t.nbr = reinterpret_cast<unsigned*>(t.p1 + 3 * K);
+    t.geo = reinterpret_cast<float*>(t.nbr + 3 * K);
     if (ctx->B) CK(dalloc(&t.gpar, 2 * ctx->B * sizeof(float4), ctx->stream));
     CK(dalloc(&ctx->d_tau, kTauSteps * kTauStages * kTauRow * sizeof(float), ctx->stream));
     for (auto& r : ctx->d_rec) CK(dalloc(&r, face_rec_floats(N, K) * sizeof(float), ctx->stream));
@@ -965,7 +968,7 @@ FaceArgs face_args(const rdg_ctx* ctx, const float* us) {
   a.p2 = ctx->face_tab.p2;
   a.p1 = ctx->face_tab.p1;
   a.nbr = ctx->face_tab.nbr;
-  a.geo = (const float*)ctx->d_geo;
+  a.geo = ctx->face_tab.geo;
   a.S = (const float*)ctx->d_S;
   a.gpart = ctx->d_gpart;
   a.K = ctx->K;

@@ -61,7 +61,7 @@ struct rdg_ctx {
   int32_t* d_f12 = nullptr;         // per edge f1 | f2 << 2
   // face form (FP32, element-wise D): parameters, two alternating record buffers, ghost data's parts
   bool face = false;
-  rdg::FaceTables face_tab{};       // p4 heads one allocation that also holds p2, p1 and nbr
+  rdg::FaceTables face_tab{};       // p4 heads one allocation that also holds p2, p1, nbr and geo
   float* d_rec[2] = {nullptr, nullptr};
   float* d_gpart = nullptr;
   float* d_tau = nullptr;           // forcing factors of a replayed chunk's stages (launch_face_tau)

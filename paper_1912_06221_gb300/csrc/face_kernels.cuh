@@ -199,9 +199,10 @@ __device__ __forceinline__ void store_parts(const FaceArgs& a, const float (&v)[
                                             const bool (&diff)[3], unsigned k, bool active) {
   constexpr int NP = np_of(N), NG = N + 1;
   const size_t K3 = 3 * (size_t)a.K;
+  const float v0 = face::Ops<N>::reference(v);
   float d[NP];
 #pragma unroll
-  for (int j = 0; j < NP; ++j) d[j] = v[j] - v[0];
+  for (int j = 0; j < NP; ++j) d[j] = v[j] - v0;
   auto one = [&](auto face_c) {
     constexpr int F = decltype(face_c)::value;
     float g[NG];
@@ -226,7 +227,7 @@ __device__ __forceinline__ void store_parts(const FaceArgs& a, const float (&v)[
     one(std::integral_constant<int, 1>{});
     one(std::integral_constant<int, 2>{});
   }
-  if (active) (a.fout + NG * K3)[k] = v[0];
+  if (active) (a.fout + NG * K3)[k] = v0;
 }
 
 // Parts of the nk (>= 1) stage input elements from k0 on, by one warp; sh: 32 rows.
@@ -277,9 +278,11 @@ __global__ void __launch_bounds__(128) face_ghost_kernel(const float* G, const f
   if (i >= n) return;
   const int64_t b = i % B;
   float d[NP], g[NG];
-  const float v0 = G[i * NP];
 #pragma unroll
-  for (int j = 0; j < NP; ++j) d[j] = G[i * NP + j] - v0;
+  for (int j = 0; j < NP; ++j) d[j] = G[i * NP + j];
+  const float v0 = face::Ops<N>::reference(d);
+#pragma unroll
+  for (int j = 0; j < NP; ++j) d[j] -= v0;
   const float4 p = gpar[2 * b], q = gpar[2 * b + 1];
   face::face_part<float, N, 1, ALG1>(d, face::Par<float>{p.x, p.y, p.z, p.w, q.x, q.y, q.z}, true, g);
 #pragma unroll
@@ -335,17 +338,18 @@ __device__ __forceinline__ void stage_tile(const FaceArgs& a, int64_t k0, int nk
 #pragma unroll
     for (int f = 0; f < 3; ++f) records(f, own[f], nb[f]);
   }
+  const float u0 = ld_stage<LIVE>(a.fin + (size_t)NG * K3 + k);   // the reference value, with the own record
   rows_wait<1>();
-  float rhs[NP], u0;
+  float rhs[NP];
   {
     float ve[O::NE], vo[O::NO];
     {
       float d[NP];
       row_get<NP>(shs + row * NP, d);
-      u0 = d[0];
+      const float uc = d[O::CENTRE];
 #pragma unroll
-      for (int j = 0; j < NP; ++j) d[j] -= u0;
-      face::volume_parts<float, N>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      for (int j = 0; j < NP; ++j) d[j] -= uc;
+      face::volume_mirror<float, N, -1, O::CENTRE>(d, uc, geo, ve, vo);
     }
     auto flux = [&](int f, float (&ge)[O::GE], float (&go)[O::GO]) {
       float (&og)[NG] = own[RECS ? f : 0], (&ng)[NG + 1] = nb[RECS ? f : 0];
@@ -514,6 +518,7 @@ __device__ __forceinline__ void team_tile(const FaceArgs& a, int64_t k0, int nk,
   if (nv * 4 + tid < n) su[nv * 4 + tid] = ld_stage<LIVE>(a.us + k0 * NP + nv * 4 + tid);
   rows_commit();
   float own[NG], nb[NG + 1];
+  const float u0 = ld_stage<LIVE>(a.fin + (size_t)NG * K3 + k);
   if (f >= 0) {
     record_get<NG, LIVE>(a.fin, K3, (unsigned)f * K + k, own);
     neighbour_get<NG, LIVE>(a, nbr, k, nb);
@@ -523,9 +528,9 @@ __device__ __forceinline__ void team_tile(const FaceArgs& a, int64_t k0, int nk,
   {
     float d[NP], rhs[NP], ve[O::NE], vo[O::NO], ge[O::GE], go[O::GO];
     row_get<NP>(su + row * NP, d);
-    const float u0 = d[0];
+    const float uc = d[O::CENTRE];
 #pragma unroll
-    for (int j = 0; j < NP; ++j) d[j] -= u0;
+    for (int j = 0; j < NP; ++j) d[j] -= uc;
     auto flux = [&]() {
       if (nbr >= K3) ghost_get<NG>(a, nbr - K3, nb);
 #pragma unroll
@@ -549,22 +554,22 @@ __device__ __forceinline__ void team_tile(const FaceArgs& a, int64_t k0, int nk,
       O::lift_odd(go, vo);
     };
     if (warp == 0) {
-      face::volume_parts<float, N, 0>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      face::volume_mirror<float, N, 0, O::CENTRE>(d, uc, geo, ve, vo);
       O::nodes(ve, vo, rhs);
     } else if (warp == 1) {
-      face::volume_parts<float, N, 1>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      face::volume_mirror<float, N, 1, O::CENTRE>(d, uc, geo, ve, vo);
       O::nodes(ve, vo, rhs);
       flux();
       clear();
       lift();
       O::join0(ve, vo, rhs);
     } else if (warp == 2) {
-      face::volume_parts<float, N, 2>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      face::volume_mirror<float, N, 2, O::CENTRE>(d, uc, geo, ve, vo);
       flux();
       lift();                           // the second face's order is the element's own
       O::nodes(ve, vo, rhs);
     } else {
-      face::volume_parts<float, N, 3>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+      face::volume_mirror<float, N, 3, O::CENTRE>(d, uc, geo, ve, vo);
       O::nodes(ve, vo, rhs);
       flux();
       clear();
@@ -613,10 +618,11 @@ __device__ __forceinline__ void team_tile(const FaceArgs& a, int64_t k0, int nk,
   }
   if (!a.fout) return;
   __syncthreads();
+  float d[NP];
+  row_get<NP>(su + row * NP, d);
+  const float v0 = face::Ops<N>::reference(d);
   if (f >= 0) {
-    float d[NP], g[NG];
-    row_get<NP>(su + row * NP, d);
-    const float v0 = d[0];
+    float g[NG];
 #pragma unroll
     for (int j = 0; j < NP; ++j) d[j] -= v0;
     if (f == 0) face::face_part<float, N, 0, ALG1>(d, par, diff, g);
@@ -624,7 +630,7 @@ __device__ __forceinline__ void team_tile(const FaceArgs& a, int64_t k0, int nk,
     else face::face_part<float, N, 2, ALG1>(d, par, diff, g);
     if (active) record_put<NG>(a.fout, K3, (unsigned)f * K + k, g);
   } else if (active) {
-    (a.fout + (size_t)NG * K3)[k] = su[lane * NP];
+    (a.fout + (size_t)NG * K3)[k] = v0;
   }
 }
 
@@ -671,12 +677,12 @@ __global__ void __launch_bounds__(kFaceBlock) face_rhs_kernel(const __grid_const
   rows_wait<0>();
   float d[NP], rhs[NP];
   row_get<NP>(sh + row * NP, d);
-  const float u0 = d[0];
+  const float u0 = face::Ops<N>::reference(d);
 #pragma unroll
   for (int j = 0; j < NP; ++j) d[j] -= u0;
   {
     float ve[O::NE], vo[O::NO];
-    face::volume_parts<float, N>(d, u0, geo[0], geo[1], geo[2], geo[3], geo[4], ve, vo);
+    face::volume_mirror<float, N>(d, u0, geo, ve, vo);
     O::nodes(ve, vo, rhs);
   }
 #pragma unroll 1
@@ -697,7 +703,7 @@ __global__ void __launch_bounds__(kFaceBlock) face_rhs_kernel(const __grid_const
       const unsigned kn = q - (unsigned)fn * K;
       float v[NP], w[NP], n[NG];
       row_get<NP>(a.us + (int64_t)kn * NP, v);
-      const float n0 = v[0];
+      const float n0 = face::Ops<N>::reference(v);
 #pragma unroll
       for (int j = 0; j < NP; ++j) w[j] = v[j] -= n0;
       O::rotate(w);

@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(128, 1) edge_gemm_kernel(EdgeArgs<float> a, co
     const int64_t nvol = (a.K + kStageBlock - 1) / kStageBlock;
     float* sh = reinterpret_cast<float*>(smem);   // the A tiles are free now
     for (int64_t v = blockIdx.x; v < nvol; v += gridDim.x) {
-      dev::stage_volume_tile<float, N>(a, v, sh);
+      dev::stage_volume_tile<float, N, false, true>(a, v, sh);
       __syncthreads();
     }
   }
@@ -724,7 +724,7 @@ __device__ __forceinline__ void pipe_volume(const EdgeArgs<float>& a, uint8_t* s
       float u[NP], vol[NP];
 #pragma unroll
       for (int j = 0; j < NP; ++j) u[j] = sh[vt * NP + j];
-      dev::volume_row<float, N>(u, a.geo[k], a.geo[a.K + k], a.geo[2 * a.K + k], a.geo[3 * a.K + k],
+      dev::volume_row<float, N, false, true>(u, a.geo[k], a.geo[a.K + k], a.geo[2 * a.K + k], a.geo[3 * a.K + k],
                                 a.geo[4 * a.K + k], vol);
 #pragma unroll
       for (int j = 0; j < NP; ++j) sh[vt * NP + j] = vol[j];   // a thread rewrites only its own row

@@ -104,7 +104,9 @@ struct Gen {
     for (int i = 0; i < n; ++i)
       if (!begun[i]) std::printf("    %s[%d] = T(0);\n", y, i);
   }
-  void open(const char* sig) const { std::printf("  template <typename T>\n  static RDG_HD __forceinline__ void %s {\n", sig); }
+  void open(const char* sig, const char* more = "", const char* ret = "void") const {
+    std::printf("  template <typename T%s>\n  static RDG_HD __forceinline__ %s %s {\n", more, ret, sig);
+  }
   void close() const { std::printf("  }\n"); }
 
   int rep(bool even, int c) const { return even ? er[c] : eo[c]; }
@@ -166,13 +168,43 @@ struct Gen {
     for (int l = 0; l < Np; ++l)
       if (P[1][l] != l) { std::fprintf(stderr, "face 2's ordering is not the element's\n"); std::exit(1); }
 
-    int fixed_face = -1, zero = -1;   // the face's middle node among the even components; node 0
+    int fixed_face = -1;   // the face's middle node among the even components
+    int centre = -1;       // the node of the mirror axis nearest the centroid
+    for (int i = 0; i < Np; ++i)
+      if (mir[i] == i && (centre < 0 || std::fabs(o->r[i] + 1.0 / 3) < std::fabs(o->r[centre] + 1.0 / 3) - 1e-9)) centre = i;
     for (int c = 0; c < NE; ++c) {
       if (Nfp % 2 && er[c] == o->hyp[Nfp / 2]) fixed_face = c;
-      if (er[c] == 0) zero = c;
     }
     std::printf("template <>\nstruct Ops<%d> {\n", N);
-    std::printf("  static constexpr int NP = %d, NE = %d, NO = %d, GE = %d, GO = %d, MID = %d;\n", Np, NE, NO, GE, GO, fixed_face);
+    std::printf("  static constexpr int NP = %d, NE = %d, NO = %d, GE = %d, GO = %d, MID = %d, CENTRE = %d;\n", Np, NE, NO, GE, GO,
+                fixed_face, centre);
+
+    // the reference value: the mean over the vertices and the innermost ring of three nodes (order 1: the
+    // vertices), taken of differences so that a constant state's is exactly its value.  All Np nodes gave
+    // the same error for 3 to 5 times the operations.
+    {
+      std::vector<int> L;
+      double inner = 1e30;
+      for (int i = 0; i < Np; ++i) {
+        const double d = std::hypot(std::hypot(o->r[i] + 1.0 / 3, o->s[i] + 1.0 / 3), o->r[i] + o->s[i] + 2.0 / 3);
+        if (P[2][i] != i && d < inner - 1e-9) {
+          inner = d;
+          L = {i, P[2][i], P[2][P[2][i]]};
+        }
+      }
+      if (N > 1) L.insert(L.end(), {0, P[2][0], P[2][P[2][0]]});
+      const double w = 1.0 / (double)L.size();
+      open("reference(const T* v)", "", "T");
+      std::printf("    T s[2] = {T(0), T(0)};\n");
+      int c = 0;
+      for (int i : L)
+        if (i != 0) {
+          std::printf("    s[%d] = fma(v[%d] - v[0], %s, s[%d]);\n", c % 2, i, lit(w).c_str(), c % 2);
+          ++c;
+        }
+      std::printf("    return v[0] + (s[0] + s[1]);\n");
+      close();
+    }
 
     // mirror sums and differences of d in face f's order (face 1: the element's own)
     for (int f = 0; f < 3; ++f) {
@@ -355,6 +387,7 @@ struct Gen {
     // volume term in halves (ve, vo): p = D+ d, m = D- d with D+- = Dr +- Ds, F+- = F_r +- F_s,
     // vol = (W+ F+ + W- F-) / 2; component by component, so only d, vol and four scalars are live.
     // al = a_r + a_s, am = a_r - a_s, be = (g_rr + 2 g_rs + g_ss)/2, ga = (g_rr - g_ss)/2, de = (g_rr - 2 g_rs + g_ss)/2
+    // REF: the node that d is taken from (0 or the centre), whose own entry is zero and left out, or -1
     const Mat Dp = add(o->Dr, o->Ds, 1), Dm = add(o->Dr, o->Ds, -1);
     Mat Wp = add(o->Wr, o->Ws, 1), Wm = add(o->Wr, o->Ws, -1);
     for (auto& v : Wp) v *= 0.5;
@@ -378,7 +411,7 @@ struct Gen {
       char sig[160];
       std::snprintf(sig, sizeof sig, "volume%s(const T* e, const T* o, T u0, T al, T am, T be, T ga, T de, T* ve, T* vo)",
                     part < 0 ? "" : std::to_string(part).c_str());
-      open(sig);
+      open(sig, ", int REF");
       bool bege = false, bego = false;
       for (int odd = 0; odd < 2; ++odd) {
         const Mat Rp = comp(Dp, !odd, !odd, false), Rm = comp(Dm, !odd, odd, false);
@@ -393,8 +426,13 @@ struct Gen {
             bool begun = false;
             for (int c = 0; c < cols; ++c) {
               const double v = R[(size_t)q * cols + c];
-              if ((skip0 && c == zero) || std::fabs(v) <= 1e-13 * top) continue;   // d at node 0 is zero
-              if (begun) std::printf("      %s = fma(%s, %s[%d], %s);\n", y, lit(v).c_str(), x, c, y);
+              if (std::fabs(v) <= 1e-13 * top) continue;
+              const int ref = skip0 && (er[c] == 0 || er[c] == centre) ? er[c] : -1;
+              if (ref >= 0 && !begun)
+                std::printf("      if constexpr (REF == %d) %s = T(0);\n      else %s = %s * %s[%d];\n", ref, y, y, lit(v).c_str(), x, c);
+              else if (ref >= 0)
+                std::printf("      if constexpr (REF != %d) %s = fma(%s, %s[%d], %s);\n", ref, y, lit(v).c_str(), x, c, y);
+              else if (begun) std::printf("      %s = fma(%s, %s[%d], %s);\n", y, lit(v).c_str(), x, c, y);
               else std::printf("      %s = %s * %s[%d];\n", y, lit(v).c_str(), x, c);
               begun = true;
             }

@@ -114,7 +114,7 @@ struct FaceArgs {
   const float2* p2;
   const float* p1;
   const unsigned* nbr;
-  const float* geo;       // [6][K]
+  const float* geo;       // [6][K]: volume_mirror's five coefficients, 1/J
   const float* S;         // [nsrc][K][Np]
   const float* gpart;     // parts of the ghost data and its reference value [nghost][B][N + 2]
   int64_t K, B;
@@ -204,14 +204,15 @@ struct FaceTables {
   float2* p2;
   float* p1;
   unsigned* nbr;
+  float* geo;
   float4* gpar;
 };
 // Largest mesh of the face form: a record's byte offset in a plane fits 32 bits.
 constexpr int64_t kMaxFaceElements = (int64_t)1 << 27;
 int setup_faces(const EdgeSetupIn& in, int64_t K, const FaceTables& t, cudaStream_t s);
+// Element coefficients [6][K]: a_r, a_s, g_rr, g_rs, g_ss, 1/J, or (mirror) the face form's.
 int setup_elements(int64_t K, const double* xy, const double* D, const double* Dy, double vx, double vy, void* geo,
-                   int elem_bytes,
-                   cudaStream_t s);
+                   int elem_bytes, bool mirror, cudaStream_t s);
 // Reference constants for the setup kernel, flattened in the order setup.cu reads them.
 std::vector<double> pack_setup_refs(const RefOps& o);
 int advance_time(TimeState* ts, long long by, cudaStream_t s);

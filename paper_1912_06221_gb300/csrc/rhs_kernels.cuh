@@ -72,10 +72,13 @@ __device__ __forceinline__ double2 ld_keep(const double2* p, uint64_t pol) {
 // u - u_0 and vol are live: 2 Np values instead of 5 Np.
 //
 // NODAL: D given at the nodes (dn, the element's Np values; the coefficients g_rr, g_rs, g_ss
-// then hold the metric alone), F_r = a_r u - D_j (g_rr u_r + g_rs u_s) node by node.  Without it the
-// products run on the mirror-even and mirror-odd halves (face_ops.h), half the multiply-adds: FP64,
-// whose pipe issues one warp instruction in 64 cycles, is bound by their number.
-template <typename T, int N, bool NODAL = false>
+// then hold the metric alone), F_r = a_r u - D_j (g_rr u_r + g_rs u_s) node by node.
+// MIRROR: the products run on the mirror-even and mirror-odd halves (face_ops.h), half the
+// multiply-adds: FP64, whose pipe issues one warp instruction in 64 cycles, is bound by their number,
+// and the GEMM form's volume role has it for nothing (its products' split leaves larger errors).  FP32
+// with stored operators keeps the plain products: the halves' own rounding made its right-hand sides up
+// to 1.2 times (order 1) further from 64 bits, and the operator stream bounds it anyway.
+template <typename T, int N, bool NODAL = false, bool MIRROR = sizeof(T) == 8>
 __device__ __forceinline__ void volume_row(const T (&u)[np_of(N)], T ar, T as, T grr, T grs, T gss,
                                            T (&vol)[np_of(N)], const T* __restrict__ dn = nullptr) {
   constexpr int NP = np_of(N);
@@ -84,10 +87,14 @@ __device__ __forceinline__ void volume_row(const T (&u)[np_of(N)], T ar, T as, T
   du[0] = T(0);
 #pragma unroll
   for (int j = 1; j < NP; ++j) du[j] = u[j] - u[0];
-  if constexpr (!NODAL) {
+  if constexpr (!NODAL && MIRROR) {
     using O = face::Ops<N>;
     T ve[O::NE], vo[O::NO];
-    face::volume_parts<T, N>(du, u[0], ar, as, grr, grs, gss, ve, vo);
+    constexpr int REF = sizeof(T) == 4 ? O::CENTRE : 0;   // FP32: smaller differences; FP64: node 0's column is the fullest
+    const T uc = u[REF];
+#pragma unroll
+    for (int j = 0; j < NP; ++j) du[j] = j == REF ? T(0) : u[j] - uc;
+    face::volume_parts<T, N, REF>(du, uc, ar, as, grr, grs, gss, ve, vo);
     O::nodes(ve, vo, vol);
     return;
   }
@@ -113,9 +120,21 @@ __device__ __forceinline__ void volume_row(const T (&u)[np_of(N)], T ar, T as, T
   }
 }
 
-// rhs -= (1/J) LIFT_F q for face F's fluxes q in the element's face order, on mirror halves.
+// rhs -= (1/J) LIFT_F q for face F's fluxes q in the element's face order; FP64 on mirror halves (see
+// volume_row).
 template <typename T, int N, int F>
 __device__ __forceinline__ void lift_face(const T* q, T ij, T* rhs) {
+  if constexpr (sizeof(T) == 4) {
+    constexpr int NP = np_of(N), NFP = nfp_of(N), OLIFT = 4 * NP * NP;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      T acc = T(0);
+#pragma unroll
+      for (int c = 0; c < NFP; ++c) acc = fma((T)RDG_TAB[OLIFT + i * 3 * NFP + F * NFP + c], q[c], acc);
+      rhs[i] -= ij * acc;
+    }
+    return;
+  }
   using O = face::Ops<N>;
   T ge[O::GE], go[O::GO], ve[O::NE], vo[O::NO];
   const T h = T(-0.5) * ij;
@@ -218,7 +237,7 @@ __host__ __device__ constexpr int stage_block() {
   return sizeof(T) == 8 ? kStageBlock64 : kStageBlock;
 }
 
-template <typename T, int N, bool NODAL = false>
+template <typename T, int N, bool NODAL = false, bool MIRROR = sizeof(T) == 8>
 __device__ __noinline__ void stage_volume_tile(const EdgeArgs<T>& a, int64_t v, T* sh) {
   constexpr int NP = np_of(N);
   constexpr bool SMEM_TAB = N >= 6 && sizeof(T) == 4;   // (FP64: 25 KB of tables, and FP64-bound anyway)
@@ -248,7 +267,7 @@ __device__ __noinline__ void stage_volume_tile(const EdgeArgs<T>& a, int64_t v, 
       volume_row_smem<T, N, NODAL>(u, a.geo[k], a.geo[a.K + k], a.geo[2 * a.K + k], a.geo[3 * a.K + k],
                                    a.geo[4 * a.K + k], tab, vol, dn);
     else
-      volume_row<T, N, NODAL>(u, a.geo[k], a.geo[a.K + k], a.geo[2 * a.K + k], a.geo[3 * a.K + k], a.geo[4 * a.K + k],
+      volume_row<T, N, NODAL, MIRROR>(u, a.geo[k], a.geo[a.K + k], a.geo[2 * a.K + k], a.geo[3 * a.K + k], a.geo[4 * a.K + k],
                               vol, dn);
 #pragma unroll
     for (int j = 0; j < NP; ++j) sh[tid * NP + j] = vol[j];   // a thread rewrites only its own row

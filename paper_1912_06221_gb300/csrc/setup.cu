@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(128) face_setup_kernel(EdgeSetupIn in, int64_t
 }
 
 __global__ void elem_setup_kernel(int64_t K, const double* xy, const double* D, const double* Dy, double vx, double vy,
-                                  void* geo, int elem_bytes) {
+                                  void* geo, int elem_bytes, bool mirror) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= K) return;
   const double* v = xy + k * 6;
@@ -543,6 +543,14 @@ __global__ void elem_setup_kernel(int64_t K, const double* xy, const double* D, 
     g[2] = Dx * rx * rx + Dyk * ry * ry;
     g[3] = Dx * rx * sx + Dyk * ry * sy;
     g[4] = Dx * sx * sx + Dyk * sy * sy;
+  }
+  if (mirror) {   // combined here, rounded once
+    const double ar = g[0], as = g[1], gm = 0.5 * (g[2] + g[4]), grs = g[3], gd = 0.5 * (g[2] - g[4]);
+    g[0] = ar + as;
+    g[1] = ar - as;
+    g[2] = gm + grs;
+    g[3] = gd;
+    g[4] = gm - grs;
   }
   for (int c = 0; c < 6; ++c) {
     if (elem_bytes == 4) static_cast<float*>(geo)[c * K + k] = (float)g[c];
@@ -612,9 +620,9 @@ int setup_faces(const EdgeSetupIn& in, int64_t K, const FaceTables& t, cudaStrea
 }
 
 int setup_elements(int64_t K, const double* xy, const double* D, const double* Dy, double vx, double vy, void* geo,
-                   int elem_bytes, cudaStream_t s) {
+                   int elem_bytes, bool mirror, cudaStream_t s) {
   if (K == 0) return RDG_OK;
-  elem_setup_kernel<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(K, xy, D, Dy, vx, vy, geo, elem_bytes);
+  elem_setup_kernel<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(K, xy, D, Dy, vx, vy, geo, elem_bytes, mirror);
   return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
 }
 
