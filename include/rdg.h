@@ -295,8 +295,10 @@ int rdg_stage_buffer(rdg_ctx* ctx, int stage, void** dev_ptr);
 int rdg_rows_gather(rdg_ctx* ctx, const void* src_dev, const int32_t* idx_dev, int64_t n, void* dst_dev);
 int rdg_rows_scatter(rdg_ctx* ctx, const void* src_dev, const int32_t* idx_dev, int64_t n, void* dst_dev);
 
-/* nsteps steps of the selected integrator from t0 with step dt, replayed from a CUDA
- * graph of a fixed chunk of steps (captured on first use for a given dt); enqueued. */
+/* nsteps steps of the selected integrator from t0 with step dt, replayed from a CUDA graph of a
+ * fixed chunk of steps; enqueued.  The first solve of a dt launches its steps directly where there
+ * are fewer than 128 (a capture costs more than it saves there); the same solve gives the same bits
+ * on either route. */
 int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps);
 
 /* Bytes of the per-edge flux operators that every stage loads with an evict-last L2 policy,

@@ -979,16 +979,16 @@ FaceArgs face_args(const rdg_ctx* ctx, const float* us) {
   return a;
 }
 
-// The forcing factors at stage time ta: a row of the replayed chunk's table, or evaluated here.
+// The forcing factors at stage time ta: a row of the chunk's table, or evaluated here.
 void face_forcing(const rdg_ctx* ctx, const TimeArg& ta, int stage, FaceArgs& a) {
   const Forcing& f = ctx->frc;
   if (f.nsrc + f.nghost == 0) return;
-  if (ta.ts) {
-    // offsets within a replayed chunk count whole steps; the stage's own offset is in its row
+  if (ta.ts || ta.table) {
+    // offsets within a chunk count whole steps; the stage's own offset is in its row
     a.tau_row = ctx->d_tau + (ctx->tau_step % kTauSteps * kTauStages + stage) * kTauRow;
     return;
   }
-  const double t = ta.t0 + ta.off * ta.dt;
+  const double t = ta.t0 + (ta.n + ta.off) * ta.dt;
   for (int m = 0; m < f.nsrc; ++m) a.tau[m] = (float)host_tau(f.kind[m], f.omega[m], t);
   for (int m = 0; m < f.nghost; ++m) a.tau[RDG_MAX_FORCING_TERMS + m] = (float)host_tau(f.gkind[m], f.gomega[m], t);
 }
@@ -1191,8 +1191,8 @@ int enqueue_ssp_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, b
 }
 
 int enqueue_rk_step(rdg_ctx* ctx, const TimeArg& base, double dt, bool fresh, bool keep) {
-  if (base.ts && use_face(ctx) && ctx->frc.nsrc + ctx->frc.nghost > 0) {
-    // replayed steps read their forcing factors from a table, refilled every kTauSteps steps
+  if ((base.ts || base.table) && use_face(ctx) && ctx->frc.nsrc + ctx->frc.nghost > 0) {
+    // these steps read their forcing factors from a table, refilled every kTauSteps steps
     ctx->tau_step = (int)base.off;
     if (ctx->tau_step % kTauSteps == 0) {
       const bool ls5 = ctx->integrator == RDG_INTEGRATOR_LSRK54;
@@ -1359,7 +1359,7 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
   if (!(dt > 0) || !std::isfinite(t0) || nsteps < 0) return fail(ctx, RDG_EINVAL, "bad t0, dt or nsteps");
   if (nsteps == 0) return RDG_OK;
   DeviceGuard g(ctx->device);
-  const int chunk = ctx->prof ? (int)(nsteps + 1) : 16;   // profiling steps without the graph
+  const int chunk = ctx->prof ? (int)(nsteps + 1) : kTauSteps;   // profiling steps without the graph
   // A graph of a chunk costs about 0.2 ms to capture and instantiate.  The first solve of a dt launches
   // its steps directly where there are few (a launch costs less than a stage takes on all but tiny
   // meshes, and the device starts at once); it is captured when the dt comes again or the solve is long.
@@ -1404,7 +1404,9 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps) {
     for (; done + chunk <= nsteps; done += chunk) CK(cudaGraphLaunch(ctx->gexec, ctx->stream));
   }
   for (; done < nsteps; ++done) {
-    TimeArg ta{nullptr, t0 + done * dt, dt, 0.0};
+    // times and forcing factors as in a replayed chunk: the same solve has the same bits on either route
+    const double i = (double)(done % kTauSteps);
+    TimeArg ta{nullptr, t0, dt, i, (double)done - i, nsteps >= kTauSteps};
     int rc = enqueue_rk_step(ctx, ta, dt, done == 0, done + 1 < nsteps);
     if (rc != RDG_OK) return fail(ctx, rc, "kernel launch failed");
   }

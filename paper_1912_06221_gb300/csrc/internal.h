@@ -43,10 +43,13 @@ struct TimeState {
   long long n;
 };
 
-// Stage time: ts ? ts->t0 + (ts->n + off) dt : t0 + off dt
+// Stage time t0 + (n + off) dt, t0 and n from ts where it is given.  Steps that a solve may launch
+// directly or replay count n and off alike on both routes, so both sum the same numbers in the same order.
 struct TimeArg {
   const TimeState* ts;
   double t0, dt, off;
+  double n = 0;
+  bool table = false;   // the face form's forcing factors come from the table, as in a replayed chunk
 };
 
 template <typename T>

@@ -16,8 +16,8 @@ __device__ __forceinline__ double tau_of(int kind, double omega, double t) {
 }
 
 __device__ __forceinline__ double stage_time(const TimeArg& ta) {
-  if (ta.ts) return ta.ts->t0 + ((double)ta.ts->n + ta.off) * ta.dt;
-  return ta.t0 + ta.off * ta.dt;
+  const double t0 = ta.ts ? ta.ts->t0 : ta.t0, n = ta.ts ? (double)ta.ts->n : ta.n;
+  return t0 + (n + ta.off) * ta.dt;
 }
 
 // Programmatic dependent launch: a kernel launched with programmatic stream serialization may

@@ -572,7 +572,8 @@ __global__ void __launch_bounds__(kTauSteps * kTauStages * kTauRow) face_tau_ker
   const bool src = m < RDG_MAX_FORCING_TERMS;
   const int i = src ? m : m - RDG_MAX_FORCING_TERMS;
   if (i >= (src ? f.nsrc : f.nghost)) return;
-  const double t = base.ts->t0 + ((double)base.ts->n + (base.off + step + off.c[st])) * base.dt;
+  const double t0 = base.ts ? base.ts->t0 : base.t0, n = base.ts ? (double)base.ts->n : base.n;
+  const double t = t0 + (n + (base.off + step + off.c[st])) * base.dt;
   const int kind = src ? f.kind[i] : f.gkind[i];
   const double w = src ? f.omega[i] : f.gomega[i];
   rows[threadIdx.x] = (float)(kind == RDG_TAU_COS ? cos(w * t) : (kind == RDG_TAU_SIN ? sin(w * t) : 1.0));
