@@ -1091,6 +1091,7 @@ int enqueue_stage(rdg_ctx* ctx, const void* us, const void* un, void* out, int m
     const EdgeArgs<T> e1 = edge_subrange(ctx, ea, ctx->e_split, ctx->E);
     if constexpr (sizeof(T) == 4) rc = launch_edge_only32(ctx->N, e1, st);
     else rc = launch_edge_only64(ctx->N, e1, st);
+    la.early = true;
     if (rc == RDG_OK) {
       if constexpr (sizeof(T) == 4) rc = launch_elem_lite32(ctx->N, mode, la, st);
       else rc = launch_elem_lite64(ctx->N, mode, la, st);

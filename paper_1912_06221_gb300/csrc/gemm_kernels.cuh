@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(128, 1) edge_gemm_kernel(EdgeArgs<float> a, co
     const int64_t nvol = (a.K + kStageBlock - 1) / kStageBlock;
     float* sh = reinterpret_cast<float*>(smem);   // the A tiles are free now
     for (int64_t v = blockIdx.x; v < nvol; v += gridDim.x) {
-      dev::stage_volume_tile<float, N, false, true>(a, v, sh);
+      dev::stage_volume_tile<float, N, false, false, true>(a, v, sh);
       __syncthreads();
     }
   }

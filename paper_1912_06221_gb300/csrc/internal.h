@@ -14,7 +14,7 @@ namespace rdg {
 constexpr int kTile = 32;            // edges per W tile (one warp, one edge per lane)
 constexpr int kElemBlock = 128;      // elements per element-kernel block
 constexpr int kStageBlock = 128;     // threads per block of the FP32 stage (edge/volume) kernel
-// ... and of the FP64 one: the multiprocessor's one FP64 pipe is what the blocks share, and their work
+// ... and of the FP64 one, but for small meshes (wide64 in rhs_kernels.cuh): the multiprocessor's one FP64 pipe is what the blocks share, and their work
 // per thread differs (order 4: an element's volume term 490 FP64 instructions, an edge 146), so
 // single-warp blocks even out the SMs (order 4, 32768 triangles: 75 us per stage, 88 with 128 threads).
 constexpr int kStageBlock64 = 32;
@@ -100,6 +100,9 @@ struct ElemArgs {
   // rka != 0), du' = rka du + dt L(us) is written to out2 and us + rkb du' to out
   T* out2;
   T rka, rkb;
+  // FP64: after a few edges only (part 1 of a split stage), so launched programmatically: the blocks that
+  // wait take no one's place
+  bool early = false;
 };
 
 constexpr unsigned kFaceJump = 0x80000000u;

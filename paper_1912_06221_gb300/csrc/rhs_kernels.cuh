@@ -232,21 +232,22 @@ __device__ __forceinline__ void stage_in(T* sh, const T* g, int n) {
 // Volume role of the stage kernel: element tile v (one thread per element, rows staged
 // through shared memory), vol = M^{-1} S^T . F written to a.vol.  Kept out of line so its
 // register demand does not set the edge role's.
-template <typename T>
+template <typename T, int N, bool WIDE>
 __host__ __device__ constexpr int stage_block() {
-  return sizeof(T) == 8 ? kStageBlock64 : kStageBlock;
+  return sizeof(T) == 8 && N > 1 && !WIDE ? kStageBlock64 : kStageBlock;
 }
 
-template <typename T, int N, bool NODAL = false, bool MIRROR = sizeof(T) == 8>
+template <typename T, int N, bool WIDE = false, bool NODAL = false, bool MIRROR = sizeof(T) == 8>
 __device__ __noinline__ void stage_volume_tile(const EdgeArgs<T>& a, int64_t v, T* sh) {
   constexpr int NP = np_of(N);
   constexpr bool SMEM_TAB = N >= 6 && sizeof(T) == 4;   // (FP64: 25 KB of tables, and FP64-bound anyway)
   __shared__ __align__(16) T tab[SMEM_TAB ? VolTab<T, N>::SIZE : 4];
   const int tid = threadIdx.x;
-  const int64_t k0 = v * stage_block<T>();
-  const int nk = (int)min((int64_t)stage_block<T>(), (a.Kvol > 0 ? a.Kvol : a.K) - k0);
+  constexpr int BLK = stage_block<T, N, WIDE>();
+  const int64_t k0 = v * BLK;
+  const int nk = (int)min((int64_t)BLK, (a.Kvol > 0 ? a.Kvol : a.K) - k0);
   {
-    Staged<T, stage_block<T>(), NP> g;
+    Staged<T, BLK, NP> g;
     g.load(a.u + k0 * NP, nk * NP);
     if constexpr (SMEM_TAB) {
       constexpr int NV = VolTab<T, N>::SIZE * (int)sizeof(T) / 16;
@@ -418,39 +419,39 @@ __device__ __noinline__ void stage_edge(const EdgeArgs<T>& a, int64_t e) {
 // flight (order 6 measured 85, 83, 86 us per stage at 2, 3, 4 blocks per SM; orders 4 and 5
 // in that form were fastest at 5 and 4).
 constexpr int kEdgeOnlyBlocks[7] = {0, 5, 5, 5, 5, 4, 3};
-template <typename T, int N, int KIND = 1>
+template <typename T, int N, int KIND, bool WIDE>
 constexpr int stage_min_blocks() {
   if (KIND == 2 && sizeof(T) == 4) return kEdgeOnlyBlocks[N];
-  return sizeof(T) == 4 ? (N <= 4 ? 5 : 6) : (N <= 3 ? 4 : 3) * 128 / kStageBlock64;
+  return sizeof(T) == 4 ? (N <= 4 ? 5 : 6) : (N <= 3 ? 4 : 3) * 128 / stage_block<T, N, WIDE>();
 }
 
 // Operator stream kinds: 0 edge blocks only, fluxes to the per-edge buffer (allocation-free
 // entry point); 1 the fused form (edge and volume blocks interleaved, fluxes to the face
 // slots); 2 edge blocks only, fluxes to the face slots (the volume term from its own
 // kernel).
-template <typename T, int N, int KIND>
-__global__ void __launch_bounds__(stage_block<T>(), stage_min_blocks<T, N, KIND>()) edge_flux_kernel(EdgeArgs<T> a) {
-  constexpr int NP = np_of(N);
+template <typename T, int N, int KIND, bool WIDE = false>
+__global__ void __launch_bounds__((stage_block<T, N, WIDE>()), (stage_min_blocks<T, N, KIND, WIDE>())) edge_flux_kernel(EdgeArgs<T> a) {
+  constexpr int NP = np_of(N), BLK = stage_block<T, N, WIDE>();
   wait_for_predecessor();
   // the element kernel may start its independent loads on SMs that the last wave leaves idle
   if constexpr (KIND != 0) allow_dependents();
   int64_t eblk = blockIdx.x;
   if constexpr (KIND == 1) {
-    __shared__ __align__(16) T sh[stage_block<T>() * NP];
+    __shared__ __align__(16) T sh[BLK * NP];
     const int64_t nb = gridDim.x;
-    const int64_t nv = ((a.Kvol > 0 ? a.Kvol : a.K) + stage_block<T>() - 1) / stage_block<T>();
+    const int64_t nv = ((a.Kvol > 0 ? a.Kvol : a.K) + BLK - 1) / BLK;
     const int64_t b = blockIdx.x;
     // FP64: the long volume blocks first, so the short edge blocks even out the SMs
     const int64_t v0 = sizeof(T) == 8 ? b : (b * nv) / nb;
     const int64_t v1 = sizeof(T) == 8 ? min(b + 1, nv) : ((b + 1) * nv) / nb;
     if (v1 > v0) {
-      if (a.Dn) stage_volume_tile<T, N, true>(a, v0, sh);    // D given at the nodes
-      else stage_volume_tile<T, N, false>(a, v0, sh);
+      if (a.Dn) stage_volume_tile<T, N, WIDE, true>(a, v0, sh);    // D given at the nodes
+      else stage_volume_tile<T, N, WIDE, false>(a, v0, sh);
       return;
     }
     eblk = b - v1;    // edge blocks so far = blocks so far minus volume blocks so far
   }
-  const int64_t e = eblk * stage_block<T>() + threadIdx.x;
+  const int64_t e = eblk * BLK + threadIdx.x;
   if (e < a.E) stage_edge<T, N, KIND != 0>(a, e);
 }
 
@@ -546,18 +547,18 @@ __global__ void __launch_bounds__(kElemBlock, elem_min_blocks<T, N, VOLIN>()) el
 // then the stage.  The edge kernel has already scattered each edge's flux into both
 // elements' face slots (q), so every input is a contiguous [K][.] row: the block stages its
 // rows of the volume term, face fluxes, stage input and step start in one round trip.
-template <typename T, int N>
+template <typename T, int N, bool WIDE>
 __host__ __device__ constexpr int lite_block() {
-  if (sizeof(T) == 8) return kStageBlock64;   // as the stage kernel's
+  if (sizeof(T) == 8) return stage_block<T, N, WIDE>();
   return 128 * (3 * np_of(N) + 3 * nfp_of(N)) * (int)sizeof(T) <= 46 * 1024
              ? 128
              : (64 * (3 * np_of(N) + 3 * nfp_of(N)) * (int)sizeof(T) <= 46 * 1024 ? 64 : 32);
 }
 
-template <typename T, int N, int MODE>
-__global__ void __launch_bounds__(lite_block<T, N>(), elem_min_blocks<T, N, true>()) elem_lite_kernel(ElemArgs<T> a) {
+template <typename T, int N, int MODE, bool WIDE = false>
+__global__ void __launch_bounds__((lite_block<T, N, WIDE>()), (elem_min_blocks<T, N, true>())) elem_lite_kernel(ElemArgs<T> a) {
   constexpr int NP = np_of(N), NFP = nfp_of(N), NQ = 3 * NFP;
-  constexpr int BLK = lite_block<T, N>();
+  constexpr int BLK = lite_block<T, N, WIDE>();
   __shared__ __align__(16) T shv[BLK * NP];
   __shared__ __align__(16) T shq[BLK * NQ];
   __shared__ __align__(16) T shs[MODE >= 1 ? BLK * NP : 4];
@@ -758,31 +759,51 @@ __global__ void __launch_bounds__(kElemBlock, (N == 1 ? 8 : 1)) elem_fused_kerne
 }  // namespace dev
 
 // Host-side launch helpers instantiated by the including translation unit.
-// Programmatic launch in FP32.  In FP64 an ordinary one: dependent blocks that come early and wait take
-// the place of the running grid's (order 2, 8192 triangles: 24.1 us per stage against 12.1).
-template <typename T, typename... KArgs, typename... Args>
-inline int launch_stage_kernel(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t s, Args&&... args) {
-  if constexpr (sizeof(T) == 4) return launch_pdl(kernel, grid, block, s, std::forward<Args>(args)...);
+// Programmatic (early) or ordinary launch of a stage kernel.
+template <typename... KArgs, typename... Args>
+inline int launch_stage_kernel(bool early, void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t s, Args&&... args) {
+  if (early) return launch_pdl(kernel, grid, block, s, std::forward<Args>(args)...);
   kernel<<<grid, block, 0, s>>>(std::forward<Args>(args)...);
   return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
 }
 
-template <typename T, int N, bool VOL = false>
-inline int launch_edge_t(const EdgeArgs<T>& a, cudaStream_t s) {
-  const int64_t kv = a.Kvol > 0 ? a.Kvol : a.K;
-  if (a.E == 0 && (!VOL || kv == 0)) return RDG_OK;
-  const int64_t ge = (a.E + dev::stage_block<T>() - 1) / dev::stage_block<T>(), gv = (kv + dev::stage_block<T>() - 1) / dev::stage_block<T>();
-  if constexpr (VOL) return launch_stage_kernel<T>(dev::edge_flux_kernel<T, N, 1>, (unsigned)(ge + gv), dev::stage_block<T>(), s, a);
-  dev::edge_flux_kernel<T, N, 0><<<(unsigned)ge, dev::stage_block<T>(), 0, s>>>(a);
-  return cudaGetLastError() == cudaSuccess ? RDG_OK : RDG_ECUDA;
+// FP64 stages: whether the kernels run in blocks of 128 threads launched programmatically (wide) or in
+// single-warp blocks launched one after another.  With more blocks than SMs, dependent blocks that come
+// early and wait take the running grid's place (order 2, 8192 triangles: 24 against 12 us per stage), so
+// those launches are ordinary; but an ordinary launch costs 2 to 4 us of its own.  Wide is faster where
+// the wide blocks have an SM each, and at order 1, whose stages are mostly launches, everywhere (us per
+// low-storage stage, stepped directly, wide / single-warp: order 1 at 4608 triangles 7.5 / 12.3, 65522
+// 21.1 / 23.7; order 2 at 4608 11.7 / 16.4; order 3 20.8 / 22.6 but replayed 20.6 / 19.5).
+template <int N>
+inline bool wide64(int64_t K, int64_t E) {
+  return N == 1 || (N == 2 && (K + kStageBlock - 1) / kStageBlock + (E + kStageBlock - 1) / kStageBlock <= sm_count());
 }
 
-// Edge blocks only, fluxes to the face slots, programmatic launch.
+template <typename T, int N, int KIND, bool WIDE>
+inline int launch_edge_blocks(const EdgeArgs<T>& a, bool early, cudaStream_t s) {
+  constexpr int BLK = dev::stage_block<T, N, WIDE>();
+  const int64_t kv = KIND == 1 ? (a.Kvol > 0 ? a.Kvol : a.K) : 0;
+  const int64_t grid = (a.E + BLK - 1) / BLK + (kv + BLK - 1) / BLK;
+  if (grid == 0) return RDG_OK;
+  return launch_stage_kernel(early, dev::edge_flux_kernel<T, N, KIND, WIDE>, (unsigned)grid, BLK, s, a);
+}
+
+template <typename T, int N, bool VOL = false>
+inline int launch_edge_t(const EdgeArgs<T>& a, cudaStream_t s) {
+  if constexpr (!VOL) return launch_edge_blocks<T, N, 0, false>(a, false, s);
+  else if constexpr (sizeof(T) == 4) return launch_edge_blocks<T, N, 1, false>(a, true, s);
+  else {
+    const bool wide = wide64<N>(a.Kvol > 0 ? a.Kvol : a.K, a.E);
+    if constexpr (N == 2)
+      if (wide) return launch_edge_blocks<T, N, 1, true>(a, true, s);
+    return launch_edge_blocks<T, N, 1, false>(a, wide, s);
+  }
+}
+
+// Edge blocks only, fluxes to the face slots, programmatic launch (FP64: of a split mesh's last few edges).
 template <typename T, int N>
 inline int launch_edge_fb_t(const EdgeArgs<T>& a, cudaStream_t s) {
-  if (a.E == 0) return RDG_OK;
-  const int64_t ge = (a.E + dev::stage_block<T>() - 1) / dev::stage_block<T>();
-  return launch_stage_kernel<T>(dev::edge_flux_kernel<T, N, 2>, (unsigned)ge, dev::stage_block<T>(), s, a);
+  return launch_edge_blocks<T, N, 2, false>(a, true, s);
 }
 
 // One-kernel stage (elem_fused_kernel), programmatic launch.
@@ -799,20 +820,32 @@ inline int launch_fused_t(int mode, const EdgeArgs<T>& ea, const ElemArgs<T>& a,
   }
 }
 
+// Surface-only element update.  early: see ElemArgs.
+template <typename T, int N, bool WIDE>
+inline int launch_lite_t(int mode, const ElemArgs<T>& a, bool early, cudaStream_t s) {
+  constexpr int BLK = dev::lite_block<T, N, WIDE>();
+  const unsigned g = (unsigned)((a.K + BLK - 1) / BLK);
+  switch (mode) {
+    case 0: return launch_stage_kernel(early, dev::elem_lite_kernel<T, N, 0, WIDE>, g, BLK, s, a);
+    case 1: return launch_stage_kernel(early, dev::elem_lite_kernel<T, N, 1, WIDE>, g, BLK, s, a);
+    case 2: return launch_stage_kernel(early, dev::elem_lite_kernel<T, N, 2, WIDE>, g, BLK, s, a);
+    case 3: return launch_stage_kernel(early, dev::elem_lite_kernel<T, N, 3, WIDE>, g, BLK, s, a);
+    case 4: return launch_stage_kernel(early, dev::elem_lite_kernel<T, N, 4, WIDE>, g, BLK, s, a);
+    default: return RDG_EINVAL;
+  }
+}
+
 template <typename T, int N, bool VOLIN = false>
 inline int launch_elem_t(int mode, const ElemArgs<T>& a, cudaStream_t s) {
   if (a.K == 0) return RDG_OK;
   const unsigned grid = (unsigned)((a.K + kElemBlock - 1) / kElemBlock);
   if constexpr (VOLIN) {
-    constexpr int BLK = dev::lite_block<T, N>();
-    const unsigned g2 = (unsigned)((a.K + BLK - 1) / BLK);
-    switch (mode) {
-      case 0: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 0>, g2, BLK, s, a);
-      case 1: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 1>, g2, BLK, s, a);
-      case 2: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 2>, g2, BLK, s, a);
-      case 3: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 3>, g2, BLK, s, a);
-      case 4: return launch_stage_kernel<T>(dev::elem_lite_kernel<T, N, 4>, g2, BLK, s, a);
-      default: return RDG_EINVAL;
+    if constexpr (sizeof(T) == 4) return launch_lite_t<T, N, false>(mode, a, true, s);
+    else {
+      const bool wide = wide64<N>(a.K, a.E);
+      if constexpr (N == 2)
+        if (wide) return launch_lite_t<T, N, true>(mode, a, true, s);
+      return launch_lite_t<T, N, false>(mode, a, wide || a.early, s);
     }
   } else {
     switch (mode) {
