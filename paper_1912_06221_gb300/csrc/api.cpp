@@ -948,10 +948,16 @@ bool one_kernel_stage(const rdg_ctx* ctx) {
 // smaller meshes by default, up to where its doubled pipe time costs more than its short chains save
 // (us per stage, rows / two kernels: order 1 at 16200 triangles 7.0 / 8.9, order 2 at 8192 9.7 / 12.1,
 // order 3 at 8192 20 / 21, order 4 at 4608 17.7 / 31.3 and at 8192 37 / 35, order 5 at 4608 43 / 51,
-// order 6 at 4608 70 / 78; 512 triangles of order 2: 5.5 / 11.2).
+// order 6 at 4608 70 / 78; 512 triangles of order 2: 5.5 / 11.2).  On a split mesh it runs whole after the
+// halo exchange, where two kernels leave little more than the element update, so the line lies lower
+// there (us after the exchange, rows / two kernels: order 1 at 8281 triangles 5.6 / 6.1, order 2 at 4096
+// 7.4 / 8.5, order 3 at 4096 13.0 / 12.7, order 4 at 4096 17.9 / 19.1, order 5 at 1024 12.6 / 28 and at
+// 4096 43 / 28, order 6 at 1024 15 / 39 and at 4096 67 / 39).
 bool rows_stage(const rdg_ctx* ctx, int mode) {
   static const int64_t kRows[kMaxN + 1] = {0, 16384, 8192, 8192, 6144, 4608, 4608};
-  return ctx->esz == 8 && mode <= 3 && ctx->stage_form == RDG_STAGE_AUTO && ctx->K <= kRows[ctx->N];
+  static const int64_t kRowsSplit[kMaxN + 1] = {0, 9216, 5120, 4224, 4352, 2304, 2304};
+  return ctx->esz == 8 && mode <= 3 && ctx->stage_form == RDG_STAGE_AUTO &&
+         ctx->K <= (ctx->n_owned < ctx->K ? kRowsSplit : kRows)[ctx->N];
 }
 
 // Whether a stage of this context can run in two parts around a halo exchange (the stage
