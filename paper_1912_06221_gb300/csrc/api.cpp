@@ -1010,7 +1010,12 @@ int enqueue_face_parts(rdg_ctx* ctx, const float* us, int64_t k0, int64_t k1, in
 
 // Elements up to which a lone right-hand side is one launch (8192 elements, us per call with the host side,
 // one launch / two: order 2 3.8 / 6.1, order 4 4.7 / 6.0; 19602: order 3 5.0 / 6.2, order 4 6.4 / 6.0).
-constexpr int64_t kDirectRhsMax[kMaxN + 1] = {0, 20000, 20000, 20000, 10000, 5000, 5000};
+// Order 1: every size, and every stage on its own but the low-storage one (rdg_rk_stage, part 1 of a
+// split stage, whose part 0 then has nothing to do): its arithmetic is less than a launch.
+constexpr int64_t kDirectRhsMax[kMaxN + 1] = {0, INT64_MAX, 20000, 20000, 10000, 5000, 5000};
+bool lone_face_stage(const rdg_ctx* ctx, int mode) {
+  return mode == 0 ? ctx->K <= kDirectRhsMax[ctx->N] : ctx->N == 1 && mode <= 3;
+}
 
 // A stage in the face form.  fresh: the records of us are formed first (they are current only after
 // a stage that kept them, with nothing else having touched its result); keep: leave the records of
@@ -1020,6 +1025,8 @@ constexpr int64_t kDirectRhsMax[kMaxN + 1] = {0, 20000, 20000, 20000, 10000, 500
 int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* out, int mode, float dt, const TimeArg& ta,
                        float* out2, float rka, float rkb, int part, bool fresh, bool keep, int stage) {
   const int buf = mode == 0 ? ctx->rec_cur ^ 1 : ctx->rec_cur;
+  const bool lone = fresh && !keep && lone_face_stage(ctx, mode);   // needs no records
+  if (lone && part == 0) return RDG_OK;
   if (part == 0) return enqueue_face_parts(ctx, us, 0, ctx->n_owned, buf);
   cudaStream_t st = ls(ctx);
   const bool prof = ctx->prof && !ctx->capturing;
@@ -1029,10 +1036,9 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
     cudaEventRecord(ev[0], st);
   }
   int rc = RDG_OK;
-  // a lone right-hand side of a small mesh needs no records
-  const bool direct = mode == 0 && part < 0 && fresh && !keep && ctx->K <= kDirectRhsMax[ctx->N];
-  if (part == 1) rc = enqueue_face_parts(ctx, us, ctx->n_owned, ctx->K, buf);
-  else if (fresh && !direct) rc = enqueue_face_parts(ctx, us, 0, ctx->K, buf);
+  if (lone) rc = RDG_OK;
+  else if (part == 1) rc = enqueue_face_parts(ctx, us, ctx->n_owned, ctx->K, buf);
+  else if (fresh) rc = enqueue_face_parts(ctx, us, 0, ctx->K, buf);
   if (prof) {
     cudaEventRecord(ev[1], st);
     cudaEventRecord(ev[2], st);
@@ -1049,8 +1055,8 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
   a.rka = rka;
   a.rkb = rkb;
   if (rc == RDG_OK)
-    rc = direct ? launch_face_rhs(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st)
-                : launch_face_stage(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st);
+    rc = lone ? launch_face_lone(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st)
+              : launch_face_stage(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, st);
   if (rc == RDG_OK && keep) ctx->rec_cur ^= 1;
   if (prof) {
     cudaEventRecord(ev[3], st);
@@ -1266,7 +1272,7 @@ int enqueue_face_rhs(rdg_ctx* ctx, const float* u, float* rhs, const TimeArg& ta
   FaceArgs a = face_args(ctx, u);
   face_forcing(ctx, ta, 0, a);
   a.out = rhs;
-  return launch_face_rhs(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, ctx->stream);
+  return launch_face_lone(ctx->N, ctx->iface == RDG_IFACE_ALG1, a, ctx->stream);
 }
 
 }  // namespace rdg

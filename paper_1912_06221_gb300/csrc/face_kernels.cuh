@@ -290,10 +290,45 @@ __global__ void __launch_bounds__(128) face_ghost_kernel(const float* G, const f
   out[i * (NG + 1) + NG] = v0;
 }
 
+// The neighbour's part (as neighbour_get's record) evaluated from its row of the stage input: the same
+// arithmetic as its own parts, so the same bits.  p: the own face's parameters; the neighbour's are the
+// same but for its apex (c, h) and the signs of C, D and s.
+template <int N, bool ALG1>
+__device__ __forceinline__ void neighbour_part(const FaceArgs& a, unsigned r, unsigned k, const face::Par<float>& p, bool diff,
+                                               float (&ng)[N + 2]) {
+  using O = face::Ops<N>;
+  constexpr int NP = np_of(N), NG = N + 1;
+  const unsigned K = (unsigned)a.K, K3 = 3u * K;
+  if (r >= K3) {
+    if (r >= K3 + (unsigned)a.B) report(a.err, kErrBadIndex);
+    r = k;
+  }
+  const int fn = r >= 2u * K ? 2 : (r >= K ? 1 : 0);
+  const unsigned kn = r - (unsigned)fn * K;
+  const float2 apex = __ldg(reinterpret_cast<const float2*>(a.p4 + r));
+  float v[NP], w[NP], n[NG];
+  row_get<NP>(a.us + (int64_t)kn * NP, v);
+  const float n0 = O::reference(v);
+#pragma unroll
+  for (int j = 0; j < NP; ++j) w[j] = v[j] -= n0;
+  O::rotate(w);
+#pragma unroll
+  for (int j = 0; j < NP; ++j) v[j] = fn == 1 ? v[j] : w[j];
+  O::rotate(w);
+#pragma unroll
+  for (int j = 0; j < NP; ++j) v[j] = fn == 0 ? w[j] : v[j];
+  face::face_part<float, N, 1, ALG1>(v, face::Par<float>{apex.x, apex.y, p.A, p.B, -p.C, -p.D, -p.s}, diff, n);
+#pragma unroll
+  for (int c = 0; c < NG; ++c) ng[c] = n[c];
+  ng[NG] = n0;
+}
+
 // One stage of the nk (>= 1) elements from k0 on, by one warp; shs, shn: 32 rows each.  EARLY, ROLL: see
-// FaceBuild.
-template <int N, bool ALG1, int EARLY, bool ROLL, bool LIVE>
+// FaceBuild.  LONE: no records are read, the own and the neighbours' parts are evaluated here (EARLY 3;
+// not for the low-storage stage, which updates the rows that other warps still read).
+template <int N, bool ALG1, int EARLY, bool ROLL, bool LIVE, bool LONE = false>
 __device__ __forceinline__ void stage_tile(const FaceArgs& a, int64_t k0, int nk, float* shs, float* shn) {
+  static_assert(!LONE || (EARLY == 3 && !ROLL && !LIVE), "see above");
   using O = face::Ops<N>;
   constexpr bool RECS = EARLY & 1, PARS = EARLY & 2;
   constexpr int NP = np_of(N), NG = N + 1;
@@ -334,12 +369,25 @@ __device__ __forceinline__ void stage_tile(const FaceArgs& a, int64_t k0, int nk
     record_get<NG, LIVE>(a.fin, K3, (unsigned)f * (unsigned)a.K + k, og);
     neighbour_get<NG, LIVE>(a, nbr[f], k, ng);
   };
-  if constexpr (RECS) {
+  if constexpr (RECS && !LONE) {
 #pragma unroll
     for (int f = 0; f < 3; ++f) records(f, own[f], nb[f]);
   }
-  const float u0 = ld_stage<LIVE>(a.fin + (size_t)NG * K3 + k);   // the reference value, with the own record
+  float u0;
+  if constexpr (!LONE) u0 = ld_stage<LIVE>(a.fin + (size_t)NG * K3 + k);   // the reference value, with the own record
   rows_wait<1>();
+  if constexpr (LONE) {
+    float d[NP];
+    row_get<NP>(shs + row * NP, d);
+    u0 = O::reference(d);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) d[j] -= u0;
+    face::face_part<float, N, 0, ALG1>(d, par[0], diff[0], own[0]);
+    face::face_part<float, N, 1, ALG1>(d, par[1], diff[1], own[1]);
+    face::face_part<float, N, 2, ALG1>(d, par[2], diff[2], own[2]);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) neighbour_part<N, ALG1>(a, nbr[f], k, par[f], diff[f], nb[f]);
+  }
   float rhs[NP];
   {
     float ve[O::NE], vo[O::NO];
@@ -642,6 +690,17 @@ __global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const 
   team_tile<N, ALG1, false>(a, k0, (int)min((int64_t)32, a.K - k0), su, sp);
 }
 
+// Order 1, where two launches cost more than the arithmetic: a stage without records in one launch
+// (us, one launch / parts and stage: 512 triangles 2.9 / 4.6, 32768 3.6 / 5.8).
+template <int N, bool ALG1>
+__global__ void __launch_bounds__(kFaceBlock, 5) face_lone_kernel(const __grid_constant__ FaceArgs a) {
+  __shared__ __align__(16) float shs[kFaceWarps][32 * np_of(N)];
+  __shared__ __align__(16) float shn[kFaceWarps][32 * np_of(N)];
+  const int warp = threadIdx.x >> 5;
+  const int64_t k0 = ((int64_t)blockIdx.x * kFaceWarps + warp) * 32;
+  if (k0 < a.K) stage_tile<N, ALG1, 3, false, false, true>(a, k0, (int)min((int64_t)32, a.K - k0), shs[warp], shn[warp]);
+}
+
 // A lone right-hand side of a small mesh in one launch: a thread evaluates its neighbours' parts beside
 // its own (the same arithmetic on the neighbour's row, so the same bits) instead of reading records of a
 // first launch.  Twice the parts' work, which is free while there is at most a warp per scheduler; what
@@ -693,30 +752,7 @@ __global__ void __launch_bounds__(kFaceBlock) face_rhs_kernel(const __grid_const
     const face::Par<float> p = face_par(a, f, k, df);
     float g[NG], ng[NG + 1];
     face::face_part<float, N, 1, ALG1>(d, p, df, g);
-    {
-      unsigned q = r;
-      if (q >= K3) {
-        if (q >= K3 + (unsigned)a.B) report(a.err, kErrBadIndex);
-        q = k;
-      }
-      const int fn = q >= 2u * K ? 2 : (q >= K ? 1 : 0);
-      const unsigned kn = q - (unsigned)fn * K;
-      float v[NP], w[NP], n[NG];
-      row_get<NP>(a.us + (int64_t)kn * NP, v);
-      const float n0 = face::Ops<N>::reference(v);
-#pragma unroll
-      for (int j = 0; j < NP; ++j) w[j] = v[j] -= n0;
-      O::rotate(w);
-#pragma unroll
-      for (int j = 0; j < NP; ++j) v[j] = fn == 1 ? v[j] : w[j];
-      O::rotate(w);
-#pragma unroll
-      for (int j = 0; j < NP; ++j) v[j] = fn == 0 ? w[j] : v[j];
-      face::face_part<float, N, 1, ALG1>(v, face_par(a, fn, kn, df), df, n);
-#pragma unroll
-      for (int c = 0; c < NG; ++c) ng[c] = n[c];
-      ng[NG] = n0;
-    }
+    neighbour_part<N, ALG1>(a, r, k, p, df, ng);
     if (r >= K3) ghost_get<NG>(a, r - K3, ng);
     float ge[O::GE], go[O::GO], ve[O::NE], vo[O::NO];
 #pragma unroll

@@ -71,11 +71,16 @@ int RDG_CAT(launch_face_stage_, RDG_ORDER)(bool alg1, const FaceArgs& a, cudaStr
   return alg1 ? launch_stage<true>(a, s) : launch_stage<false>(a, s);
 }
 
-int RDG_CAT(launch_face_rhs_, RDG_ORDER)(bool alg1, const FaceArgs& a, cudaStream_t s) {
-  if (a.K == 0) return RDG_OK;
+template <bool ALG1>
+static int launch_lone(const FaceArgs& a, cudaStream_t s) {
   const unsigned grid = (unsigned)((a.K + dev::kFaceBlock - 1) / dev::kFaceBlock);
-  return alg1 ? launch_pdl(dev::face_rhs_kernel<RDG_ORDER, true>, grid, dev::kFaceBlock, s, a)
-              : launch_pdl(dev::face_rhs_kernel<RDG_ORDER, false>, grid, dev::kFaceBlock, s, a);
+  if constexpr (RDG_ORDER == 1) return launch_pdl(dev::face_lone_kernel<RDG_ORDER, ALG1>, grid, dev::kFaceBlock, s, a);
+  else return a.mode == 0 ? launch_pdl(dev::face_rhs_kernel<RDG_ORDER, ALG1>, grid, dev::kFaceBlock, s, a) : RDG_EINVAL;
+}
+
+int RDG_CAT(launch_face_lone_, RDG_ORDER)(bool alg1, const FaceArgs& a, cudaStream_t s) {
+  if (a.K == 0) return RDG_OK;
+  return alg1 ? launch_lone<true>(a, s) : launch_lone<false>(a, s);
 }
 
 int RDG_CAT(launch_face_ghost_, RDG_ORDER)(bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out,

@@ -167,8 +167,8 @@ int launch_edge_only64(int N, const EdgeArgs<double>& a, cudaStream_t s);
 // Face form: parts of elements [k_begin, k_end) from us into fout; a stage; the ghost data's parts.
 int launch_face_parts(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
 int launch_face_stage(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
-// One-launch right-hand side (mode 0, no records), for small meshes.
-int launch_face_rhs(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
+// One launch without records: a right-hand side (mode 0), at order 1 any stage but the low-storage one.
+int launch_face_lone(int N, bool alg1, const FaceArgs& a, cudaStream_t s);
 int launch_face_ghost(int N, bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out, cudaStream_t s);
 // Rows of tau values for kTauSteps steps from step n of the replay: row (step, stage) of kTauStages
 // stage offsets, 2 RDG_MAX_FORCING_TERMS floats each.

@@ -86,14 +86,14 @@ int launch_rows64(int N, int mode, const EdgeArgs<double>& ea, const ElemArgs<do
 #define RDG_FACE_DECL(n)                                                                               \
   int launch_face_parts_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                             \
   int launch_face_stage_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                             \
-  int launch_face_rhs_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                               \
+  int launch_face_lone_##n(bool alg1, const FaceArgs& a, cudaStream_t s);                              \
   int launch_face_ghost_##n(bool alg1, const float* G, const float4* gpar, int64_t B, int nghost, float* out, cudaStream_t s);
 RDG_FACE_DECL(1) RDG_FACE_DECL(2) RDG_FACE_DECL(3) RDG_FACE_DECL(4) RDG_FACE_DECL(5) RDG_FACE_DECL(6)
 
 #define CALL_FACE_PARTS(tag, n) launch_face_parts_##n(alg1, a, s)
 #define CALL_FACE_STAGE(tag, n) launch_face_stage_##n(alg1, a, s)
-#define CALL_FACE_RHS(tag, n) launch_face_rhs_##n(alg1, a, s)
-int launch_face_rhs(int N, bool alg1, const FaceArgs& a, cudaStream_t s) { RDG_SWITCH(f, CALL_FACE_RHS) }
+#define CALL_FACE_LONE(tag, n) launch_face_lone_##n(alg1, a, s)
+int launch_face_lone(int N, bool alg1, const FaceArgs& a, cudaStream_t s) { RDG_SWITCH(f, CALL_FACE_LONE) }
 #define CALL_FACE_GHOST(tag, n) launch_face_ghost_##n(alg1, G, gpar, B, nghost, out, s)
 int launch_face_parts(int N, bool alg1, const FaceArgs& a, cudaStream_t s) { RDG_SWITCH(f, CALL_FACE_PARTS) }
 int launch_face_stage(int N, bool alg1, const FaceArgs& a, cudaStream_t s) { RDG_SWITCH(f, CALL_FACE_STAGE) }

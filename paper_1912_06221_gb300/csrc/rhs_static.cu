@@ -9,7 +9,7 @@
 // and calls no allocating routine at all.  It runs the unfused pair of kernels (edge fluxes
 // into that array, then the element kernel with the volume term, LIFT and sources), not the
 // fused pair of rdg_rhs_eval; the two agree to rounding.  In the face form (FP32, element-wise D) it
-// is one launch that recomputes the neighbours' parts (face_rhs_kernel) and needs no scratch at all:
+// is one launch that recomputes the neighbours' parts (launch_face_lone) and needs no scratch at all:
 // the context's record buffers belong to its stages, one of which may be between its two parts or
 // running elsewhere when this is called or replayed.  The paper has no counterpart to it.
 #include <cuda_runtime.h>
