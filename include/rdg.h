@@ -232,8 +232,10 @@ int rdg_set_integrator(rdg_ctx* ctx, int integrator);
  *                        stage of any kind, a lone right-hand side in one or two), small FP64
  *                        meshes one kernel with a lane per (element, node), everything else
  *                        two kernels.
- * Setting a per-edge form on an FP32 context builds its operators there and then (device memory
- * as rdg_query_bytes says; RDG_ENOMEM if there is none).
+ * On an FP32 context set-up builds what the form set by then reads (device memory as
+ * rdg_query_bytes says).  Changing between a per-edge form and RDG_STAGE_AUTO later builds the
+ * other beside it, there and then (together up to twice rdg_query_bytes; RDG_ENOMEM if there is
+ * no room); a persistent batch does the same for a member with a per-edge form.
  * The one-kernel form serves rdg_rhs_eval and SSP-RK3 stages of contexts with stored
  * operators; the low-storage integrator (which updates its input in place), the GEMM form
  * and FP32 order 6 (tensor-core volume term) keep two kernels whatever is set.  Errors:
@@ -319,9 +321,11 @@ int rdg_kernel_stats(rdg_ctx* ctx, int64_t* launches, double* ms, int reset);
  * index self-check found a corrupt edge table (the device error word is then cleared). */
 int rdg_synchronize(rdg_ctx* ctx);
 
-/* Device bytes a context allocates for order N, nt triangles, n_edges edges (n_boundary of
- * them boundary edges), precision, nsrc/nghost forcing terms: the admission figure a
- * scheduler compares with its memory budget. */
+/* Upper bound of the device bytes a context allocates for order N, nt triangles, n_edges edges
+ * (n_boundary of them boundary edges), precision, nsrc/nghost forcing terms, whichever interface
+ * rule and stage form it is set up with (see rdg_set_stage_form for a form set later): the
+ * admission figure a scheduler compares with its memory budget.  In FP32 the stored per-edge
+ * operators set it; the default face form needs less at orders 2..6 (order 4: a third). */
 int rdg_query_bytes(int N, int64_t nt, int64_t n_edges, int64_t n_boundary, int precision, int nsrc, int nghost,
                     int64_t* bytes);
 

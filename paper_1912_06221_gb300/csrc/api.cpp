@@ -134,6 +134,9 @@ struct DeviceGuard {
   }
 };
 
+// Face parameters {c, h, A, B}, {C, D}, s and neighbour word of three faces, six coefficients.
+constexpr int64_t kFaceTableBytes = 3 * (sizeof(float4) + sizeof(float2) + sizeof(float) + sizeof(unsigned)) + 6 * sizeof(float);
+
 int64_t w_bytes(int N, int64_t E, int esz) {
   const int64_t tiles = (E + kTile - 1) / kTile;
   return tiles * w_vecs_per_edge(N, esz) * kTile * 16;
@@ -451,6 +454,13 @@ int rdg_query_bytes(int N, int64_t nt, int64_t n_edges, int64_t n_boundary, int 
   b += 6 * esz * nt;                           // element coefficients
   b += n_edges * Nfp * esz;                    // edge fluxes
   b += 4 * nt * Np * esz;                      // state, two stage buffers, volume terms
+  // the face form: parameters and coefficients, ghosts' parameters and parts, the forcing table, two
+  // record buffers, state and two stage buffers (a few bytes more than the per-edge form at order 1)
+  if (precision != RDG_FP64) {
+    const int64_t f = nt * (kFaceTableBytes + 3 * Np * esz) + 2 * face_rec_floats(N, nt) * 4 + n_boundary * 32 +
+                      (int64_t)nghost * n_boundary * (N + 2) * 4 + kTauSteps * kTauStages * kTauRow * 4;
+    b = std::max(b, f);
+  }
   b += (int64_t)nsrc * nt * Np * esz + (int64_t)nghost * n_boundary * Np * esz;
   *bytes = b;
   return RDG_OK;
@@ -458,10 +468,10 @@ int rdg_query_bytes(int N, int64_t nt, int64_t n_edges, int64_t n_boundary, int 
 
 }  // extern "C"
 
-// Per-edge operators in the forms asked for (each may be null), the face form's parameters (faces),
-// and, unless W_dense is wanted alone, the element coefficients.
+// Per-edge operators in the forms asked for (each may be null), the face form's parameters and
+// coefficients (faces), and, unless W_dense is wanted alone, the element coefficients.
 static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz, double* W_dense,
-                          float* P_tiled = nullptr, bool faces = false) {
+                          float* P_tiled = nullptr, const FaceTables* faces = nullptr) {
   const int64_t K = ctx->K, E = ctx->E;
   std::vector<int32_t> k1(E), f1(E), k2(E), f2(E);
   std::vector<double> sh(2 * E);
@@ -538,10 +548,10 @@ static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz,
   EdgeSetupIn in{d_xy, d_i, d_i + E, d_i + 2 * E, d_i + 3 * E, d_sh, d_D, d_Dy, d_Dn64, d_nref, d_refs, E, ctx->vx,
                  ctx->vy, ctx->iface, (int64_t)refs.size()};
   if (W_tiled || W_dense || P_tiled) rc = setup_edges(ctx->N, in, W_tiled, esz, W_dense, P_tiled, s);
-  if (rc == RDG_OK && faces) rc = setup_faces(in, K, ctx->face_tab, s);
-  if (rc == RDG_OK && ctx->d_geo && !W_dense)
+  if (rc == RDG_OK && faces) rc = setup_faces(in, K, *faces, s);
+  if (rc == RDG_OK && ctx->d_geo && !W_dense && !faces)
     rc = setup_elements(K, d_xy, nodal ? nullptr : d_D, d_Dy, ctx->vx, ctx->vy, ctx->d_geo, esz, false, s);
-  if (rc == RDG_OK && faces) rc = setup_elements(K, d_xy, d_D, d_Dy, ctx->vx, ctx->vy, ctx->face_tab.geo, 4, true, s);
+  if (rc == RDG_OK && faces) rc = setup_elements(K, d_xy, d_D, d_Dy, ctx->vx, ctx->vy, faces->geo, 4, true, s);
   e = cudaStreamSynchronize(s);
   cleanup();
   if (rc != RDG_OK) return fail(ctx, rc, "setup kernel launch failed");
@@ -552,6 +562,17 @@ static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz,
 extern "C" {
 
 }  // extern "C"
+
+// The parts of the ghost data's boundary fluxes in the face form, from d_G.
+static int ghost_parts(rdg_ctx* ctx) {
+  dfree(ctx->d_gpart, ctx->stream);
+  const int nghost = ctx->frc.nghost;
+  if (nghost == 0) return RDG_OK;
+  CK(dalloc(&ctx->d_gpart, (int64_t)nghost * ctx->B * (ctx->N + 2) * sizeof(float), ctx->stream));
+  int rc = launch_face_ghost(ctx->N, ctx->iface == RDG_IFACE_ALG1, (const float*)ctx->d_G, ctx->face_tab.gpar, ctx->B, nghost,
+                             ctx->d_gpart, ctx->stream);
+  return rc == RDG_OK ? RDG_OK : fail(ctx, rc, "kernel launch failed");
+}
 
 namespace rdg {
 
@@ -603,6 +624,38 @@ int ensure_edge_form(rdg_ctx* ctx) {
   return RDG_OK;
 }
 
+// Buffers and parameters of the face form, likewise (contexts with ctx->face).
+int ensure_face_form(rdg_ctx* ctx) {
+  if (ctx->face_tab.p4) return RDG_OK;
+  const int64_t K = ctx->K;
+  FaceTables t{};   // kept only when complete
+  float *rec[2] = {nullptr, nullptr}, *tau = nullptr;
+  cudaStream_t s = ctx->stream;
+  cudaError_t e = dalloc(&t.p4, K * kFaceTableBytes, s);
+  if (e == cudaSuccess && ctx->B) e = dalloc(&t.gpar, 2 * ctx->B * sizeof(float4), s);
+  if (e == cudaSuccess) e = dalloc(&tau, kTauSteps * kTauStages * kTauRow * sizeof(float), s);
+  for (auto& r : rec)
+    if (e == cudaSuccess) e = dalloc(&r, face_rec_floats(ctx->N, K) * sizeof(float), s);
+  t.p2 = reinterpret_cast<float2*>(t.p4 + 3 * K);
+  t.p1 = reinterpret_cast<float*>(t.p2 + 3 * K);
+  t.nbr = reinterpret_cast<unsigned*>(t.p1 + 3 * K);
+  t.geo = reinterpret_cast<float*>(t.nbr + 3 * K);
+  int rc = e == cudaSuccess ? build_edge_ops(ctx, get_refops(ctx->N, nullptr), nullptr, ctx->esz, nullptr, nullptr, &t)
+                            : cuda_fail(ctx, e, "face form buffers");
+  if (rc != RDG_OK) {
+    dfree(t.p4, s);
+    dfree(t.gpar, s);
+    dfree(tau, s);
+    for (auto& r : rec) dfree(r, s);
+    return rc;
+  }
+  ctx->face_tab = t;
+  ctx->d_tau = tau;
+  ctx->d_rec[0] = rec[0];
+  ctx->d_rec[1] = rec[1];
+  return ghost_parts(ctx);
+}
+
 }  // namespace rdg
 
 // Operator set-up; Dy (may be null) is the y diffusion of a diagonal tensor (D_elem then
@@ -645,18 +698,6 @@ static int operator_setup_impl(rdg_ctx* ctx, int N, const double* D_elem, const 
   CK(dalloc(&ctx->d_u, stb, ctx->stream));
   CK(dalloc(&ctx->d_u1, stb, ctx->stream));
   CK(dalloc(&ctx->d_u2, stb, ctx->stream));
-  if (ctx->face) {
-    FaceTables& t = ctx->face_tab;
-    CK(dalloc(&t.p4, 3 * K * (sizeof(float4) + sizeof(float2) + sizeof(float) + sizeof(unsigned)) + 6 * K * sizeof(float),
-              ctx->stream));
-    t.p2 = reinterpret_cast<float2*>(t.p4 + 3 * K);
-    t.p1 = reinterpret_cast<float*>(t.p2 + 3 * K);
-    t.nbr = reinterpret_cast<unsigned*>(t.p1 + 3 * K);
-    t.geo = reinterpret_cast<float*>(t.nbr + 3 * K);
-    if (ctx->B) CK(dalloc(&t.gpar, 2 * ctx->B * sizeof(float4), ctx->stream));
-    CK(dalloc(&ctx->d_tau, kTauSteps * kTauStages * kTauRow * sizeof(float), ctx->stream));
-    for (auto& r : ctx->d_rec) CK(dalloc(&r, face_rec_floats(N, K) * sizeof(float), ctx->stream));
-  }
   if (Dn) {   // the volume term's nodal D, in the context's precision
     CK(dalloc(&ctx->d_Dn, K * Np * esz, ctx->stream));
     if (esz == 8) {
@@ -669,9 +710,7 @@ static int operator_setup_impl(rdg_ctx* ctx, int N, const double* D_elem, const 
     }
   }
   CK(cudaMemsetAsync(ctx->d_u, 0, stb, ctx->stream));
-  int rc = RDG_OK;
-  if (ctx->face) rc = build_edge_ops(ctx, o, nullptr, (int)esz, nullptr, nullptr, true);
-  if (rc == RDG_OK && !use_face(ctx)) rc = ensure_edge_form(ctx);
+  int rc = use_face(ctx) ? ensure_face_form(ctx) : ensure_edge_form(ctx);
   if (rc != RDG_OK) {
     free_ops(ctx);
     return rc;
@@ -834,15 +873,7 @@ int rdg_set_forcing(rdg_ctx* ctx, int nsrc, const double* S, const int32_t* src_
     f.gomega[m] = ghost_omega[m];
   }
   ctx->frc = f;
-  if (ctx->face) {   // the ghost data's parts of the boundary fluxes
-    dfree(ctx->d_gpart, ctx->stream);
-    if (nghost) {
-      CK(dalloc(&ctx->d_gpart, (int64_t)nghost * ctx->B * (ctx->N + 2) * sizeof(float), ctx->stream));
-      rc = launch_face_ghost(ctx->N, ctx->iface == RDG_IFACE_ALG1, (const float*)ctx->d_G, ctx->face_tab.gpar, ctx->B, nghost,
-                             ctx->d_gpart, ctx->stream);
-      if (rc != RDG_OK) return fail(ctx, rc, "kernel launch failed");
-    }
-  }
+  if (ctx->face_tab.p4 && (rc = ghost_parts(ctx)) != RDG_OK) return rc;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
   return RDG_OK;
@@ -1441,9 +1472,9 @@ int rdg_set_stage_form(rdg_ctx* ctx, int form) {
   if (!ctx) return RDG_EINVAL;
   if (form != RDG_STAGE_AUTO && form != RDG_STAGE_TWO_KERNELS && form != RDG_STAGE_ONE_KERNEL)
     return fail(ctx, RDG_EINVAL, "form must be RDG_STAGE_AUTO, RDG_STAGE_TWO_KERNELS or RDG_STAGE_ONE_KERNEL");
-  if (ctx->ops_ok && ctx->face && form != RDG_STAGE_AUTO) {   // what the per-edge forms stream
+  if (ctx->ops_ok && ctx->face) {   // what the form reads
     DeviceGuard g(ctx->device);
-    int rc = ensure_edge_form(ctx);
+    int rc = form == RDG_STAGE_AUTO && ctx->gemm_hold == 0 ? ensure_face_form(ctx) : ensure_edge_form(ctx);
     if (rc != RDG_OK) return rc;
   }
   ctx->stage_form = form;
@@ -1456,9 +1487,9 @@ int rdg_set_stage_form(rdg_ctx* ctx, int form) {
 int rdg_gemm_hold_tile(rdg_ctx* ctx, int64_t tile) {
   if (!ctx) return RDG_EINVAL;
   if (tile < -1) return fail(ctx, RDG_EINVAL, "tile must be >= -1");
-  if (ctx->ops_ok && ctx->face && tile >= 0) {   // the held kernel belongs to the per-edge form
+  if (ctx->ops_ok && ctx->face) {   // the held kernel belongs to the per-edge form
     DeviceGuard g(ctx->device);
-    int rc = ensure_edge_form(ctx);
+    int rc = tile < 0 && ctx->stage_form == RDG_STAGE_AUTO ? ensure_face_form(ctx) : ensure_edge_form(ctx);
     if (rc != RDG_OK) return rc;
   }
   ctx->gemm_hold = tile + 1;

@@ -114,6 +114,10 @@ void free_persistent(rdg_batch* b) {
 int prepare_persistent(rdg_batch* b) {
   if (!b->dirty) return RDG_OK;
   free_persistent(b);
+  for (auto& m : b->members) {   // a member with a per-edge stage form has none of the face form's buffers
+    int rc = rdg::ensure_face_form(m.ctx);
+    if (rc != RDG_OK) return bfail(b, rc, std::string("member: ") + rdg_last_error(m.ctx));
+  }
   const int nm = (int)b->members.size();
   std::vector<rdg::BMember> hm(nm);
   // by order: each order's members are one list of items

@@ -59,7 +59,7 @@ struct rdg_ctx {
   void* d_vol = nullptr;            // volume terms of the current stage [K][Np]
   void* d_fb = nullptr;             // face fluxes of the current stage [K][3][Nfp]
   int32_t* d_f12 = nullptr;         // per edge f1 | f2 << 2
-  // face form (FP32, element-wise D): parameters, two alternating record buffers, ghost data's parts
+  // face form (face: FP32, element-wise D, so it may run; built when p4 is set): parameters, two alternating record buffers, ghost data's parts
   bool face = false;
   rdg::FaceTables face_tab{};       // p4 heads one allocation that also holds p2, p1, nbr and geo
   float* d_rec[2] = {nullptr, nullptr};
@@ -85,10 +85,11 @@ struct rdg_ctx {
 };
 
 namespace rdg {
-// Whether stages run in the face form, and building what the per-edge forms need beside it (an
-// explicitly set stage form).
+// Whether stages run in the face form, and building what a form needs where it is not there yet: set-up
+// builds the one in use, a stage form set later (and a batch, for its members) the other beside it.
 bool use_face(const rdg_ctx* ctx);
 int ensure_edge_form(rdg_ctx* ctx);
+int ensure_face_form(rdg_ctx* ctx);
 // One step of ctx's resident state with every launch on stream s (which may be capturing); used by
 // the batch, whose member steps run on per-member branch streams.  fresh: the face records of the
 // state are formed first; keep: the last stage leaves the records of its result.
