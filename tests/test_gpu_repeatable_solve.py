@@ -21,7 +21,7 @@ def _built():
 
 
 @pytest.mark.parametrize("prec,N,kind", [(rdg.FP32, 1, "elem"), (rdg.FP32, 3, "elem"), (rdg.FP32, 6, "elem"), (rdg.FP32, 2, "nodal"),
-                                         (rdg.FP64, 2, "elem"), (rdg.FP64, 4, "nodal"), (rdg.FP32_3XTF32, 3, "elem")])
+                                         (rdg.FP32, 4, "tensor"), (rdg.FP64, 3, "tensor"), (rdg.FP64, 2, "elem"), (rdg.FP64, 4, "nodal"), (rdg.FP32_3XTF32, 3, "elem")])
 @pytest.mark.parametrize("integ", [rdg.SSP_RK3, rdg.LSRK54])
 @pytest.mark.parametrize("steps", [16, 53])
 def test_forced_solve_repeats_bitwise(prec, N, kind, integ, steps):
@@ -29,7 +29,7 @@ def test_forced_solve_repeats_bitwise(prec, N, kind, integ, steps):
     xy, tri = unit_square_mesh(m, 0.1, 3)
     K = tri.shape[0]
     rng = np.random.default_rng(4)
-    D = rng.uniform(0.3, 1.0, (K, rdg.np_of(N)) if kind == "nodal" else K)
+    D = rng.uniform(0.3, 1.0, {"nodal": (K, rdg.np_of(N)), "tensor": (K, 2), "elem": K}[kind])
     s = rdg.Solver(xy, tri, N, D, v=(0.3, 0.2), bc=rdg.BC_DIRICHLET, precision=prec)
     s.set_integrator(integ)
     dt = 0.05 / m ** 2 / (N + 1) ** 4
