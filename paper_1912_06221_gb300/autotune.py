@@ -1,12 +1,11 @@
 """Measured per-order choices for batched and served FP32 solves.
 
-For each order N the library has two FP32-accurate edge-flux forms: the stored per-edge
-operators (RDG_FP32, an HBM-bound GEMV) and the GEMM form on the tensor cores
-(RDG_FP32_3XTF32, N <= 5).  Which is faster depends on the order and the problem size, so
-the tuner times both on the caller's own problem (a few replayed stages after a warm-up) and
+For each order N the library has two FP32-accurate edge-flux forms: the face form (RDG_FP32,
+no per-edge operators) and the GEMM form on the tensor cores (RDG_FP32_3XTF32, N <= 5).  The
+tuner times both on the caller's own problem (a few replayed stages after a warm-up) and
 caches the winner per (device, N, size class).  The graph chunk of a batch (steps per
 replayed graph) is tuned the same way on the batch itself, and so is the persistent batch
-launch's tile mapping per order (edges per thread of an edge work item) and the batch form
+launch's tiles per work item, per order, and the batch form
 (persistent launch or branch graph).  All timing is CUDA events on the solver's or batch's
 stream; nothing here computes the method.
 """
@@ -29,7 +28,8 @@ def size_class(n_triangles: int) -> int:
 
 def _time_steps(torch, solver, u0, dt, steps, reps=3):
     solver.set_state(u0)
-    solver.solve_to_time(0.0, dt, steps)        # warm-up (and graph capture)
+    for _ in range(2):                          # warm-up: the first solve of a dt is direct, the second captures
+        solver.solve_to_time(0.0, dt, steps)
     torch.cuda.synchronize()
     ts = []
     for _ in range(reps):
@@ -107,11 +107,11 @@ def _time_batch(torch, batch, members, u0s, steps):
 
 
 def choose_tiles(batch, members: List, u0s: List, steps: int) -> dict:
-    """Per-order tile mapping of the persistent batch launch: for every order present, one
-    or two edges per thread of an edge tile and one, two or four tiles per work item, chosen
-    one order at a time (the others kept at their best so far) by timing the batch itself.  Then the batch form (the persistent
-    launch or the branch graph) by timing both.  The batch is left with the best choices;
-    returns them and every time."""
+    """Per-order tile mapping of the persistent batch launch: for every order present, one,
+    two, four or eight tiles per work item (the product of rdg_batch_set_tiles' two numbers),
+    chosen one order at a time (the others kept at their best so far) by timing the batch
+    itself.  Then the batch form (the persistent launch or the branch graph) by timing both.
+    The batch is left with the best choices; returns them and every time."""
     import torch
     orders = sorted({s.N for s in members})
     times = {}
@@ -120,16 +120,12 @@ def choose_tiles(batch, members: List, u0s: List, steps: int) -> dict:
         return {"mode": "graph", "edges_per_thread_tiles_per_item": {}, "ms": {}}
     for N in orders:
         tN = {}
-        for e in (1, 2):                       # edges per thread, one tile per item
-            batch.set_tiles(N, e, 1)
-            tN[(e, 1)] = _time_batch(torch, batch, members, u0s, steps)
-        e = min((1, 2), key=lambda x: tN[(x, 1)])
-        for tpi in (2, 4):                     # then tiles per item
+        for e, tpi in ((1, 1), (1, 2), (1, 4), (2, 4)):
             batch.set_tiles(N, e, tpi)
             tN[(e, tpi)] = _time_batch(torch, batch, members, u0s, steps)
         best[N] = min(tN, key=tN.get)
         batch.set_tiles(N, *best[N])
-        times["N%d" % N] = {"%d edges/thread, %d tiles/item" % k: v for k, v in tN.items()}
+        times["N%d" % N] = {"%d x %d tiles/item" % k: v for k, v in tN.items()}
     # the last order's best time was taken with every order at its best
     t_pers = min(times["N%d" % orders[-1]].values())
     batch.set_mode(rdg.BATCH_GRAPH)
