@@ -119,13 +119,17 @@ int rdg_mesh_upload_partition(rdg_ctx* ctx, int64_t nv, const double* xy, int64_
 /* Operators for order N (1..6) with element-wise diffusion D_elem[nt] (> 0), constant
  * velocity (vx, vy), arithmetic precision RDG_FP64, RDG_FP32 or RDG_FP32_3XTF32, interface rule
  * RDG_IFACE_ALG2, RDG_IFACE_ALG1 or RDG_IFACE_HARMONIC for the edge diffusion (Algorithm 1
- * folds D1 and D2 into the operator in place of D~).  Builds, in FP64 on the GPU,
- * the element metric terms and for every edge the enclosed parallelogram (Sec. 4.2), the
- * projections V^{-1} V_p V_rf^{-1} of both sides (Eq. totalProjection), the least-squares
- * reconstruction (Sec. 4.5) and the edge-normal gradient, folded with D~ = RDG(D1, D2)
- * (Algorithm 2), the edge Jacobian J_f and the upwind convective trace into one
- * Nfp x 2Np flux operator per edge, stored in the chosen precision.  With RDG_FP32_3XTF32
- * (N <= 5) no operator is stored: each edge keeps a parameter record (the orthonormal basis
+ * uses D1 and D2 in place of D~).  Builds, in FP64 on the GPU, the element metric terms and for
+ * every edge the enclosed parallelogram (Sec. 4.2).  In FP64, and in FP32 under a per-edge stage
+ * form (rdg_set_stage_form), the projections V^{-1} V_p V_rf^{-1} of both sides (Eq.
+ * totalProjection), the least-squares reconstruction (Sec. 4.5) and the edge-normal gradient are
+ * folded with D~ = RDG(D1, D2) (Algorithm 2), the edge Jacobian J_f and the upwind convective
+ * trace into one Nfp x 2Np flux operator per edge, stored in the chosen precision.  In FP32 by
+ * default (the face form) no operator is stored: seven numbers per face (the apex of its
+ * sub-triangle, the weights of the reconstructed gradient's constant matrices, J_f v.n) and every
+ * stage evaluates the same chain in FP32; its right-hand sides are no further from 64-bit
+ * arithmetic than the stored operators' (a lone right-hand side of random data 1.2e-7 to 1.6e-7
+ * normwise at orders 2..6).  With RDG_FP32_3XTF32 (N <= 5) neither is stored: each edge keeps a parameter record (the orthonormal basis
  * at both sides' apex coordinates, kappa_R, kappa_S, -J_f D~_i, J_f v.n1), and the edge
  * kernel forms the flux as a tensor-core GEMM against reference matrices of the order (see
  * rdg_reference_operator which = 6).
@@ -138,8 +142,8 @@ int rdg_operator_setup(rdg_ctx* ctx, int N, const double* D_elem, double vx, dou
  * volume flux F = v u - (Dx u_x, Dy u_y), and on every edge the chosen interface rule applied
  * per component (Algorithm 2: n . (D~x u~_x, D~y u~_y) with D~x = RDG(Dx1, Dx2) and likewise
  * for y; Algorithm 1: n . RDG((Dx^1 u~^1_x, Dy^1 u~^1_y), (Dx^2 u~^2_x, Dy^2 u~^2_y)); harmonic:
- * the per-component harmonic means), folded into the per-edge operators as for scalar D.
- * Stored operators only: with RDG_FP32_3XTF32 the RDG_FP32 path runs.  Errors: as
+ * the per-component harmonic means), as for scalar D.  With RDG_FP32_3XTF32 the RDG_FP32 path
+ * runs.  Errors: as
  * rdg_operator_setup (RDG_EINVAL when Dy is NULL). */
 int rdg_operator_setup_aniso(rdg_ctx* ctx, int N, const double* Dx, const double* Dy, double vx, double vy,
                              int precision, int interface_rule);
@@ -207,10 +211,10 @@ int rdg_rhs_eval(rdg_ctx* ctx, const void* u_dev, void* rhs_dev, double t);
  * process, so the address is valid only while that device's primary context lives (not after
  * a cudaDeviceReset); make that first call before any stream capture.  Contexts using the
  * GEMM form of the edge flux (RDG_FP32_3XTF32 with N <= 5 and an interface rule other than
- * RDG_IFACE_ALG1) have no stored operators and get RDG_ESTATE.  All calls that use the array share it; it keeps the last call's contents (every
- * flux is rewritten before it is read, so nothing is cleared): calls whose GPU work
- * overlaps (different streams or devices' contexts sharing a device) race on it.  The paper
- * has no counterpart to this entry point. */
+ * RDG_IFACE_ALG1) have no stored operators and get RDG_ESTATE.  All calls that use the array
+ * share it; it keeps the last call's contents (every flux is rewritten before it is read, so
+ * nothing is cleared): calls whose GPU work overlaps (different streams or devices' contexts
+ * sharing a device) race on it.  The paper has no counterpart to this entry point. */
 int rdg_rhs_eval_static(rdg_ctx* ctx, const void* u_dev, void* rhs_dev, double t);
 
 /* Time integrator of rdg_rk_step, rdg_solve_to_time and batch steps:
@@ -221,8 +225,8 @@ int rdg_rhs_eval_static(rdg_ctx* ctx, const void* u_dev, void* rhs_dev, double t
 enum { RDG_INTEGRATOR_SSP_RK3 = 0, RDG_INTEGRATOR_LSRK54 = 1 };
 int rdg_set_integrator(rdg_ctx* ctx, int integrator);
 
-/* Kernel form of a right-hand-side stage (Algorithm aRDG, Sec. 4.5, and the SSP-RK3 update;
- * the arithmetic is the same in every form):
+/* Kernel form of a right-hand-side stage (Algorithm aRDG, Sec. 4.5, and the SSP-RK3 update; the
+ * same right-hand side in every form, to rounding):
  * RDG_STAGE_TWO_KERNELS  a stage kernel (edge fluxes into the two elements' face slots,
  *                        volume terms) and an element kernel (LIFT, sources, stage update);
  * RDG_STAGE_ONE_KERNEL   one element kernel that also computes its three edges' fluxes (each
@@ -250,9 +254,9 @@ int rdg_get_stage_form(const rdg_ctx* ctx, int* form);
  * the next stage on, tile `tile` of every launch of the context's tensor-core kernel is never
  * released (the GEMM form of the edge flux: edge tile of 128 edges, never handed to the MMAs
  * by its producer; FP32 order 6: element tile of 128 elements of the volume term, whose MMAs
- * are never issued), so the threads that wait for it give up after 1-2 s, the launch leaves
- * early (its results undefined) and the next rdg_synchronize returns RDG_ETIMEOUT; tile = -1
- * removes the hold.  Other contexts ignore it.  Errors: RDG_EINVAL for tile < -1. */
+ * are never issued; a held context runs the per-edge form), so the threads that wait for it give
+ * up after 1-2 s, the launch leaves early (its results undefined) and the next rdg_synchronize
+ * returns RDG_ETIMEOUT; tile = -1 removes the hold.  Other contexts ignore it.  Errors: RDG_EINVAL for tile < -1. */
 int rdg_gemm_hold_tile(rdg_ctx* ctx, int64_t tile);
 
 /* One step of the resident state from time t with step dt with the selected integrator;
@@ -260,23 +264,27 @@ int rdg_gemm_hold_tile(rdg_ctx* ctx, int64_t tile);
 int rdg_rk_step(rdg_ctx* ctx, double t, double dt);
 
 /* One stage of one step of the selected integrator from step start t with step dt
- * (SSP-RK3: stage 0, 1, 2 at t, t+dt, t+dt/2; the low-storage scheme: stages 0..4): the same
- * launches as the stage inside rdg_rk_step, enqueued.  Stages 0..last in order make one step.
+ * (SSP-RK3: stage 0, 1, 2 at t, t+dt, t+dt/2; the low-storage scheme: stages 0..4), enqueued.
+ * Stages 0..last in order make one step, with rdg_rk_step's bits.  In the face form (FP32) the
+ * stage input's face data are formed first, in a launch of their own (order 1: in the stage).
  * For a mesh split across ranks the caller refreshes the halo rows of rdg_stage_buffer(stage)
  * before each stage.  Errors: RDG_ESTATE, RDG_EINVAL (stage out of range, bad dt). */
 int rdg_rk_stage(rdg_ctx* ctx, int stage, double t, double dt);
 
 /* The same stage in two parts, so that a split mesh's halo exchange overlaps the work that
  * does not need it (the per-stage exchange of the partitioned Algorithm aRDG, Sec. 4.5: an
- * edge reads all 2 Np values of both neighbours).  Part 0 enqueues the edges with no halo
- * side (the first e_split edges of a partitioned upload; e_split is a multiple of 32) and the
- * owned elements' volume terms: it reads owned rows of the stage input only.  Part 1 enqueues
- * the remaining edges and the element update; the caller writes the halo rows of
- * rdg_stage_buffer(stage) between the two (rdg_rows_scatter).  Parts 0 then 1 give the same
- * owned rows as rdg_rk_stage (halo rows of the stage output are not defined).  Contexts that
- * cannot split a stage (not partitioned, the GEMM form, FP32 order 6, the one-kernel form)
- * run the whole stage in part 1 and nothing in part 0.  Errors: as rdg_rk_stage, RDG_EINVAL
- * for a part other than 0 or 1. */
+ * edge reads all 2 Np values of both neighbours).  Part 0 reads owned rows of the stage input
+ * only; the caller writes the halo rows of rdg_stage_buffer(stage) between the two
+ * (rdg_rows_scatter).  Stored operators: part 0 enqueues the edges with no halo side (the first
+ * e_split edges of a partitioned upload; e_split is a multiple of 32) and the owned elements'
+ * volume terms, part 1 the remaining edges and the element update.  Face form (FP32): part 0
+ * forms the owned elements' shares of their face fluxes, part 1 the halo elements', then runs
+ * the stage (order 4, 131044 owned triangles: 6 and 9.7 us, against 23 and 9.4 with stored
+ * operators).  Parts 0 then 1 give the same owned rows as rdg_rk_stage (halo rows of the stage
+ * output are not defined).  Where a stage is not split (not partitioned, the GEMM form, FP32
+ * order 6 with stored operators, the one-kernel forms: FP32 order 1 with SSP-RK3, FP64 with
+ * SSP-RK3 on a few thousand triangles) the whole stage runs in part 1 and nothing in part 0.
+ * Errors: as rdg_rk_stage, RDG_EINVAL for a part other than 0 or 1. */
 int rdg_rk_stage_part(rdg_ctx* ctx, int stage, int part, double t, double dt);
 
 /* Owned elements and e_split (edges [0, e_split) touch no halo element) of the uploaded
@@ -309,11 +317,13 @@ int rdg_solve_to_time(rdg_ctx* ctx, double t0, double dt, int64_t nsteps);
  * has none.  Affects speed only, never results. */
 int rdg_set_l2_resident_bytes(rdg_ctx* ctx, int64_t bytes);
 
-/* Per-kernel timing.  With enable != 0 every later edge-flux and element-update kernel launch
- * of ctx is bracketed by CUDA events on the context stream (rdg_solve_to_time then steps
- * without its graph).  rdg_kernel_stats waits for the stream and returns, for kernel class
- * 0 (edge flux) and 1 (element update), the number of launches and the summed device
- * milliseconds since the last reset; reset != 0 clears them afterwards. */
+/* Per-kernel timing.  With enable != 0 the two parts of every later stage of ctx are bracketed
+ * by CUDA events on the context stream (rdg_solve_to_time then steps without its graph).
+ * rdg_kernel_stats waits for the stream and returns, for class 0 (edge fluxes and volume terms;
+ * face form: the shares of the face fluxes, where they are formed apart) and 1 (element update;
+ * face form: the stage kernel), the number of brackets, empty ones included (one-kernel stages
+ * leave class 0 empty), and the summed device milliseconds since the last reset; reset != 0
+ * clears them afterwards. */
 int rdg_profile(rdg_ctx* ctx, int enable);
 int rdg_kernel_stats(rdg_ctx* ctx, int64_t* launches, double* ms, int reset);
 
@@ -413,7 +423,7 @@ int rdg_batch_set_chunk(rdg_batch* b, int chunk);
 /* Number of members into *n. */
 int rdg_batch_size(const rdg_batch* b, int* n);
 /* Enqueue nsteps SSP-RK3 steps of every member: floor(nsteps/chunk) replays of the graph
- * (captured on first use after the membership changed) and the remainder as direct
+ * (captured on first use after the membership or a member changed) and the remainder as direct
  * launches on the branch streams.  Each member continues from its own time. */
 int rdg_batch_step(rdg_batch* b, int64_t nsteps);
 /* Wait for the batch stream, then check every member as rdg_synchronize does.  Returns

@@ -559,10 +559,6 @@ static int build_edge_ops(rdg_ctx* ctx, const RefOps* o, void* W_tiled, int esz,
   return RDG_OK;
 }
 
-extern "C" {
-
-}  // extern "C"
-
 // The parts of the ghost data's boundary fluxes in the face form, from d_G.
 static int ghost_parts(rdg_ctx* ctx) {
   dfree(ctx->d_gpart, ctx->stream);
@@ -1097,9 +1093,9 @@ int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* ou
   return rc;
 }
 
-// part -1: the whole stage.  On a split mesh, part 0: the edges with no halo side and the owned
-// elements' volume terms (they read owned rows only); part 1: the remaining edges and the
-// element update.  A stage that cannot be split runs whole in part 1 (part 0 enqueues nothing).
+// part -1: the whole stage.  On a split mesh with stored operators, part 0: the edges with no halo
+// side and the owned elements' volume terms (they read owned rows only); part 1: the remaining edges
+// and the element update.  A stage that cannot be split runs whole in part 1 (part 0 enqueues nothing).
 template <typename T>
 int enqueue_stage(rdg_ctx* ctx, const void* us, const void* un, void* out, int mode, T dt, const TimeArg& ta,
                   void* out2 = nullptr, T rka = T(0), T rkb = T(0), int part = -1, bool fresh = true, bool keep = false, int stage = 0) {

@@ -34,7 +34,7 @@ constexpr int kFaceBlock = 32 * kFaceWarps;
 // the loop is faster there (order 6, 20402 elements: 7.9 against 8.9 us per stage; order 4 no gain).
 // More tiles than those warps (large): all tiles resident at once beats two uneven waves.  131072
 // elements, small / large: order 1 4.2 / 3.4 us, 2 5.5 / 4.5, 3 7.2 / 6.1, 4 10.8 / 9.2; 65522
-// elements: order 5 10.9 / 9.2, 6 14.7 / 13.5.
+// elements: order 5 10.9 / 9.2, 6 14.7 / 13.5 (all with node 0 as the reference value; its mean adds 0 to 2%).
 struct FaceBuild {
   int early, blocks;
   bool roll;
@@ -691,7 +691,8 @@ __global__ void __launch_bounds__(128, team_blocks<N>()) face_team_kernel(const 
 }
 
 // Order 1, where two launches cost more than the arithmetic: a stage without records in one launch
-// (us, one launch / parts and stage: 512 triangles 2.9 / 4.6, 32768 3.6 / 5.8).
+// (us per stage called on its own, one launch / parts and stage: up to 32768 triangles 2.8 / 4.6, 131072
+// 4.7 / 5.8; a right-hand side of 32768 3.8 / 5.9, of 524288 12.8 / 15.4).
 template <int N, bool ALG1>
 __global__ void __launch_bounds__(kFaceBlock, 5) face_lone_kernel(const __grid_constant__ FaceArgs a) {
   __shared__ __align__(16) float shs[kFaceWarps][32 * np_of(N)];

@@ -9,8 +9,9 @@ owning rank), uploads it with rdg_mesh_upload_partition, and before every stage 
 rows its neighbours hold as halo and receives its own halo rows (one grouped send/receive per
 neighbour per stage, NCCL over torch.distributed on GPUs, gloo on CPUs).  Each rank computes
 every local row; the owned rows are exact because the halo rows hold the owners' values.
-The exchange overlaps the part of the stage that reads owned rows only (the edges with no
-halo side, which the partitioned upload puts first, and the owned volume terms).
+The exchange overlaps the part of the stage that reads owned rows only (FP32: the owned
+elements' shares of their face fluxes; FP64: the edges with no halo side, which the
+partitioned upload puts first, and the owned volume terms).
 
 Host logic only: the partition (recursive coordinate bisection of element centroids), face
 adjacency (vertex ids, then midpoints modulo the period, as the library's mesh upload
@@ -203,9 +204,9 @@ class SplitSolver:
             self.unpack(dst, p, self.recv_bufs[p])
 
     def rk_step(self, t: float, dt: float, dist, group=None, stages: int = 3, overlap: bool = True):
-        """One step.  overlap: each stage's exchange runs while the edges with no halo side
-        and the owned volume terms are computed (rdg_rk_stage_part 0), the rest after it
-        (part 1); otherwise the halo rows are refreshed before each whole stage."""
+        """One step.  overlap: each stage's exchange runs while what reads owned rows only is
+        computed (rdg_rk_stage_part 0), the rest after it (part 1); otherwise the halo rows are
+        refreshed before each whole stage."""
         for st in range(stages):
             buf = self.s.stage_buffer(st)
             if overlap:
