@@ -12,7 +12,8 @@
 // A block takes items of one order, if it can that of its SM (a share of the SMs by the order's work),
 // until that list is used up, then of the others: an order's code is 5 to 70 KB.  With one list for all
 // orders the batch named below took 18.3 us per stage, with lists and as many blocks to each as it has
-// items 14.5 (and 11.7 once no ticket was taken before the item ahead of it was done).
+// items 14.5; no ticket is taken before the item ahead of it is done (a block would hold two items of a
+// phase while others had none: two members of orders 2 and 3, 8.7 against 5.4 us).
 //
 // One phase per stage: with per-edge operators a stage took two dependent parts (edge fluxes and volume
 // terms, then the element updates) and streamed 584 B per edge; 12 members of orders 2..6 and 200 to

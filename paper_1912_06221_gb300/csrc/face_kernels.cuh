@@ -34,7 +34,7 @@ constexpr int kFaceBlock = 32 * kFaceWarps;
 // the loop is faster there (order 6, 20402 elements: 7.9 against 8.9 us per stage; order 4 no gain).
 // More tiles than those warps (large): all tiles resident at once beats two uneven waves.  131072
 // elements, small / large: order 1 4.2 / 3.4 us, 2 5.5 / 4.5, 3 7.2 / 6.1, 4 10.8 / 9.2; 65522
-// elements: order 5 10.9 / 9.2, 6 14.7 / 13.5 (all with node 0 as the reference value; its mean adds 0 to 2%).
+// elements: order 5 10.9 / 9.2, 6 14.7 / 13.5 (all with node 0 as the reference value; its mean adds 0 to 2.5%).
 struct FaceBuild {
   int early, blocks;
   bool roll;

@@ -45,8 +45,8 @@ static int resident_blocks(K kernel, std::atomic<int>* cached) {
 }
 
 // Which kernel runs a stage, by the number of 32-element tiles:
-//  - at orders 4..6, up to one tile per SM: four warps to a tile (512 elements, order 4 / 5 / 6: 2.6 / 3.6
-//    / 4.4 us per stage against 3.1 / 4.7 / 6.8; at 8192 elements it no longer gains);
+//  - at orders 4..6, up to one tile per SM: four warps to a tile (512 elements, order 4 / 5 / 6: 2.8 / 3.6
+//    / 4.5 us per stage against 3.1 / 4.7 / 6.8; at 8192 elements it no longer gains);
 //  - the small build while its warps hold all tiles, the large one (more, leaner warps) beyond, as long
 //    as few waves of it remain (2 up to order 4, 1 above): with many waves the difference is gone and
 //    the small build's early loads win (order 3, 1M elements: 53 against 57 us per stage).
