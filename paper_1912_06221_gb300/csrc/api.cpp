@@ -1047,11 +1047,13 @@ bool lone_face_stage(const rdg_ctx* ctx, int mode) {
 // A stage in the face form.  fresh: the records of us are formed first (they are current only after
 // a stage that kept them, with nothing else having touched its result); keep: leave the records of
 // the result, in the other buffer.  On a split mesh, part 0: the owned elements' records (they read
-// owned rows only), part 1: the halo elements' records, then the stage.  Between the two the current
-// buffer holds the pending stage's records, so a lone right-hand side forms its own in the other one.
+// owned rows only), part 1: the halo elements' records, then the stage.  Between the two buffer 0 holds
+// the pending stage's records (fresh ones always go there), so a lone right-hand side, also one that a
+// caller captured earlier and replays, forms its own in buffer 1.
 int enqueue_face_stage(rdg_ctx* ctx, const float* us, const float* un, float* out, int mode, float dt, const TimeArg& ta,
                        float* out2, float rka, float rkb, int part, bool fresh, bool keep, int stage) {
-  const int buf = mode == 0 ? ctx->rec_cur ^ 1 : ctx->rec_cur;
+  if (mode != 0 && fresh) ctx->rec_cur = 0;
+  const int buf = mode == 0 ? 1 : ctx->rec_cur;
   const bool lone = fresh && !keep && lone_face_stage(ctx, mode);   // needs no records
   if (lone && part == 0) return RDG_OK;
   if (part == 0) return enqueue_face_parts(ctx, us, 0, ctx->n_owned, buf);

@@ -60,3 +60,43 @@ def test_lone_rhs_between_stage_parts(N, m, entry, integ):
     assert np.array_equal(plain, mixed)
     assert all(torch.equal(g, alone) for g in got)
     s.close()
+
+
+@pytest.mark.parametrize("N,m", [(3, 150), (5, 75)])
+@pytest.mark.parametrize("steps_before", [1, 2])
+def test_replayed_rhs_between_stage_parts(N, m, steps_before):
+    """The same with a right-hand side that was captured earlier, before a solve of an even or odd number
+    of stages."""
+    xy, tri = unit_square_mesh(m, 0.1, 3)
+    plan = build_plan(rcb_partition(xy, tri, 2), face_adjacency(xy, tri), 0, 2)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        sp = SplitSolver(xy, tri, N, np.full(len(tri), 0.4), plan, v=(0.5, -0.3), precision=rdg.FP32, stream=st)
+        s = sp.s
+        w = torch.tensor(random_nodal(s.K, s.Np, 9), dtype=torch.float32, device="cuda")
+        r = torch.empty_like(w)
+        s.rhs_eval(w, r, 0.0)
+        st.synchronize()
+        alone = r.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            s.rhs_eval(w, r, 0.0)
+    dt = 0.02 / m ** 2 / (N + 1) ** 4
+
+    def step(between):
+        sp.set_owned_state(random_nodal(len(tri), s.Np, 2))
+        s.solve_to_time(0.0, dt, steps_before)
+        for stage in range(3):
+            s.rk_stage_part(stage, 0, 0.0, dt)
+            if between:
+                with torch.cuda.stream(st):
+                    r.zero_()
+                    graph.replay()
+            s.rk_stage_part(stage, 1, 0.0, dt)
+        return sp.owned_state()
+
+    plain, mixed = step(False), [step(True) for _ in range(2)]
+    s.synchronize()
+    assert all(np.array_equal(plain, x) for x in mixed)
+    assert torch.equal(r, alone)
+    s.close()
