@@ -55,6 +55,17 @@ void dfree(T*& p, cudaStream_t s) {
   p = nullptr;
 }
 
+void free_face(rdg_ctx* ctx) {
+  cudaStream_t s = ctx->stream;
+  dfree(ctx->face_tab.p4, s);
+  dfree(ctx->face_tab.gpar, s);
+  ctx->face_tab = FaceTables{};
+  dfree(ctx->d_rec[0], s);
+  dfree(ctx->d_rec[1], s);
+  dfree(ctx->d_gpart, s);
+  dfree(ctx->d_tau, s);
+}
+
 void free_ops(rdg_ctx* ctx) {
   cudaStream_t s = ctx->stream;
   ++ctx->setup_gen;
@@ -73,13 +84,7 @@ void free_ops(rdg_ctx* ctx) {
   dfree(ctx->d_fb, s);
   dfree(ctx->d_f12, s);
   dfree(ctx->d_Dn, s);
-  dfree(ctx->face_tab.p4, s);
-  dfree(ctx->face_tab.gpar, s);
-  ctx->face_tab = FaceTables{};
-  dfree(ctx->d_rec[0], s);
-  dfree(ctx->d_rec[1], s);
-  dfree(ctx->d_gpart, s);
-  dfree(ctx->d_tau, s);
+  free_face(ctx);
   ctx->face = false;
   if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
   ctx->gexec = nullptr;
@@ -649,7 +654,9 @@ int ensure_face_form(rdg_ctx* ctx) {
   ctx->d_tau = tau;
   ctx->d_rec[0] = rec[0];
   ctx->d_rec[1] = rec[1];
-  return ghost_parts(ctx);
+  rc = ghost_parts(ctx);
+  if (rc != RDG_OK) free_face(ctx);
+  return rc;
 }
 
 }  // namespace rdg
@@ -852,7 +859,11 @@ int rdg_set_forcing(rdg_ctx* ctx, int nsrc, const double* S, const int32_t* src_
   DeviceGuard g(ctx->device);
   CK(cudaStreamSynchronize(ctx->stream));
   const int64_t Np = np_of(ctx->N);
-  ++ctx->setup_gen;   // the old arrays go, whatever follows
+  // the old arrays go, whatever follows: a failure leaves no forcing and no graph that reads them
+  ++ctx->setup_gen;
+  ctx->frc = Forcing();
+  if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
+  ctx->gexec = nullptr;
   int rc = upload_converted(ctx, &ctx->d_S, S, (int64_t)nsrc * ctx->K * Np);
   if (rc != RDG_OK) return rc;
   rc = upload_converted(ctx, &ctx->d_G, G, (int64_t)nghost * ctx->B * Np);
@@ -869,9 +880,10 @@ int rdg_set_forcing(rdg_ctx* ctx, int nsrc, const double* S, const int32_t* src_
     f.gomega[m] = ghost_omega[m];
   }
   ctx->frc = f;
-  if (ctx->face_tab.p4 && (rc = ghost_parts(ctx)) != RDG_OK) return rc;
-  if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
-  ctx->gexec = nullptr;
+  if (ctx->face_tab.p4 && (rc = ghost_parts(ctx)) != RDG_OK) {
+    ctx->frc = Forcing();
+    return rc;
+  }
   return RDG_OK;
 }
 
